@@ -277,8 +277,8 @@ uint64_t lsm_capacity(const lsm_t* h);
  * lsm_sort_pairs - the library's batch sort as a stand-alone call: stable
  * radix sort of n (key, value) pairs on the full 32-bit key (§IV-A sorts each
  * batch with a radix sort over the whole key variable): for n <= 2^20 a
- * bucket sort on the top byte followed by a sort of each bucket on the low
- * 24 bits, above that four 8-bit least-significant-digit passes.
+ * bucket sort (256 parts of the key range that the input spans, then the
+ * elements of each), above that four 8-bit least-significant-digit passes.
  * d_keys_in/d_vals_in are read, d_keys_out/d_vals_out receive the sorted
  * pairs (they must not overlap the inputs).  Uses the handle's scratch, so
  * n <= b.  Asynchronous.  Used by tests of the sort in isolation.
@@ -294,7 +294,7 @@ lsm_status lsm_sort_pairs(lsm_t* h, const uint32_t* d_keys_in, const uint32_t* d
  * raw cudaMalloc, or a latency-bound loop that cannot take the device-wide
  * synchronisation and unbounded time of a cudaMalloc/cudaFree).  No handle
  * is needed and nothing is allocated: every byte of scratch comes from one
- * fixed array with static storage inside the library (about 17 MB), which
+ * fixed array with static storage inside the library (about 9 MB), which
  * each GPU that loads the library keeps until the process exits.
  *   n        at most LSM_SORT_NOALLOC_MAX_PAIRS; larger n is refused with
  *            LSM_ERR_CAPACITY before any work is queued.  n = 0 is a no-op.

@@ -277,7 +277,7 @@ cudaError_t sort_positions(lsm_t* h, const uint32_t* keys, uint64_t n, uint64_t 
     if ((e = cudaMemset(h->d_qctl, 0, sizeof(uint32_t) * 2 * kSortCtlWords)) != cudaSuccess) return e;
     h->qsws.flip = 0;
   }
-  if (!h->qsws.tilecnt && (e = dalloc(&h->qsws.tilecnt, kMsdWsWords)) != cudaSuccess) return e;
+  if (!h->qsws.tilecnt && (e = dalloc(&h->qsws.tilecnt, kMsdRunWords)) != cudaSuccess) return e;
   h->qsws.ctl = h->d_qctl;
   h->qsws.sticky = h->d_misc + kMiscSticky;
   uint32_t* base = reinterpret_cast<uint32_t*>(h->d_q);
@@ -506,7 +506,7 @@ lsm_status lsm_create(lsm_t** out, uint32_t b, uint64_t max_elements, int device
   if (e == cudaSuccess) e = dalloc(&h->sws.ctl, 2 * kSortCtlWords);
   if (e == cudaSuccess) e = cudaMemset(h->sws.ctl, 0, sizeof(uint32_t) * 2 * kSortCtlWords);
   if (e == cudaSuccess) e = dalloc(&h->sws.lookback, uint64_t(kSortPasses) * sort_tiles * 256);
-  if (e == cudaSuccess && b <= kMsdMaxN) e = dalloc(&h->sws.tilecnt, msd_ws_words(b));
+  if (e == cudaSuccess && b <= kMsdMaxN) e = dalloc(&h->sws.tilecnt, kMsdRunWords);
   if (e == cudaSuccess) e = dalloc(&h->d_part, h->part_words);
   for (uint32_t i = 0; i < L + kBatchBufs; ++i) {
     h->fshift[i] = fence_shift_for(i < L ? (uint64_t(b) << i) : uint64_t(b));
@@ -787,7 +787,7 @@ lsm_status lsm_bulk_build(lsm_t* h, const uint32_t* d_keys, const uint32_t* d_va
   cudaError_t e = dalloc(&buf, 4 * npad + fence_words(fs));
   if (e == cudaSuccess) e = dalloc(&ctl, 2 * kSortCtlWords);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 0, 4ull * 2 * kSortCtlWords, st);
-  if (e == cudaSuccess) e = dalloc(&tilecnt, msd_ws_words(n < kMsdMaxN ? n : kMsdMaxN));
+  if (e == cudaSuccess) e = dalloc(&tilecnt, kMsdRunWords);
   if (e == cudaSuccess) e = dalloc(&lookback, uint64_t(kSortPasses) * tiles * 256);
   if (e == cudaSuccess) e = cudaMemsetAsync(lookback, 0, 8ull * kSortPasses * tiles * 256, st);
   if (e == cudaSuccess) {

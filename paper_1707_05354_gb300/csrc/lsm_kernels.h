@@ -124,21 +124,21 @@ struct SortWorkspace {
   uint32_t max_tiles;
   uint32_t epoch;       // bumped per sort; 0 never used
   uint32_t* sticky;     // persistent device error word (wait timeouts)
-  uint32_t* tilecnt;    // msd_ws_words(n) words for every sort of n <= kMsdMaxN it serves, or null
+  uint32_t* tilecnt;    // kMsdRunWords words for sorts of n <= kMsdMaxN, or null
 };
 // The bucket sort (n <= kMsdMaxN): the run table (per bucket and tile, the
-// start and length of the bucket's run in the tile), then the spill area of
-// buckets too large for shared memory (n keys, then n values).
+// start and length of the bucket's run in the tile).
 constexpr uint32_t kMsdMaxN = 1u << 20;
 constexpr uint32_t kMsdTile = 4096;
 constexpr uint32_t kMsdMaxTiles = kMsdMaxN / kMsdTile;
 constexpr uint32_t kMsdRunWords = 2 * kMsdMaxTiles * 256;
-// Workspace words for sorts of at most max_n <= kMsdMaxN elements (the spill
-// area holds a sort's n keys, then its n values).
-constexpr uint64_t msd_ws_words(uint64_t max_n) { return kMsdRunWords + 2 * max_n; }
-constexpr uint64_t kMsdWsWords = msd_ws_words(kMsdMaxN);
 constexpr int kSortCtlWords = kSortPasses * 256 + kSortPasses + 4;
 constexpr int kSortCtlStatus = kSortPasses * 256 + kSortPasses;
+// The bucket sort keeps its key map (two words) after the status word, and
+// its buckets' lower bounds in the first pass's histogram, which it does not
+// use.
+constexpr int kSortCtlMap = kSortCtlStatus + 1;
+constexpr int kSortCtlBounds = 0;
 
 // Enqueues the whole sort.  If `status` is given (a device-visible word,
 // typically mapped pinned host memory), the first kernel stores kErrBadKey

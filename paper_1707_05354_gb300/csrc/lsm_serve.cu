@@ -189,7 +189,7 @@ uint64_t slot_bytes(const lsm_server_config& c, uint32_t max_levels, uint32_t ma
   const uint64_t b = rup(c.b, 32) + 32, G = rup(c.group_keys, 32) + 32;
   return b * 9 + G * (4 + 4 + 1) + G * 12 + G * (4 + 4 + 4 + 8ull * max_levels) + (G + 1) * 8 +
          (G / 2048 + 2) * 8 + uint64_t(c.range_cap) * 8 + uint64_t(max_req) * (8 + 8 + 1) + 8 * 4 * G +
-         4ull * msd_ws_words(G < kMsdMaxN ? G : kMsdMaxN) + 64;
+         4ull * kMsdRunWords + 64;
 }
 
 // Device bytes of a dictionary with L levels of batch size b, as lsm_create
@@ -269,7 +269,7 @@ cudaError_t alloc_slot(Slot& s, const lsm_server_config& c, uint32_t max_levels,
   for (int i = 0; i < 6 && e == cudaSuccess; ++i) e = cudaEventCreate(&s.ev_ph[i]);
   if (e == cudaSuccess) e = dalloc(&s.sort_ctl, 2 * kSortCtlWords);
   if (e == cudaSuccess) e = cudaMemset(s.sort_ctl, 0, 4ull * 2 * kSortCtlWords);
-  if (e == cudaSuccess) e = dalloc(&s.sort_tilecnt, msd_ws_words(G < kMsdMaxN ? G : kMsdMaxN));
+  if (e == cudaSuccess) e = dalloc(&s.sort_tilecnt, kMsdRunWords);
   for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
     e = dalloc(&s.sa[i], G);
     if (e == cudaSuccess) e = dalloc(&s.sb[i], G);

@@ -254,24 +254,26 @@ __global__ void __launch_bounds__(kThreads, LSM_SORT_MINB) sort_pass(Loader ld, 
 }
 
 // ---------------------------------------------------------------------------
-// Bucket sort for n <= kMsdMaxN (the batch sizes of the plain form): the top
-// byte of the key variable first, then the low 24 bits inside each bucket.
-// Two kernels, so that a batch sort is one dependent launch after another:
+// Bucket sort for n <= kMsdMaxN (the batch sizes of the plain form): 256 key
+// ranges ("buckets") first, then the elements of each.  Two kernels, so that
+// a batch sort is one dependent launch after another:
 //   msd_tile     per 4096-element tile of the (encoded, reversed) input: the
-//                tile stably sorted by its top byte in shared memory and
-//                written back to the scratch at the tile's own place (one
-//                coalesced write), so bucket d's elements of tile t form the
-//                run runs[d][t] = (start, count) there; the grand total of
-//                each bucket (global atomics) and the key check.
+//                tile stably sorted by bucket in shared memory and written
+//                back to the scratch at the tile's own place (one coalesced
+//                write), so bucket d's elements of tile t form the run
+//                runs[d][t] = (start, count) there; the grand total of each
+//                bucket (global atomics) and the key check.
 //   bucket_sort  per bucket, one CTA: the bucket's runs, in tile order (the
 //                stable order), gathered into shared memory -- the start of
 //                the bucket in the output is the sum of the totals before
-//                it, so no tile waits for another -- then sorted on bits
-//                0..23 and written out with the prefix index entries of its
-//                256 bins.  A bucket above kBucketCap elements (heavy
-//                duplicate keys) is gathered into the spill area and sorted
-//                by the same CTA in chunks through global memory, still
-//                stably.
+//                it, so no tile waits for another -- then sorted and written
+//                out with the prefix index entries of the bins that start in
+//                its range.  A bucket above kBucketCap elements (many copies
+//                of a few keys, or keys in clusters) is taken by the same
+//                CTA in parts that fit.
+// The buckets split the range of the keys that the batch holds (KeyMap), not
+// the 32 bits of the key variable: ids below 2^25 would otherwise fall in
+// four buckets and be sorted by four CTAs.
 // ---------------------------------------------------------------------------
 constexpr int kBucketThreads = 512;
 constexpr int kBucketWarps = kBucketThreads / 32;
@@ -288,27 +290,60 @@ constexpr int kScatterIPT = int(kMsdTile) / kScatterThreads;  // 8
 static_assert(kScatterIPT * kScatterThreads == int(kMsdTile), "tile");
 static_assert(kMsdMaxTiles <= uint32_t(kBucketThreads), "one thread per tile run in the bucket kernel");
 
-// Start of bucket d in the output: the sum of the totals of the buckets
-// before it (every thread of the block gets it).
+// The buckets of one sort: bucket(kv) = floor((kv - lo) * mul / 2^32), kept
+// within [0, 255]; monotone, so bucket d holds the key variables of
+// [lower(d), lower(d + 1)).  lo and mul come from the smallest and largest of
+// 512 elements taken at even distances (every CTA of the tile kernel reads
+// the same ones), the range widened by 1/128 at both ends: for evenly spread
+// keys the widened range misses elements with a probability of about e^-5 at
+// either end, and those then fall in the first or last bucket.
+// With the top byte as the bucket, batches of 2^18 ids below 2^25 took 553 us
+// in bucket_sort and 2^20 keys below 2^30 154 us; now 21.7 and 21.3 us.
+struct KeyMap {
+  uint32_t lo, mul;
+  __device__ __forceinline__ uint32_t bucket(uint32_t kv) const {
+    return min(__umulhi(max(kv, lo) - lo, mul), uint32_t(kRadix - 1));
+  }
+  // smallest key variable of bucket d in 1 .. 255 (2^32 - 1 for a bucket the
+  // 32 bits do not reach: key variables are below it)
+  __device__ __forceinline__ uint32_t lower(uint32_t d) const {
+    return uint32_t(min(lo + ((uint64_t(d) << 32) + mul - 1) / mul, uint64_t(0xFFFFFFFFu)));
+  }
+};
+
+// Key map of the batch (every thread of a CTA of NT threads gets it).
 template <int NT>
-__device__ __forceinline__ uint32_t bucket_start(const uint32_t* ctl, uint32_t d, uint32_t* s_scan) {
-  uint32_t x = 0;
-  for (uint32_t i = threadIdx.x; i < kRadix; i += NT)
-    if (i < d) x += ctl[3 * kRadix + i];
-  uint32_t tot;
-  block_excl_scan<NT>(x, s_scan, tot);
-  return tot;
+__device__ __forceinline__ KeyMap sample_map(const Loader& ld, uint32_t* s_min, uint32_t* s_max) {
+  static_assert(NT == 512, "one sample a thread");
+  const uint32_t npad = ld.npad(), cnt = ld.n - npad;
+  bool bad;
+  const uint32_t kv = ld.load_key(npad + uint32_t(uint64_t(threadIdx.x) * cnt / NT), bad);
+  const uint32_t mn = __reduce_min_sync(0xffffffffu, kv), mx = __reduce_max_sync(0xffffffffu, kv);
+  if (lane_id() == 0) {
+    s_min[threadIdx.x >> 5] = mn;
+    s_max[threadIdx.x >> 5] = mx;
+  }
+  __syncthreads();
+  const uint32_t w = lane_id() & uint32_t(NT / 32 - 1);
+  const uint32_t lo = __reduce_min_sync(0xffffffffu, s_min[w]), hi = __reduce_max_sync(0xffffffffu, s_max[w]);
+  const uint32_t ext = (hi - lo) / 128 + 1;
+  const uint32_t l = lo > ext ? lo - ext : 0u, h = hi < ~ext ? hi + ext : 0xFFFFFFFFu;
+  // (a float quotient: any factor near 2^40 / range does, the same in every
+  // CTA; the conversion saturates)
+  return KeyMap{l, max(1u, __float2uint_rd(__fdividef(1099511627776.0f, float(h - l) + 1.0f)))};
 }
 
 // Stable in-shared-memory rank of up to IPT items per thread of a warp-striped
 // block (item j of lane l of warp w is element w*32*IPT + j*32 + l): on return
 // s_whist[w][d] holds warp w's start inside digit d's run, s_excl[d] the run's
 // start, and rank[j] the item's position among its warp's items of its digit.
-template <int NT, int IPT>
-__device__ __forceinline__ void rank_block(const uint32_t (&kv)[IPT], uint32_t m, uint32_t base, int shift,
+// digit(kv) is below kRadix.  With ipt < IPT only the first ipt items of each
+// thread are ranked (the caller lays the block out with 32 ipt items a warp).
+template <int NT, int IPT, class Digit>
+__device__ __forceinline__ void rank_block(const uint32_t (&kv)[IPT], uint32_t m, uint32_t base, const Digit& digit,
                                            uint32_t (&rank)[IPT], uint32_t (*s_whist)[kRadix],
                                            uint32_t* s_excl, uint32_t* s_scan, uint32_t* digit_total,
-                                           uint32_t lo = 0) {
+                                           uint32_t lo = 0, int ipt = IPT) {
   constexpr int NW = NT / 32;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   for (uint32_t i = lane; i < kRadix; i += 32) s_whist[warp][i] = 0;
@@ -316,8 +351,9 @@ __device__ __forceinline__ void rank_block(const uint32_t (&kv)[IPT], uint32_t m
   const uint32_t lt = lanemask_lt();
 #pragma unroll
   for (int j = 0; j < IPT; ++j) {
+    if (j >= ipt) break;  // the same for the whole block
     const uint32_t p = base + j * 32 + lane;
-    const uint32_t d = (p < m && p >= lo) ? ((kv[j] >> shift) & 255u) : kNoDigit;
+    const uint32_t d = (p < m && p >= lo) ? digit(kv[j]) : kNoDigit;
     const uint32_t peers = warp_peers<9>(d);  // d <= kNoDigit = 256
     const uint32_t before = __popc(peers & lt);
     const uint32_t cnt = (d != kNoDigit) ? s_whist[warp][d] : 0u;
@@ -376,12 +412,21 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
       bad_any |= bad;
     }
   }
-  rank_block<kScatterThreads, kScatterIPT>(kv, n, base, 24, rank, s_whist, s_excl, s_scan, s_cnt, npad);
+  const KeyMap map = sample_map<kScatterThreads>(ld, s_cnt, s_cnt + kScatterWarps);
+  if (tile == gridDim.x - 1) {  // the last tile's CTA (the shortest) publishes the map and the buckets' bounds
+    if (tid < kRadix) ctl[kSortCtlBounds + tid] = tid ? map.lower(tid) : 0u;
+    if (tid == kRadix) {
+      ctl[kSortCtlMap] = map.lo;
+      ctl[kSortCtlMap + 1] = map.mul;
+    }
+  }
+  rank_block<kScatterThreads, kScatterIPT>(kv, n, base, [&](uint32_t k) { return map.bucket(k); }, rank, s_whist,
+                                           s_excl, s_scan, s_cnt, npad);
 #pragma unroll
   for (int j = 0; j < kScatterIPT; ++j) {
     const uint32_t p = base + j * 32 + lane;
     if (p < n && p >= npad) {
-      const uint32_t d = kv[j] >> 24;
+      const uint32_t d = map.bucket(kv[j]);
       const uint32_t pos = s_excl[d] + s_whist[warp][d] + rank[j];
       s_keys[pos] = kv[j];
       s_vals[pos] = v[j];
@@ -401,62 +446,84 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
   }
   if (tile == 0 && tid == 0 && npad) {
     bool bad;
-    atomicAdd(ctl + 3 * kRadix + (ld.load_key(0, bad) >> 24), npad);
+    atomicAdd(ctl + 3 * kRadix + map.bucket(ld.load_key(0, bad)), npad);
   }
   if (any_bad && tid == 0 && status) *reinterpret_cast<volatile uint32_t*>(status) = kErrBadKey;
 }
 
-// First position i in [0, m) with (a[i] >> fshift) >= bin, a sorted.
-__device__ __forceinline__ uint32_t lower_bound_bin(const uint32_t* a, uint32_t m, uint32_t bin, int fshift) {
+// First position i in [0, m) with a[i] >= kv, a sorted.
+__device__ __forceinline__ uint32_t lower_bound_sorted(const uint32_t* a, uint32_t m, uint32_t kv) {
   uint32_t lo = 0, hi = m;
   while (lo < hi) {
     const uint32_t mid = (lo + hi) >> 1;
-    if ((a[mid] >> fshift) < bin) lo = mid + 1; else hi = mid;
+    if (a[mid] < kv) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
 
-// Prefix-index entries of bins [bin0, bin0 + nbins) from the sorted run
-// a[0, m) that starts at position start and holds exactly those bins.
-__device__ __forceinline__ void bucket_fence(const uint32_t* a, uint32_t m, uint32_t start, uint32_t bin0,
-                                             uint32_t nbins, uint32_t* fence, int fshift) {
-  for (uint32_t i = threadIdx.x; i < nbins; i += blockDim.x)
-    fence[bin0 + i] = start + lower_bound_bin(a, m, bin0 + i, fshift);
-}
+// A bucket: its elements' key variables lie in [lo, hi]; `map` spreads them
+// over the sub-bins of the counting pass.
+// Sub-bin of kv: floor((kv - off) * mul / 2^32), for kv below base as for
+// base, kept below kSubBins; monotone.
+struct SubMap {
+  uint32_t base, off, mul;
+  // `width` key variables from base: for up to kSubBins of them each has a
+  // sub-bin of its own (off = base - 1: (x + 1) (2^32 - 1) / 2^32 is x)
+  static __device__ __forceinline__ SubMap of(uint32_t base, float width) {
+    if (width <= float(kSubBins)) return SubMap{base, base - 1u, 0xFFFFFFFFu};
+    return SubMap{base, base, __float2uint_rd(__fdividef(float(1ull << 44), width))};
+  }
+  __device__ __forceinline__ uint32_t sub(uint32_t kv) const {
+    return min(__umulhi(max(kv, base) - off, mul), kSubBins - 1);
+  }
+  // the largest key variable of sub-bin s
+  __device__ __forceinline__ uint32_t last(uint32_t s) const {
+    return off + uint32_t(((uint64_t(s + 1) << 32) + mul - 1) / mul) - 1;
+  }
+};
+static_assert(kSubBins == 4096, "2^44 = kSubBins * 2^32");
+struct BucketRange {
+  uint32_t lo, hi;
+  SubMap map;
+};
+struct PadRun {   // n copies of (kv, v) that belong to the bucket but are not among its elements
+  uint32_t n, kv, v;
+};
+struct BinRange {  // prefix-index entries [bin0, bin1) to write (bin P starts at key variable P << fshift)
+  uint32_t* fence;
+  int fshift;
+  uint32_t bin0, bin1;
+};
 
-// Writes the sorted run a/av[0, m) (shared memory) to out[start ..) with
-// the padding run inserted before the first element >= pad_kv, and the
-// prefix-index entries of bins [bin0, bin0 + nbins) of the result.
-__device__ __forceinline__ void bucket_write(const uint32_t* a, const uint32_t* av, uint32_t m, uint32_t* out_k,
-                                             uint32_t* out_v, uint32_t start, uint32_t pad, uint32_t pad_kv,
-                                             uint32_t pad_v, uint32_t* fence, int fshift, uint32_t bin0,
-                                             uint32_t nbins) {
-  uint32_t L = m;
-  if (pad) {
-    uint32_t lo = 0, hi = m;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (a[mid] < pad_kv) lo = mid + 1; else hi = mid;
-    }
-    L = lo;
+// A bucket after its sort, for reading back: either sorted (cnt null), or in
+// sub-bins in no order, cnt[s] being the first position of sub-bin s.
+struct SortedView {
+  const uint32_t* a;
+  uint32_t m;
+  const uint32_t* cnt;
+  SubMap map;
+  __device__ __forceinline__ uint32_t end(uint32_t s) const { return s + 1 < kSubBins ? cnt[s + 1] : m; }
+  // number of elements below kv
+  __device__ __forceinline__ uint32_t less(uint32_t kv) const {
+    if (!cnt) return lower_bound_sorted(a, m, kv);
+    const uint32_t s = map.sub(kv), e = end(s);
+    uint32_t c = cnt[s];
+    for (uint32_t y = c; y < e; ++y) c += a[y] < kv ? 1u : 0u;
+    return c;
   }
-  for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-    const uint32_t dst = start + i + (i >= L ? pad : 0u);
-    out_k[dst] = a[i];
-    out_v[dst] = av[i];
+  __device__ __forceinline__ uint32_t smallest() const {
+    uint32_t k = a[0];
+    if (cnt)
+      for (uint32_t y = 1, e = end(map.sub(k)); y < e; ++y) k = min(k, a[y]);
+    return k;
   }
-  for (uint32_t j = threadIdx.x; j < pad; j += blockDim.x) {
-    out_k[start + L + j] = pad_kv;
-    out_v[start + L + j] = pad_v;
+  __device__ __forceinline__ uint32_t largest() const {
+    uint32_t k = a[m - 1];
+    if (cnt)
+      for (uint32_t y = cnt[map.sub(k)]; y < m; ++y) k = max(k, a[y]);
+    return k;
   }
-  if (fence) {
-    const uint32_t pad_bin = pad ? fence_bin(pad_kv, fshift) : 0xFFFFFFFFu;
-    for (uint32_t i = threadIdx.x; i < nbins; i += blockDim.x) {
-      const uint32_t bin = bin0 + i;
-      fence[bin] = start + lower_bound_bin(a, m, bin, fshift) + (bin > pad_bin ? pad : 0u);
-    }
-  }
-}
+};
 
 // Where element i of a bucket lives in the scratch its sort reads.
 // ContigSrc: elements start .. start + m - 1 (the batched form's scatter
@@ -464,23 +531,30 @@ __device__ __forceinline__ void bucket_write(const uint32_t* a, const uint32_t* 
 // tiles, in tile order (the stable order); rstart[t] is the first bucket
 // position of run t (an exclusive scan of the run lengths) and run t's
 // element i - rstart[t] sits at rbase[t] + i (both in shared memory).
+// at(i) serves buckets in shared memory; find(i) any; seek(i, t) any, for i
+// that never go down from call to call (t starts at 0 and follows the runs).
 struct ContigSrc {
   uint32_t start;
   __device__ __forceinline__ uint32_t at(uint32_t i) const { return start + i; }
+  __device__ __forceinline__ uint32_t find(uint32_t i) const { return start + i; }
+  __device__ __forceinline__ uint32_t seek(uint32_t i, uint32_t&) const { return start + i; }
 };
 struct RunSrc {
   const uint32_t* rstart;  // nruns + 1 entries, rstart[nruns] = the bucket's size
   const uint32_t* rbase;
-  const uint8_t* chunk;    // run holding element 16 c, per 16-element chunk c (buckets in shared memory), or null
+  const uint8_t* chunk;    // run holding element 16 c, per 16-element chunk c (buckets in shared memory only)
   uint32_t nruns;          // >= 1
-  // the largest t with rstart[t] <= i: the run holding i (empty runs share
-  // their start with the next run, so they are never the largest)
   __device__ __forceinline__ uint32_t at(uint32_t i) const {
-    if (chunk) {  // from the run of the chunk's first element, forward (runs of ~16 elements)
-      uint32_t t = chunk[i >> 4];
-      while (rstart[t + 1] <= i) ++t;
-      return rbase[t] + i;
-    }
+    uint32_t t = chunk[i >> 4];  // from the run of the chunk's first element, forward (runs of ~16 elements)
+    return seek(i, t);
+  }
+  // the run holding i: the largest t with rstart[t] <= i (empty runs share
+  // their start with the next run, so they are never the largest)
+  __device__ __forceinline__ uint32_t seek(uint32_t i, uint32_t& t) const {
+    while (rstart[t + 1] <= i) ++t;
+    return rbase[t] + i;
+  }
+  __device__ __forceinline__ uint32_t find(uint32_t i) const {
     uint32_t lo = 0, hi = nruns - 1;
     while (lo < hi) {
       const uint32_t mid = (lo + hi + 1) >> 1;
@@ -491,300 +565,472 @@ struct RunSrc {
 };
 static_assert(kMsdMaxTiles <= 256u, "a run index fits in a byte");
 
-// One bucket, one CTA of kBucketThreads: sorts the m elements src.at(0 ..
-// m - 1) of (src_k, src_v) stably by the low `rest` bits of the key variable
-// (the bits above are the bucket's and equal) into out[start, start + m),
-// and writes the prefix-index entries of the bucket's bins [bin0, bin0 +
-// nbins) when fence is given.
-//   Fast path (bucket in shared memory, no sub-bin above kSubBinMax): one
-//   counting pass on the top 12 of the `rest` bits places every element in
-//   its sub-bin (about one element each for spread keys), at an arbitrary
-//   slot; every element then goes to its sub-bin's start plus its rank in
-//   the sub-bin by (key variable, index in the bucket), the stable order.
-//   Otherwise: ceil(rest / 8) stable 8-bit passes in shared memory, or, for
-//   a bucket above kBucketCap (heavy duplicate keys), the same passes in
-//   chunks through global memory, alternating between out and spill (both
-//   indexed like out: [start, start + m) belongs to this bucket alone).
-// A run of `pad` copies of (pad_kv, pad_v) (a short batch's padding, which
-// comes first among equal key variables in the stable order) is written at
-// its sorted place: the output holds m + pad elements.
-// bsm holds 4 kBucketCap words plus kBucketCap 16-bit indexes.
-template <class Src>
-__device__ __forceinline__ void bucket_body(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
-                                            uint32_t* spill_k, uint32_t* spill_v, uint32_t* out_k, uint32_t* out_v,
-                                            uint32_t start, uint32_t m, int rest, uint32_t* __restrict__ fence,
-                                            int fshift, uint32_t bin0, uint32_t nbins, uint32_t* bsm,
-                                            uint32_t* s_scan, uint32_t pad, uint32_t pad_kv, uint32_t pad_v) {
-  __shared__ uint32_t s_whist[kBucketWarps][kRadix];
-  __shared__ uint32_t s_excl[kRadix], s_run[kRadix], s_tot[kRadix];
-  __shared__ uint32_t s_max;
-  uint32_t* ak = bsm;
-  uint32_t* av = bsm + kBucketCap;
-  uint32_t* bk = bsm + 2 * kBucketCap;
-  uint32_t* bv = bsm + 3 * kBucketCap;
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  const uint32_t wbase = warp * (32 * kBucketIPT);
-  const int npass = (rest + 7) / 8;
-  uint32_t kv[kBucketIPT], v[kBucketIPT], rank[kBucketIPT];
-  static_assert(kSubBins == kBucketWarps * kRadix, "the counters reuse the per-warp histograms");
+// Shared memory of a bucket's CTA.
+struct BucketShared {
+  uint32_t whist[kBucketWarps][kRadix];  // also the kSubBins counters
+  uint32_t excl[kRadix], scan[kBucketWarps];
+  uint32_t max, cnt[3], mn, mx;
+  uint64_t scan64[kBucketWarps];
+  uint32_t cand[kBucketWarps], votes[kBucketWarps];
+};
 
-  if (m <= kBucketCap && rest >= 12) {
-    uint32_t* cnt = &s_whist[0][0];
-    uint16_t* bi = reinterpret_cast<uint16_t*>(bsm + 4 * kBucketCap);
-    const int sh = rest - 12;
-    for (uint32_t i = tid; i < kSubBins; i += kBucketThreads) cnt[i] = 0u;
-    if (tid == 0) s_max = 0u;
+// Sorts m <= kBucketCap elements stably by the key variable (all in
+// [range.lo, range.hi]) and hands each to emit(position, kv, value).  With
+// kGather the elements are read from the source, otherwise bsm holds them in
+// order (kBucketCap words of keys, then the values).
+//   Fast path (no sub-bin above kSubBinMax): one counting pass places every
+//   element in its sub-bin (about one element each for spread keys), at an
+//   arbitrary slot; every element is then emitted at its sub-bin's start plus
+//   its rank in the sub-bin by (key variable, index), the stable order.  Its
+//   place differs from its slot by less than a sub-bin, so the caller's
+//   stores are nearly in order.
+//   Otherwise stable 8-bit passes over the bits in which the range differs.
+// bsm holds 4 kBucketCap words plus kBucketCap 16-bit indexes.  The view
+// returned stays valid until bsm or sh.whist change.
+template <bool kGather, class Src, class Emit>
+__device__ __forceinline__ SortedView sort_resident(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
+                                                    uint32_t m, const BucketRange& range, uint32_t* bsm,
+                                                    BucketShared& sh, const Emit& emit) {
+  static_assert(kSubBins == kBucketWarps * kRadix, "the counters reuse the per-warp histograms");
+  uint32_t *ak = bsm, *av = bsm + kBucketCap, *bk = bsm + 2 * kBucketCap, *bv = bsm + 3 * kBucketCap;
+  uint16_t* bi = reinterpret_cast<uint16_t*>(bsm + 4 * kBucketCap);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  uint32_t* cnt = &sh.whist[0][0];
+  uint32_t kv[kBucketIPT], v[kBucketIPT];
+#pragma unroll
+  for (int j = 0; j < kBucketIPT; ++j) {
+    const uint32_t i = tid + j * kBucketThreads;
+    if (i < m) {
+      const uint32_t at = kGather ? src.at(i) : i;
+      kv[j] = kGather ? src_k[at] : ak[at];
+      v[j] = kGather ? src_v[at] : av[at];
+    }
+  }
+  for (uint32_t i = tid; i < kSubBins; i += kBucketThreads) cnt[i] = 0u;
+  if (tid == 0) sh.max = 0u;
+  __syncthreads();
+  uint32_t slot[kBucketIPT];  // sub-bin, and above bit 16 the slot there
+#pragma unroll
+  for (int j = 0; j < kBucketIPT; ++j) {
+    if (tid + j * kBucketThreads < m) {
+      const uint32_t sb = range.map.sub(kv[j]);
+      slot[j] = sb | (atomicAdd(&cnt[sb], 1u) << 16);
+    }
+  }
+  __syncthreads();
+  // sub-bin starts: thread t owns counters [8 t, 8 t + 8)
+  constexpr int kPer = int(kSubBins) / kBucketThreads;
+  uint32_t c[kPer], sum = 0, mx = 0;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
+    c[e] = cnt[tid * kPer + e];
+    sum += c[e];
+    mx = max(mx, c[e]);
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0 && mx > kSubBinMax) atomicMax(&sh.max, mx);
+  uint32_t all;
+  uint32_t run = block_excl_scan<kBucketThreads>(sum, sh.scan, all);
+  if (sh.max <= kSubBinMax) {  // uniform: sh.max settled before the scan's barriers
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      cnt[tid * kPer + e] = run;
+      run += c[e];
+    }
     __syncthreads();
-    uint32_t slot[kBucketIPT];
 #pragma unroll
     for (int j = 0; j < kBucketIPT; ++j) {
       const uint32_t i = tid + j * kBucketThreads;
       if (i < m) {
-        const uint32_t at = src.at(i);
-        const uint32_t k = src_k[at];
-        ak[i] = k;
-        av[i] = src_v[at];
-        slot[j] = atomicAdd(&cnt[(k >> sh) & (kSubBins - 1)], 1u);
+        const uint32_t pos = cnt[slot[j] & 0xFFFFu] + (slot[j] >> 16);
+        bk[pos] = kv[j];
+        bv[pos] = v[j];
+        bi[pos] = uint16_t(i);
       }
     }
     __syncthreads();
-    // sub-bin starts: thread t owns counters [8 t, 8 t + 8)
-    constexpr int kPer = int(kSubBins) / kBucketThreads;
-    uint32_t c[kPer], sum = 0, mx = 0;
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-      c[e] = cnt[tid * kPer + e];
-      sum += c[e];
-      mx = max(mx, c[e]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0 && mx > kSubBinMax) atomicMax(&s_max, mx);
-    uint32_t all;
-    uint32_t run = block_excl_scan<kBucketThreads>(sum, s_scan, all);
-    if (s_max <= kSubBinMax) {  // uniform: s_max settled before the scan's barriers
-#pragma unroll
-      for (int e = 0; e < kPer; ++e) {
-        cnt[tid * kPer + e] = run;
-        run += c[e];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t i = tid + j * kBucketThreads;
-        if (i < m) {
-          const uint32_t k = ak[i];
-          const uint32_t pos = cnt[(k >> sh) & (kSubBins - 1)] + slot[j];
-          bk[pos] = k;
-          bv[pos] = av[i];
-          bi[pos] = uint16_t(i);
-        }
-      }
-      __syncthreads();
-      // Every element's place: its sub-bin's start plus its rank there by
-      // (key variable, index), the stable order.  Each element counts the
-      // members of its sub-bin that precede it (independent loads, about
-      // two a sub-bin for spread keys) rather than a per-sub-bin insertion
-      // sort, whose shifting chain made a warp wait for its fullest sub-bin.
+    // Each element counts the members of its sub-bin that precede it
+    // (independent loads, about two a sub-bin for spread keys) rather than a
+    // per-sub-bin insertion sort, whose shifting chain made a warp wait for
+    // its fullest sub-bin.
+    const SortedView view{bk, m, cnt, range.map};
 #pragma unroll 2
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t x = tid + j * kBucketThreads;
-        if (x < m) {
-          const uint32_t k = bk[x], vv = bv[x];
+    for (int j = 0; j < kBucketIPT; ++j) {
+      const uint32_t x = tid + j * kBucketThreads;
+      if (x < m) {
+        const uint32_t k = bk[x], vv = bv[x];
+        const uint32_t b = range.map.sub(k);
+        const uint32_t s0 = cnt[b], s1 = view.end(b);
+        // The first four members without a branch (a sub-bin rarely holds
+        // more for spread keys, and a loop made each warp run as long as
+        // its fullest sub-bin), then the rest; equal key variables, which
+        // are rare too, are told apart by index afterwards.
+        uint32_t r = 0, eq = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+          const uint32_t ky = s0 + u < s1 ? bk[s0 + u] : 0xFFFFFFFFu;
+          r += ky < k ? 1u : 0u;
+          eq += ky == k ? 1u : 0u;
+        }
+        for (uint32_t y = s0 + 4; y < s1; ++y) {
+          r += bk[y] < k ? 1u : 0u;
+          eq += bk[y] == k ? 1u : 0u;
+        }
+        if (eq > 1) {
           const uint16_t ix = bi[x];
-          const uint32_t b = (k >> sh) & (kSubBins - 1);
-          const uint32_t s0 = cnt[b], s1 = b + 1 < kSubBins ? cnt[b + 1] : m;
-          // The first four members without a branch (a sub-bin rarely holds
-          // more for spread keys, and a loop made each warp run as long as
-          // its fullest sub-bin), then the rest.
-          uint32_t r = 0;
-#pragma unroll
-          for (uint32_t u = 0; u < 4; ++u) {
-            if (s0 + u < s1) {
-              const uint32_t ky = bk[s0 + u];
-              r += (ky < k || (ky == k && bi[s0 + u] < ix)) ? 1u : 0u;
-            }
-          }
-          for (uint32_t y = s0 + 4; y < s1; ++y) {
-            const uint32_t ky = bk[y];
-            r += (ky < k || (ky == k && bi[y] < ix)) ? 1u : 0u;
-          }
-          ak[s0 + r] = k;
-          av[s0 + r] = vv;
+          for (uint32_t y = s0; y < s1; ++y) r += bk[y] == k && bi[y] < ix ? 1u : 0u;
         }
+        emit(s0 + r, k, vv);
       }
-      __syncthreads();
-      // The prefix-index entries come from the sub-bin starts when a bin is
-      // a whole number of sub-bins (fshift >= sh): entry bin0 + j is the
-      // start of sub-bin j << (fshift - sh), after the padding run when the
-      // bin lies above the padding's bin.
-      const bool direct_fence = fence && fshift >= sh;
-      bucket_write(ak, av, m, out_k, out_v, start, pad, pad_kv, pad_v, direct_fence ? nullptr : fence, fshift, bin0,
-                   nbins);
-      if (direct_fence) {
-        const uint32_t pad_bin = pad ? fence_bin(pad_kv, fshift) : 0xFFFFFFFFu;
-        for (uint32_t j = tid; j < nbins; j += kBucketThreads) {
-          const uint32_t sb = j << (fshift - sh);
-          fence[bin0 + j] = start + (sb < kSubBins ? cnt[sb] : m) + (bin0 + j > pad_bin ? pad : 0u);
-        }
-      }
-      return;
     }
-    __syncthreads();  // skewed bucket: the pass-by-pass path below reloads it
+    return view;
   }
+  __syncthreads();
+  // Many copies of one key, or a cluster.  The block is laid out with as many
+  // items a thread as m needs, so that a small bucket's passes are short.
+  if (kGather) {
+#pragma unroll
+    for (int j = 0; j < kBucketIPT; ++j) {
+      const uint32_t i = tid + j * kBucketThreads;
+      if (i < m) {
+        ak[i] = kv[j];
+        av[i] = v[j];
+      }
+    }
+    __syncthreads();
+  }
+  const int ipt = int((m + kBucketThreads - 1) / kBucketThreads);
+  const uint32_t wbase = warp * 32u * uint32_t(ipt);
+  const int bits = 32 - __clz(int(range.hi - range.lo));
+  uint32_t rank[kBucketIPT];
+  for (int shift = 0; shift < bits; shift += 8) {
+#pragma unroll
+    for (int j = 0; j < kBucketIPT; ++j) {
+      if (j >= ipt) break;
+      const uint32_t p = wbase + j * 32 + lane;
+      kv[j] = p < m ? ak[p] : 0u;
+      v[j] = p < m ? av[p] : 0u;
+    }
+    const auto digit = [&](uint32_t k) { return ((k - range.lo) >> shift) & 255u; };
+    rank_block<kBucketThreads, kBucketIPT>(kv, m, wbase, digit, rank, sh.whist, sh.excl, sh.scan, nullptr, 0u, ipt);
+#pragma unroll
+    for (int j = 0; j < kBucketIPT; ++j) {
+      if (j >= ipt) break;
+      const uint32_t p = wbase + j * 32 + lane;
+      if (p < m) {
+        const uint32_t dg = digit(kv[j]);
+        const uint32_t pos = sh.excl[dg] + sh.whist[warp][dg] + rank[j];
+        bk[pos] = kv[j];
+        bv[pos] = v[j];
+      }
+    }
+    __syncthreads();
+    uint32_t* t;
+    t = ak; ak = bk; bk = t;
+    t = av; av = bv; bv = t;
+  }
+  for (uint32_t i = tid; i < m; i += kBucketThreads) emit(i, ak[i], av[i]);
+  return SortedView{ak, m, nullptr, range.map};
+}
 
-  if (m <= kBucketCap) {
-    if (rest < 12) {  // otherwise the fast path above has loaded the bucket already
-      for (uint32_t i = tid; i < m; i += kBucketThreads) {
-        const uint32_t at = src.at(i);
-        ak[i] = src_k[at];
-        av[i] = src_v[at];
-      }
-      __syncthreads();
-    }
-    uint32_t *sk = ak, *sv = av, *dk = bk, *dv = bv;
-    for (int pass = 0; pass < npass; ++pass) {
-      const int shift = 8 * pass;
+// A bucket above kBucketCap elements: taken in key order, a part at a time.
+// Each round looks at the elements of [a, b], the keys still to do:
+//   at most kBucketCap of them        gathered in order, sorted, written;
+//   all but at most kBucketCap have   the hot key's tombstones and regular
+//   one key (a hot key)               elements go straight to their places in
+//                                     order, the others as above, around them;
+//   otherwise                         b is lowered to the end of the longest
+//                                     prefix of sub-bins that fits.
+// A round reads the bucket two or three times (from L2), 8 independent loads
+// a thread at a time.  Bound by the one CTA's chain of rounds.  (Stable 8-bit
+// passes in chunks through global memory before: a sort of 2^20 pairs of which
+// 8 % have one key 448 -> 164 us, of 2^18 Zipf(1.1) pairs 130 -> 64 us.)
+template <class Src>
+__device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src_v, const Src src, uint32_t* out_k,
+                                      uint32_t* out_v, uint32_t start, uint32_t m, const BucketRange range,
+                                      const PadRun pad, uint32_t* bsm, BucketShared& sh) {
+  constexpr uint32_t kItems = 8, kChunk = kItems * kBucketThreads;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  uint32_t* cnt = &sh.whist[0][0];
+  const auto shift = [&](uint32_t kv) { return pad.n && kv >= pad.kv ? pad.n : 0u; };
+  // f(kv, valid) for every element, whole warps at a time, in no order
+  const auto for_each = [&](const auto& f) {
+    uint32_t t = 0;
+    for (uint32_t i0 = 0; i0 < m; i0 += kChunk) {
+      uint32_t k[kItems];
 #pragma unroll
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t p = wbase + j * 32 + lane;
-        kv[j] = p < m ? sk[p] : 0u;
-        v[j] = p < m ? sv[p] : 0u;
+      for (uint32_t j = 0; j < kItems; ++j) {
+        const uint32_t i = i0 + j * kBucketThreads + tid;
+        k[j] = i < m ? src_k[src.seek(i, t)] : 0u;
       }
-      rank_block<kBucketThreads, kBucketIPT>(kv, m, wbase, shift, rank, s_whist, s_excl, s_scan, nullptr);
 #pragma unroll
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t p = wbase + j * 32 + lane;
-        if (p < m) {
-          const uint32_t dg = (kv[j] >> shift) & 255u;
-          const uint32_t pos = s_excl[dg] + s_whist[warp][dg] + rank[j];
-          dk[pos] = kv[j];
-          dv[pos] = v[j];
-        }
-      }
-      __syncthreads();
-      uint32_t* t;
-      t = sk; sk = dk; dk = t;
-      t = sv; sv = dv; dv = t;
+      for (uint32_t j = 0; j < kItems; ++j) f(k[j], i0 + j * kBucketThreads + tid < m);
     }
-    bucket_write(sk, sv, m, out_k, out_v, start, pad, pad_kv, pad_v, fence, fshift, bin0, nbins);
-    return;
+  };
+  if (pad.n) {
+    if (tid == 0) sh.cnt[0] = 0u;
+    __syncthreads();
+    uint32_t L = 0;
+    for_each([&](uint32_t k, bool ok) { L += ok && k < pad.kv ? 1u : 0u; });
+    L = __reduce_add_sync(0xffffffffu, L);
+    if (lane == 0) atomicAdd(&sh.cnt[0], L);
+    __syncthreads();
+    L = sh.cnt[0];
+    for (uint32_t j = tid; j < pad.n; j += kBucketThreads) {
+      out_k[start + L + j] = pad.kv;
+      out_v[start + L + j] = pad.v;
+    }
   }
-  // Chunked: npass stable passes through global memory, kBucketCap elements
-  // at a time in order: pass 0 from the source to out, then alternating
-  // out -> spill -> out ...; an even pass count ends in spill and is copied
-  // to out.
-  const uint32_t* curk = out_k;
-  const uint32_t* curv = out_v;
-  uint32_t* dstk = out_k;
-  uint32_t* dstv = out_v;
-  for (int pass = 0; pass < npass; ++pass) {
-    const int shift = 8 * pass;
-    if (tid < kRadix) s_tot[tid] = 0;
+  uint32_t a = range.lo, b = range.hi, done = 0;
+  while (done < m) {
+    // A key that may be hot: the most frequent one within a warp among 512
+    // elements taken at even distances.
     __syncthreads();
-    for (uint32_t i = tid; i < m; i += kBucketThreads) {
-      const uint32_t k = pass == 0 ? src_k[src.at(i)] : curk[start + i];
-      atomicAdd(&s_tot[(k >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    uint32_t all;
-    const uint32_t ex = block_excl_scan<kBucketThreads>(tid < kRadix ? s_tot[tid] : 0u, s_scan, all);
-    if (tid < kRadix) s_run[tid] = ex;
-    __syncthreads();
-    for (uint32_t c0 = 0; c0 < m; c0 += kBucketCap) {
-      const uint32_t cm = (m - c0) < kBucketCap ? (m - c0) : kBucketCap;
-#pragma unroll
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t p = wbase + j * 32 + lane;
-        kv[j] = 0u;
-        v[j] = 0u;
-        if (p < cm) {
-          if (pass == 0) {
-            const uint32_t at = src.at(c0 + p);
-            kv[j] = src_k[at];
-            v[j] = src_v[at];
-          } else {
-            kv[j] = curk[start + c0 + p];
-            v[j] = curv[start + c0 + p];
-          }
-        }
-      }
-      rank_block<kBucketThreads, kBucketIPT>(kv, cm, wbase, shift, rank, s_whist, s_excl, s_scan, s_tot);
-#pragma unroll
-      for (int j = 0; j < kBucketIPT; ++j) {
-        const uint32_t p = wbase + j * 32 + lane;
-        if (p < cm) {
-          const uint32_t dg = (kv[j] >> shift) & 255u;
-          const uint32_t pos = s_run[dg] + s_whist[warp][dg] + rank[j];
-          dstk[start + pos] = kv[j];
-          dstv[start + pos] = v[j];
-        }
-      }
-      __syncthreads();
-      if (tid < kRadix) s_run[tid] += s_tot[tid];
-      __syncthreads();
-    }
-    curk = dstk;
-    curv = dstv;
-    dstk = (dstk == out_k) ? spill_k : out_k;
-    dstv = (dstv == out_v) ? spill_v : out_v;
-  }
-  if (curk != out_k) {
-    for (uint32_t i = tid; i < m; i += kBucketThreads) {
-      out_k[start + i] = curk[start + i];
-      out_v[start + i] = curv[start + i];
-    }
-    __syncthreads();
-  }
-  if (pad) {
-    // open a gap of `pad` before the first element >= pad_kv: move the tail
-    // up, a block at a time from the end (each block read before written)
-    __shared__ uint32_t s_L;
     if (tid == 0) {
-      uint32_t lo = 0, hi = m;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (out_k[start + mid] < pad_kv) lo = mid + 1; else hi = mid;
-      }
-      s_L = lo;
+      sh.cnt[0] = sh.cnt[1] = sh.cnt[2] = 0u;
+      sh.mn = 0xFFFFFFFFu;
+      sh.mx = 0u;
+    }
+    const uint32_t one = src_k[src.find(uint32_t(uint64_t(tid) * m / kBucketThreads))];
+    const bool has = one >= a && one <= b;
+    const uint32_t peers = __match_any_sync(0xffffffffu, key_of(one)) & __ballot_sync(0xffffffffu, has);
+    const uint32_t most = __reduce_max_sync(0xffffffffu, has ? (uint32_t(__popc(peers)) << 5) | lane : 0u);
+    const uint32_t cand = __shfl_sync(0xffffffffu, key_of(one), int(most & 31u));
+    if (lane == 0) {
+      sh.cand[warp] = cand;
+      sh.votes[warp] = most >> 5;
     }
     __syncthreads();
-    const uint32_t L = s_L;
-    for (uint32_t e = m; e > L;) {
-      const uint32_t c = (e - L) < kBucketThreads ? (e - L) : kBucketThreads;
-      uint32_t k = 0, x = 0;
-      if (tid < c) {
-        k = out_k[start + e - c + tid];
-        x = out_v[start + e - c + tid];
+    uint32_t votes = 0, hot = 0;
+    for (int w = 0; w < kBucketWarps; ++w)
+      if (sh.votes[w] > votes) {
+        votes = sh.votes[w];
+        hot = sh.cand[w];
       }
-      __syncthreads();
-      if (tid < c) {
-        out_k[start + e - c + tid + pad] = k;
-        out_v[start + e - c + tid + pad] = x;
+    // the elements of [a, b]: how many, the range they span, how many below
+    // the candidate key and of it
+    uint32_t c = 0, mn = 0xFFFFFFFFu, mx = 0u, below = 0, copies = 0, tombs = 0;
+    for_each([&](uint32_t k, bool ok) {
+      if (ok && k >= a && k <= b) {
+        ++c;
+        mn = min(mn, k);
+        mx = max(mx, k);
+        below += key_of(k) < hot ? 1u : 0u;
+        copies += key_of(k) == hot ? 1u : 0u;
+        tombs += k == hot << 1 ? 1u : 0u;
       }
-      __syncthreads();
-      e -= c;
+    });
+    c = __reduce_add_sync(0xffffffffu, c);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    below = __reduce_add_sync(0xffffffffu, below);
+    copies = __reduce_add_sync(0xffffffffu, copies);
+    tombs = __reduce_add_sync(0xffffffffu, tombs);
+    if (lane == 0 && c) {
+      atomicAdd(&sh.cnt[0], c);
+      atomicMin(&sh.mn, mn);
+      atomicMax(&sh.mx, mx);
+      if (below) atomicAdd(&sh.cnt[1], below);
+      if (copies) atomicAdd(&sh.cnt[2], copies);
     }
-    for (uint32_t j = tid; j < pad; j += kBucketThreads) {
-      out_k[start + L + j] = pad_kv;
-      out_v[start + L + j] = pad_v;
+    if (lane == 0) sh.excl[warp] = tombs;
+    __syncthreads();
+    c = sh.cnt[0];
+    mn = sh.mn;
+    mx = sh.mx;
+    below = sh.cnt[1];
+    copies = sh.cnt[2];
+    tombs = 0;
+    for (int w = 0; w < kBucketWarps; ++w) tombs += sh.excl[w];
+    if (c == 0) {  // (only below an upper part that is still to do)
+      a = b + 1;
+      b = range.hi;
+      continue;
+    }
+    if (mn == mx) {  // one key variable (the candidate may be another key)
+      hot = key_of(mn);
+      below = 0;
+      copies = c;
+      tombs = mn & 1u ? 0u : c;
+    }
+    if (c - copies > kBucketCap) {
+      // Sub-bins over [mn, mx]; the lanes that share the sub-bin of the
+      // warp's first active lane add their count at once (hot keys would
+      // serialise the adds).
+      const SubMap map = SubMap::of(mn, float(mx - mn) + 1.0f);
+      __syncthreads();
+      for (uint32_t i = tid; i < kSubBins; i += kBucketThreads) cnt[i] = 0u;
+      if (tid == 0) sh.max = 0u;
+      __syncthreads();
+      for_each([&](uint32_t k, bool ok) {
+        const uint32_t s = ok && k >= a && k <= b ? map.sub(k) : kSubBins;
+        const uint32_t act = __ballot_sync(0xffffffffu, s < kSubBins);
+        if (!act) return;
+        const int lead = __ffs(int(act)) - 1;
+        const uint32_t same = __ballot_sync(0xffffffffu, s == __shfl_sync(0xffffffffu, s, lead));
+        if (int(lane) == lead) atomicAdd(&cnt[s], uint32_t(__popc(same)));
+        else if (s < kSubBins && !((same >> lane) & 1u)) atomicAdd(&cnt[s], 1u);
+      });
+      __syncthreads();
+      constexpr uint32_t kPer = kSubBins / kBucketThreads;
+      uint32_t sum = 0;
+      for (uint32_t e = 0; e < kPer; ++e) sum += cnt[tid * kPer + e];
+      uint32_t all, fit = 0;  // sub-bins [0, fit) hold at most kBucketCap elements
+      uint32_t run = block_excl_scan<kBucketThreads>(sum, sh.scan, all);
+      for (uint32_t e = 0; e < kPer; ++e) {
+        run += cnt[tid * kPer + e];
+        if (run <= kBucketCap) fit = tid * kPer + e + 1;
+      }
+      if (fit) atomicMax(&sh.max, fit);
+      __syncthreads();
+      fit = sh.max;
+      a = mn;
+      b = map.last(fit ? fit - 1 : 0u);
+      continue;
+    }
+    if (c <= kBucketCap) copies = tombs = 0;  // all of them fit: no key is singled out
+    // gather [a, b] in order: copies of the hot key to their places, the
+    // rest to shared memory; a warp takes 256 consecutive elements
+    uint32_t *ak = bsm, *av = bsm + kBucketCap;
+    uint32_t kept = 0, dst0 = start + done + below + shift(hot << 1),
+             dst1 = start + done + below + tombs + shift((hot << 1) | 1u), t = 0;
+    const uint32_t lt = lanemask_lt();
+    for (uint32_t c0 = 0; c0 < m; c0 += kChunk) {
+      uint32_t k[kItems], v[kItems];
+#pragma unroll
+      for (uint32_t j = 0; j < kItems; ++j) {
+        const uint32_t i = c0 + warp * (32 * kItems) + j * 32 + lane;
+        const uint32_t at = i < m ? src.seek(i, t) : 0u;
+        k[j] = i < m ? src_k[at] : 0u;
+        v[j] = i < m ? src_v[at] : 0u;
+      }
+      // kind of element j of this lane, two bits: 0 outside [a, b], 1 to
+      // shared memory, 2 a tombstone of the hot key, 3 a regular element of it
+      uint32_t kind = 0, n1 = 0, n2 = 0, n3 = 0;
+#pragma unroll
+      for (uint32_t j = 0; j < kItems; ++j) {
+        const bool in = c0 + warp * (32 * kItems) + j * 32 + lane < m && k[j] >= a && k[j] <= b;
+        const uint32_t x = !in ? 0u : (copies && key_of(k[j]) == hot ? 2u + (k[j] & 1u) : 1u);
+        kind |= x << (2 * j);
+        const uint32_t lo = __ballot_sync(0xffffffffu, x & 1u), hi = __ballot_sync(0xffffffffu, x & 2u);
+        n1 += __popc(lo & ~hi);
+        n2 += __popc(hi & ~lo);
+        n3 += __popc(lo & hi);
+      }
+      __syncthreads();
+      if (lane == 0) sh.cand[warp] = n1 | (n2 << 10) | (n3 << 20);
+      __syncthreads();
+      uint32_t p1 = kept, p2 = dst0, p3 = dst1;
+      for (uint32_t w = 0; w < uint32_t(kBucketWarps); ++w) {
+        const uint32_t x = sh.cand[w];
+        const bool before = w < warp;
+        p1 += before ? x & 1023u : 0u;
+        p2 += before ? (x >> 10) & 1023u : 0u;
+        p3 += before ? x >> 20 : 0u;
+        kept += x & 1023u;
+        dst0 += (x >> 10) & 1023u;
+        dst1 += x >> 20;
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < kItems; ++j) {
+        const uint32_t x = (kind >> (2 * j)) & 3u;
+        const uint32_t lo = __ballot_sync(0xffffffffu, x & 1u), hi = __ballot_sync(0xffffffffu, x & 2u);
+        const uint32_t mask = (x & 1u ? lo : ~lo) & (x & 2u ? hi : ~hi);
+        const uint32_t at = (x == 1u ? p1 : (x == 2u ? p2 : p3)) + __popc(mask & lt);
+        if (x == 1u) {
+          ak[at] = k[j];
+          av[at] = v[j];
+        } else if (x) {
+          out_k[at] = k[j];
+          out_v[at] = v[j];
+        }
+        p1 += __popc(lo & ~hi);
+        p2 += __popc(hi & ~lo);
+        p3 += __popc(lo & hi);
+      }
     }
     __syncthreads();
+    if (kept) {
+      const BucketRange part{mn, mx, SubMap::of(mn, float(mx - mn) + 1.0f)};
+      sort_resident<false>(src_k, src_v, src, kept, part, bsm, sh, [&](uint32_t i, uint32_t kk, uint32_t vv) {
+        const uint32_t dst = start + done + i + (copies && key_of(kk) > hot ? copies : 0u) + shift(kk);
+        out_k[dst] = kk;
+        out_v[dst] = vv;
+      });
+    }
+    done += c;
+    a = b + 1;
+    b = range.hi;
   }
-  if (fence) bucket_fence(out_k + start, m + pad, start, bin0, nbins, fence, fshift);
+  __syncthreads();  // the caller reads the output back
+}
+
+// One bucket, one CTA of kBucketThreads: sorts the m elements src.at(0 ..
+// m - 1) of (src_k, src_v) stably by the key variable into out[start, start +
+// m + pad.n) and writes the prefix-index entries `bins` of the result.  The
+// padding run (a short batch's, which comes first among equal key variables
+// in the stable order) is written at its sorted place.  `ends`: bit 0 when
+// the bucket holds the first element of the output, bit 1 the last; its
+// entries are then written inside the populated bin range only, whose bound
+// is recorded.
+template <class Src>
+__device__ __forceinline__ void bucket_body(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
+                                            uint32_t* out_k, uint32_t* out_v, uint32_t start, uint32_t m,
+                                            const BucketRange& range, const PadRun& pad, BinRange bins, int ends,
+                                            uint32_t* bsm, BucketShared& sh) {
+  SortedView view{out_k + start, m + pad.n, nullptr, range.map};
+  uint32_t extra = 0;  // padding elements that the view does not hold
+  if (m > kBucketCap) {
+    sort_big(src_k, src_v, src, out_k, out_v, start, m, range, pad, bsm, sh);
+  } else {
+    if (m)
+      view = sort_resident<true>(src_k, src_v, src, m, range, bsm, sh, [&](uint32_t i, uint32_t k, uint32_t v) {
+        const uint32_t dst = start + i + (pad.n && k >= pad.kv ? pad.n : 0u);
+        out_k[dst] = k;
+        out_v[dst] = v;
+      });
+    view.m = m;
+    extra = pad.n;
+    if (pad.n) {
+      const uint32_t L = m ? view.less(pad.kv) : 0u;
+      for (uint32_t j = threadIdx.x; j < pad.n; j += blockDim.x) {
+        out_k[start + L + j] = pad.kv;
+        out_v[start + L + j] = pad.v;
+      }
+    }
+  }
+  if (!bins.fence) return;
+  if (ends) {
+    const uint32_t nb = fence_bins(bins.fshift);
+    if (ends & 1) {
+      const uint32_t kv = min(view.m ? view.smallest() : pad.kv, extra ? pad.kv : 0xFFFFFFFFu);
+      bins.bin0 = max(bins.bin0, fence_bin(kv, bins.fshift) + 1);
+      if (threadIdx.x == 0) bins.fence[nb + 2] = fence_bin(kv, bins.fshift);
+    }
+    if (ends & 2) {
+      const uint32_t kv = max(view.m ? view.largest() : pad.kv, extra ? pad.kv : 0u);
+      bins.bin1 = min(bins.bin1, fence_bin(kv, bins.fshift) + 1);
+      if (threadIdx.x == 0) {
+        bins.fence[nb + 3] = fence_bin(kv, bins.fshift);
+        bins.fence[nb] = start + m + pad.n;
+      }
+    }
+  }
+  for (uint32_t P = bins.bin0 + threadIdx.x; P < bins.bin1; P += blockDim.x) {
+    const uint32_t kv = P << bins.fshift;
+    bins.fence[P] = start + (view.m ? view.less(kv) : 0u) + (extra && kv > pad.kv ? extra : 0u);
+  }
 }
 
 __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, const uint32_t* __restrict__ tmp_k,
                                                               const uint32_t* __restrict__ tmp_v,
-                                                              const uint2* __restrict__ runs, uint32_t* spill_k,
-                                                              uint32_t* spill_v, uint32_t* __restrict__ out_k,
-                                                              uint32_t* __restrict__ out_v,
-                                                              const uint32_t* __restrict__ ctl, uint32_t n,
-                                                              uint32_t* __restrict__ fence, int fshift,
+                                                              const uint2* __restrict__ runs, uint32_t* out_k,
+                                                              uint32_t* out_v, const uint32_t* __restrict__ ctl,
+                                                              uint32_t n, uint32_t* fence, int fshift,
                                                               uint32_t* __restrict__ next_ctl,
                                                               uint32_t* defer_err) {
   extern __shared__ __align__(16) uint32_t bsm[];
-  __shared__ uint32_t s_scan[kBucketWarps];
+  __shared__ BucketShared sh;
   __shared__ uint32_t s_rstart[kMsdMaxTiles + 1], s_rbase[kMsdMaxTiles];
   __shared__ uint8_t s_chunk[kBucketCap / 16];
   pdl_trigger();
@@ -815,10 +1061,18 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
     if (d == 0 && tid == 0) atomicOr(defer_err, kErrBadKey);
     return;
   }
-  // this bucket's run in every tile, in tile order
+  // this bucket's run in every tile, in tile order, and the buckets' totals
+  // (one round trip); one scan for the runs' starts and the sum of the totals
+  // before the bucket, its start in the output
   const uint2 run = tid < ntiles ? runs[d * kMsdMaxTiles + tid] : make_uint2(0u, 0u);
-  uint32_t m;
-  const uint32_t rs = block_excl_scan<kBucketThreads>(run.y, s_scan, m);
+  const uint32_t before = tid < d ? ctl[3 * kRadix + tid] : 0u;
+  const KeyMap map{ctl[kSortCtlMap], ctl[kSortCtlMap + 1]};
+  const bool top = d == kRadix - 1;
+  const uint32_t lo = ctl[kSortCtlBounds + d], next = top ? 0xFFFFFFFFu : ctl[kSortCtlBounds + d + 1];
+  const uint32_t hi = next == 0xFFFFFFFFu ? next : next - 1;
+  uint64_t sums;
+  const uint32_t rs = uint32_t(block_excl_scan<kBucketThreads, uint64_t>(run.y | (uint64_t(before) << 32), sh.scan64, sums));
+  const uint32_t m = uint32_t(sums), start = uint32_t(sums >> 32);
   if (tid < ntiles) {
     s_rstart[tid] = rs;
     s_rbase[tid] = run.x - rs;
@@ -827,24 +1081,29 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
       for (uint32_t c = (rs + 15) >> 4; c < ((rs + run.y + 15) >> 4); ++c) s_chunk[c] = uint8_t(tid);
   }
   if (tid == 0) s_rstart[ntiles] = m;
-  const uint32_t start = bucket_start<kBucketThreads>(ctl, d, s_scan);  // its barriers publish the tables
+  __syncthreads();
   // a short batch's padding: one run in the bucket of its key variable
-  uint32_t pad = ld.npad(), pad_kv = 0, pad_v = 0;
-  if (pad) {
+  PadRun pad{ld.npad(), 0u, 0u};
+  if (pad.n) {
     bool bad;
-    ld.load(0, pad_kv, pad_v, bad);
-    if ((pad_kv >> 24) != d) pad = 0;
+    ld.load(0, pad.kv, pad.v, bad);
+    if (map.bucket(pad.kv) != d) pad.n = 0;
   }
-  const uint32_t per = fence ? 1u << (24 - fshift) : 0u;  // bins per bucket
-  const RunSrc src{s_rstart, s_rbase, m <= kBucketCap ? s_chunk : nullptr, ntiles};
-  bucket_body(tmp_k, tmp_v, src, spill_k, spill_v, out_k, out_v, start, m, 24, fence, fshift, d * per, per, bsm,
-              s_scan, pad, pad_kv, pad_v);
-  // the bucket sort writes every entry: the populated range is all bins
-  if (fence && d == kRadix - 1 && tid == 0) {
-    fence[fence_bins(fshift)] = n;
-    fence[fence_bins(fshift) + 2] = 0u;
-    fence[fence_bins(fshift) + 3] = fence_bins(fshift) - 1;
+  const uint32_t total = m + pad.n;
+  // An empty bucket writes its bins too (they share the next element's
+  // position), unless nothing comes before or after it.
+  if (total == 0 && (start == 0 || start == n)) return;
+  BinRange bins{fence, fshift, 0u, 0u};
+  if (fence) {
+    bins.bin0 = d ? ((lo - 1) >> fshift) + 1 : 0u;
+    bins.bin1 = (hi >> fshift) + 1;
   }
+  // keys below the sampled range (bucket 0) and above it (bucket 255) share
+  // the sub-bins at that end
+  const BucketRange range{lo, hi, SubMap::of(d ? lo : map.lo, __fdividef(4294967296.0f, float(map.mul)) + 1.0f)};
+  const int ends = (total && start == 0 ? 1 : 0) | (total && start + total == n ? 2 : 0);
+  const RunSrc src{s_rstart, s_rbase, s_chunk, ntiles};
+  bucket_body(tmp_k, tmp_v, src, out_k, out_v, start, m, range, pad, bins, ends, bsm, sh);
 }
 
 __global__ void __launch_bounds__(256) check_keys(const uint32_t* __restrict__ keys, uint64_t n,
@@ -971,7 +1230,7 @@ __global__ void __launch_bounds__(kThreads) mseg_scatter(MultiArena ar, MultiBat
     if (p < m) multi_load(in, d, nops, t0 + p, kv[j], v[j]);
   }
   s_gbase[tid] = ar.tilecnt[uint64_t(gt) * 512 + 256 + tid];
-  rank_block<kThreads, kMultiIPT>(kv, m, base, shift, rank, s_whist, s_excl, s_scan, nullptr);
+  rank_block<kThreads, kMultiIPT>(kv, m, base, [&](uint32_t k) { return k >> shift; }, rank, s_whist, s_excl, s_scan, nullptr);
 #pragma unroll
   for (int j = 0; j < kMultiIPT; ++j) {
     const uint32_t p = base + j * 32 + lane;
@@ -1001,7 +1260,7 @@ __global__ void __launch_bounds__(kThreads) mseg_scatter(MultiArena ar, MultiBat
 // buffer, with that run's prefix-index entries.
 __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) {
   extern __shared__ __align__(16) uint32_t bsm[];
-  __shared__ uint32_t s_scan[kBucketWarps];
+  __shared__ BucketShared sh;
   const uint32_t gb = blockIdx.x;
   const uint32_t i = find_instance(ar.bucket_prefix, ar.n, gb);
   const int k = ar.k[i];
@@ -1024,8 +1283,10 @@ __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) 
   const uint32_t per = 1u << (rest - fs);             // bins per bucket
   uint32_t* tk = ar.tkeys + d.boff;
   uint32_t* tv = ar.tvals + d.boff;
-  bucket_body(tk, tv, ContigSrc{start}, tk, tv, ok, ov, start, m, rest, of, fs, bucket * per, per, bsm, s_scan, 0u,
-              0u, 0u);
+  const uint32_t blo = bucket << rest;
+  bucket_body(tk, tv, ContigSrc{start}, ok, ov, start, m,
+              BucketRange{blo, blo + ((1u << rest) - 1u), SubMap::of(blo, float(1u << rest))}, PadRun{0u, 0u, 0u},
+              BinRange{of, fs, bucket * per, bucket * per + per}, 0, bsm, sh);
   if (bucket == (1u << d.msd_bits) - 1 && threadIdx.x == 0) {
     const uint32_t nb = fence_bins(fs);
     of[nb] = d.b;
@@ -1047,8 +1308,6 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   if ((e = set_smem_attr_once(bucket_sort, kBucketSmem, dev, g_bucket_attr)) != cudaSuccess) return e;
   const uint32_t ntiles = (a.n + kMsdTile - 1) / kMsdTile;
   uint2* runs = reinterpret_cast<uint2*>(ws.tilecnt);
-  uint32_t* spill_k = ws.tilecnt + kMsdRunWords;
-  uint32_t* spill_v = spill_k + a.n;
   uint32_t* ctl = ws.ctl + ws.flip * kSortCtlWords;
   uint32_t* next = ws.ctl + (ws.flip ^ 1) * kSortCtlWords;
   Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, a.n_in, a.n};
@@ -1062,7 +1321,7 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   count_launches(1);
   if ((e = launch_pdl(bucket_sort, dim3(kRadix), dim3(kBucketThreads), kBucketSmem, st, ld,
                       static_cast<const uint32_t*>(a.tmp_keys), static_cast<const uint32_t*>(a.tmp_vals),
-                      static_cast<const uint2*>(runs), spill_k, spill_v, a.out_keys, a.out_vals,
+                      static_cast<const uint2*>(runs), a.out_keys, a.out_vals,
                       static_cast<const uint32_t*>(ctl), a.n, a.fence, a.fshift, next, a.defer_err)) != cudaSuccess)
     return e;
   ws.flip ^= 1;
@@ -1159,7 +1418,7 @@ cudaError_t multi_sort_launch(const MultiArena& ar, const MultiBatch& in, cudaSt
 // raw cudaMalloc, or a latency-bound loop that cannot afford the implicit
 // device-wide synchronisation and the unbounded time a cudaMalloc/cudaFree
 // may take.  For them the sort below takes all of its scratch (the
-// bucket sort's tile scratch, control words, run table and spill area) from
+// bucket sort's tile scratch, control words and run table) from
 // one fixed array with static storage in this file, which every GPU that
 // loads the library holds until the process exits.  Its size is set by
 // kNoAllocMaxPairs.
@@ -1179,12 +1438,12 @@ constexpr size_t kNoAllocCtl = 2112;                    // > 2 * kSortCtlWords, 
 constexpr size_t kNoAllocSticky = kNoAllocCtl - 1;      // last ctl word: device error bits
 constexpr size_t kNoAllocTmpK = kNoAllocCtl;
 constexpr size_t kNoAllocTmpV = kNoAllocTmpK + kNoAllocMaxPairs;
-constexpr size_t kNoAllocRuns = kNoAllocTmpV + kNoAllocMaxPairs;  // run table + spill area
-constexpr size_t kNoAllocWords = kNoAllocRuns + kMsdWsWords;
+constexpr size_t kNoAllocRuns = kNoAllocTmpV + kNoAllocMaxPairs;  // run table
+constexpr size_t kNoAllocWords = kNoAllocRuns + kMsdRunWords;
 static_assert(kNoAllocCtl > 2 * size_t(kSortCtlWords), "both control halves and the error word fit");
 static_assert(kNoAllocRuns % 2 == 0, "the run table holds 8-byte entries");
 
-// The scratch itself: about 17 MB for kNoAllocMaxPairs = 2^20.
+// The scratch itself: about 9 MB for kNoAllocMaxPairs = 2^20.
 static __device__ __align__(256) uint32_t g_sort_scratch[kNoAllocWords];
 
 constexpr int kNoAllocMaxDevices = 64;

@@ -1,0 +1,107 @@
+"""The batch sort over key ranges and repetitions (needs a GPU).
+
+The bucket sort splits the sampled key range of the batch; these inputs put its edges to work: ranges of a few keys,
+ranges away from zero and at the top, outliers that the sample misses, clusters that overflow one bucket, hot keys
+(alone, several in one bucket, with the padding of a short batch among them).  Every comparison is exact.
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOP = (1 << 31) - 1
+
+
+@pytest.fixture(scope="module")
+def g(lsm_lib):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return lsm_lib
+
+
+def draw(dist, n, rng):
+    """n keys below 2^31 - 1."""
+    if dist == "one":
+        return np.full(n, 12345, np.uint32)
+    if dist == "two":
+        return rng.integers(TOP - 2, TOP, n).astype(np.uint32)
+    if dist == "ids":
+        return rng.permutation(n).astype(np.uint32)
+    if dist == "offset":
+        return (1500000000 + rng.integers(0, 3 * n, n)).astype(np.uint32)
+    if dist == "outliers":   # a few keys far from the rest: the range they span leaves most buckets empty
+        k = 700000000 + rng.integers(0, 1 << 18, n)
+        at = rng.integers(0, n, max(1, n // 5000))
+        k[at] = rng.integers(0, TOP, len(at))
+        return k.astype(np.uint32)
+    if dist == "cluster":    # half of the keys in 2^12 values, the rest spread
+        return np.where(rng.random(n) < 0.5, 5000 + rng.integers(0, 1 << 12, n), rng.integers(0, TOP, n)).astype(np.uint32)
+    if dist == "hot":        # one key three tenths, two neighbours a tenth each
+        u = rng.random(n)
+        k = rng.integers(0, TOP, n)
+        return np.where(u < 0.3, 1 << 30, np.where(u < 0.4, (1 << 30) + 1, np.where(u < 0.5, (1 << 30) - 7, k))).astype(np.uint32)
+    if dist == "zipf":
+        return ((rng.zipf(1.1, n) % (1 << 30)).astype(np.uint64) * 0x9E3779B1 % (1 << 30)).astype(np.uint32)
+    raise ValueError(dist)
+
+
+DISTS = ["one", "two", "ids", "offset", "outliers", "cluster", "hot", "zipf"]
+
+
+@pytest.mark.parametrize("n", [1, 511, 4097, 70001, 1 << 18, 1 << 20])
+@pytest.mark.parametrize("dist", DISTS)
+def test_sort_over_ranges(g, dist, n):
+    rng = np.random.default_rng(n * 31 + DISTS.index(dist))
+    # keys of sort_pairs are whole 32-bit words; values are positions, so stability shows
+    keys = (draw(dist, n, rng) << np.uint32(1)) | rng.integers(0, 2, n).astype(np.uint32)
+    vals = np.arange(n, dtype=np.uint32)
+    lsm = g.LSM(n, n)
+    kd, vd = g.as_device_u32(keys, 0), g.as_device_u32(vals, 0)
+    ko, vo = torch.zeros_like(kd), torch.zeros_like(vd)
+    g.lsm_sort_pairs(lsm.h, kd.data_ptr(), vd.data_ptr(), ko.data_ptr(), vo.data_ptr(), n,
+                     torch.cuda.current_stream().cuda_stream)
+    order = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(g.to_numpy_u32(ko), keys[order])
+    np.testing.assert_array_equal(g.to_numpy_u32(vo), vals[order])
+    assert lsm.device_errors() == 0
+    lsm.close()
+
+
+@pytest.mark.parametrize("short", [0, 1, 20000])
+@pytest.mark.parametrize("dist", DISTS)
+def test_levels_over_ranges(g, dist, short):
+    """Five batches, the last one short (padded), against the structural oracle and the ordered map."""
+    b, rng = 30000, np.random.default_rng(short + DISTS.index(dist))
+    lsm, s, o1 = g.LSM(b, 8 * b), oracle.StructuralOracle(b), oracle.MapOracle(b)
+    seen = []
+    for t in range(5):
+        n = b if t < 4 else b - short
+        k = draw(dist, n, rng)
+        v = rng.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+        d = (rng.random(n) < 0.2).astype(np.uint8)
+        for x in (lsm, s, o1):
+            x.call("update", k, v, d)
+        seen.append(k)
+    lv = lsm.levels()
+    assert lsm.r == s.r
+    for i, (kv, vv) in lv.items():
+        ekv, ev = s.level(i)
+        np.testing.assert_array_equal(kv, ekv)
+        np.testing.assert_array_equal(vv, ev)
+    keys = np.concatenate(seen)
+    q = np.concatenate([rng.choice(keys, 4000), rng.choice(keys, 500) + 1, [0, TOP - 1, TOP, 0xFFFFFFFF],
+                        rng.integers(0, TOP, 2000)]).astype(np.uint32)
+    val, found = lsm.lookup(q)
+    ev, ef = o1.lookup(q)
+    np.testing.assert_array_equal(found.cpu().numpy(), ef)
+    np.testing.assert_array_equal(g.to_numpy_u32(val), ev)
+    k1 = np.minimum(q[:3000], TOP - 1)
+    k2 = np.minimum(k1.astype(np.int64) + rng.integers(0, 300, len(k1)), TOP - 1).astype(np.uint32)
+    np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), o1.count(k1, k2))
+    assert lsm.device_errors() == 0
+    lsm.close()
