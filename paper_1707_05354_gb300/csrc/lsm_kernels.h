@@ -83,20 +83,8 @@ enum SortInput : int {
   kSortQueries = 4    // (keys[i], i): sort query keys with their positions
 };
 
-// Tuning of the batch sort (compile-time): items per thread (tile =
-// 256 * LSM_SORT_IPT elements), minimum resident CTAs per SM requested from
-// the compiler, and the number of predecessor tiles read per look-back step.
-#ifndef LSM_SORT_IPT
-#define LSM_SORT_IPT 16
-#endif
-#ifndef LSM_SORT_MINB
-#define LSM_SORT_MINB 1
-#endif
-#ifndef LSM_SORT_LBW
-#define LSM_SORT_LBW 8
-#endif
 constexpr int kSortPasses = 4;
-constexpr int kSortTile = 256 * LSM_SORT_IPT;  // elements per CTA tile of a pass
+constexpr int kSortTile = 8192;  // elements per CTA tile of a pass
 
 struct SortArgs {
   int mode;

@@ -7,7 +7,7 @@
 //   * sort_histogram reads the input once and counts all four digits; in the
 //     batch modes it also encodes each op as (key << 1) | status and checks
 //     that keys are below 2^31 - 1.
-//   * sort_pass ranks a tile of 4096 elements per CTA in shared memory, gets
+//   * sort_pass ranks a tile of 8192 elements per CTA in shared memory, gets
 //     the tile's global offset per digit from the tiles before it by
 //     decoupled look-back (tile order comes from an atomic ticket, so a CTA
 //     only ever waits on CTAs that already started), and scatters.
@@ -22,11 +22,13 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kIPT = kSortTile / kThreads;  // 16 items per thread
 constexpr int kRadix = 256;
 constexpr uint32_t kNoDigit = 256;
-constexpr int kLookbackWindow = LSM_SORT_LBW;
-static_assert(kThreads == kRadix, "one thread per digit in the look-back");
+// A pass: 512 threads of 16 items, the first 256 of them one digit each.
+constexpr int kPassThreads = 512;
+constexpr int kPassWarps = kPassThreads / 32;
+constexpr int kIPT = kSortTile / kPassThreads;
+constexpr int kLookbackWords = 8;  // predecessors a look-back thread reads per step
 
 // Look-back word: [epoch:30][flag:2][value:32].
 constexpr uint64_t kFlagAgg = 1, kFlagIncl = 2;
@@ -39,7 +41,7 @@ struct Loader {
   const uint32_t* keys;
   const uint32_t* vals;
   const uint8_t* del;
-  uint64_t n_in;
+  uint32_t n_in;  // ops in the input, 1 .. n
   uint32_t n;
 
   // Element p of the logical sequence.  Batch modes: position p of the
@@ -56,8 +58,7 @@ struct Loader {
       v = p;
       return;
     }
-    uint64_t s = uint64_t(n) - 1 - p;
-    if (s >= n_in) s = n_in - 1;
+    const uint32_t s = min(n - 1 - p, n_in - 1);
     // the key, delete flag and value loads are independent (insert and
     // update calls always pass values), so they are in flight together
     const uint32_t k = __ldg(keys + s);
@@ -72,15 +73,23 @@ struct Loader {
   // of op n_in - 1); 0 outside the batch modes.
   __device__ __forceinline__ uint32_t npad() const {
     if (mode == kSortPairs || mode == kSortQueries) return 0u;
-    return uint64_t(n) > n_in ? uint32_t(uint64_t(n) - n_in) : 0u;
+    return n - n_in;
+  }
+
+  // The value of element p, whose key variable is kv.
+  __device__ __forceinline__ uint32_t load_val(uint32_t p, uint32_t kv) const {
+    if (mode == kSortPairs) return __ldg(vals + p);
+    if (mode == kSortQueries) return p;
+    if (mode == kSortDelete || !(kv & 1u)) return 0u;  // tombstones (bad keys are placebo tombstones) carry 0
+    const uint32_t s = min(n - 1 - p, n_in - 1);
+    return __ldg(vals + s);
   }
 
   // Key variable only (the histogram needs no values).
   __device__ __forceinline__ uint32_t load_key(uint32_t p, bool& bad) const {
     bad = false;
     if (mode == kSortPairs || mode == kSortQueries) return __ldg(keys + p);
-    uint64_t s = uint64_t(n) - 1 - p;
-    if (s >= n_in) s = n_in - 1;
+    const uint32_t s = min(n - 1 - p, n_in - 1);
     const uint32_t k = __ldg(keys + s);
     const bool is_del = (mode == kSortDelete) || (mode == kSortUpdate && __ldg(del + s) != 0);
     bad = k > kMaxUserKey;
@@ -88,167 +97,207 @@ struct Loader {
   }
 };
 
-__global__ void __launch_bounds__(kThreads) sort_histogram(Loader ld, uint32_t* __restrict__ ctl,
-                                                           uint32_t* status) {
+// 8 elements a thread at a time, so that as many loads are in flight.
+constexpr uint32_t kHistItems = 8, kHistChunk = kHistItems * kPassThreads;
+__global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32_t* __restrict__ ctl,
+                                                               uint32_t* status) {
   __shared__ uint32_t s_h[kSortPasses * kRadix];
-  for (int i = threadIdx.x; i < kSortPasses * kRadix; i += kThreads) s_h[i] = 0;
+  for (int i = threadIdx.x; i < kSortPasses * kRadix; i += kPassThreads) s_h[i] = 0;
   __syncthreads();
   bool bad_any = false;
-  for (uint32_t p = blockIdx.x * kThreads + threadIdx.x; p < ld.n; p += gridDim.x * kThreads) {
-    bool bad;
-    const uint32_t kv = ld.load_key(p, bad);
-    bad_any |= bad;
+  for (uint64_t p0 = uint64_t(blockIdx.x) * kHistChunk; p0 < ld.n; p0 += uint64_t(gridDim.x) * kHistChunk) {
+    uint32_t kv[kHistItems];
 #pragma unroll
-    for (int d = 0; d < kSortPasses; ++d) atomicAdd(&s_h[d * kRadix + ((kv >> (8 * d)) & 255u)], 1u);
+    for (uint32_t j = 0; j < kHistItems; ++j) {
+      const uint64_t p = p0 + j * kPassThreads + threadIdx.x;
+      bool bad = false;
+      kv[j] = p < ld.n ? ld.load_key(uint32_t(p), bad) : 0u;
+      bad_any |= bad;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kHistItems; ++j) {
+      if (p0 + j * kPassThreads + threadIdx.x < ld.n) {
+#pragma unroll
+        for (int d = 0; d < kSortPasses; ++d) atomicAdd(&s_h[d * kRadix + ((kv[j] >> (8 * d)) & 255u)], 1u);
+      }
+    }
   }
   const int any_bad = __syncthreads_or(bad_any);
-  for (int i = threadIdx.x; i < kSortPasses * kRadix; i += kThreads) {
+  for (int i = threadIdx.x; i < kSortPasses * kRadix; i += kPassThreads) {
     const uint32_t c = s_h[i];
     if (c) atomicAdd(ctl + i, c);
   }
   if (any_bad && threadIdx.x == 0 && status) *reinterpret_cast<volatile uint32_t*>(status) = kErrBadKey;
 }
 
+// One 8-bit pass over a tile of 8192 elements, bound by the chain of phases
+// of a tile (loads, ranks, look-back, scatter) with two tiles an SM in flight:
+// 290 us a pass at n = 5 10^7 (2.8 TB/s of reads and writes).  Tiles of 4096
+// in CTAs of 143 registers, one an SM, took 1161 us: the look-back advances by
+// at most its window (8 tiles) per round trip to L2, and one CTA an SM hides
+// nothing.  Keys are ranked and put in shared memory before the values are
+// loaded, so that 16 items a thread fit 64 registers.  Measured beside it (four
+// passes and the histogram, 5 10^7 pairs: 1170 us): tiles of 6144 at three CTAs
+// an SM 1413 us, of 10240 1258 us, windows of 4 and 12 tiles 1207 and 1242 us.
+struct PassShared {
+  union {
+    struct {
+      uint32_t keys[kSortTile], vals[kSortTile];
+    };
+    uint32_t match[kPassWarps][kRadix];  // while ranking: the lanes of the warp that hold the digit
+  };
+  uint32_t whist[kPassWarps][kRadix];
+  uint32_t gbase[kRadix];           // global position of a digit's element minus its tile position
+  uint32_t scan[kPassWarps];
+  uint32_t tile;
+};
+constexpr size_t kPassSmem = sizeof(PassShared);
+
 template <bool kFirst>
-__global__ void __launch_bounds__(kThreads, LSM_SORT_MINB) sort_pass(Loader ld, const uint32_t* __restrict__ in_k,
+__global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const uint32_t* __restrict__ in_k,
                                                       const uint32_t* __restrict__ in_v,
                                                       uint32_t* __restrict__ out_k,
                                                       uint32_t* __restrict__ out_v,
                                                       uint32_t* __restrict__ ctl, uint64_t* lookback,
                                                       int pass, uint32_t epoch, uint32_t* sticky) {
-  __shared__ __align__(16) uint32_t s_keys[kSortTile];
-  __shared__ __align__(16) uint32_t s_vals[kSortTile];
-  __shared__ uint32_t s_whist[kWarps][kRadix];
-  __shared__ uint32_t s_excl[kRadix];   // tile-local start of each digit
-  __shared__ uint32_t s_gbase[kRadix];  // global start of this tile's run of each digit
-  __shared__ uint32_t s_scan[kWarps];
-  __shared__ uint32_t s_tile;
-
+  extern __shared__ __align__(16) unsigned char pass_smem[];
+  PassShared& sh = *reinterpret_cast<PassShared*>(pass_smem);
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t n = ld.n;
   const int shift = 8 * pass;
-  if (tid == 0) s_tile = atomicAdd(ctl + kSortPasses * kRadix + pass, 1u);
-  for (uint32_t i = lane; i < kRadix; i += 32) s_whist[warp][i] = 0;
+  if (tid == 0) sh.tile = atomicAdd(ctl + kSortPasses * kRadix + pass, 1u);
+  for (uint32_t i = lane; i < kRadix; i += 32) sh.whist[warp][i] = sh.match[warp][i] = 0;
   __syncthreads();
-  const uint32_t tile = s_tile;
-  const uint32_t base = tile * kSortTile + warp * (32 * kIPT);
+  const uint32_t tile = sh.tile;
+  const uint32_t tile_start = tile * uint32_t(kSortTile);
+  const uint32_t tile_n = (n - tile_start) < uint32_t(kSortTile) ? (n - tile_start) : uint32_t(kSortTile);
+  const uint32_t e0 = warp * (32 * kIPT) + lane;  // item j: element e0 + 32 j of the tile
 
-  uint32_t kv[kIPT], v[kIPT], rank[kIPT];
+  uint32_t kv[kIPT], at[kIPT];
 #pragma unroll
   for (int j = 0; j < kIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    kv[j] = 0;
-    v[j] = 0;
-    if (p < n) {
-      if (kFirst) {
-        bool bad;
-        ld.load(p, kv[j], v[j], bad);
-      } else {
-        kv[j] = __ldg(in_k + p);
-        v[j] = __ldg(in_v + p);
-      }
-    }
+    const uint32_t e = e0 + j * 32;
+    bool bad;
+    kv[j] = 0xFFFFFFFFu;  // past the end: the last digit, after every element of it
+    if (e < tile_n) kv[j] = kFirst ? ld.load_key(tile_start + e, bad) : __ldg(in_k + tile_start + e);
   }
+  const uint32_t hist = tid < kRadix ? ctl[pass * kRadix + tid] : 0u;
 
-  // Rank within the warp, items in (j, lane) order = input order.
+  // Rank within the warp, items in (j, lane) order = input order.  The lanes
+  // with an item's digit are found by ballots for every other item and
+  // through shared memory for the rest: ballots alone kept the ALUs 66 % busy
+  // and the shared-memory pipe 44 %, atomics alone 24 % and 55 %; halves of
+  // each took 1311 us against 1368 and 1466 for 5 10^7 pairs.
   const uint32_t lt = lanemask_lt();
 #pragma unroll
   for (int j = 0; j < kIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    const uint32_t d = (p < n) ? ((kv[j] >> shift) & 255u) : kNoDigit;
-    const uint32_t peers = warp_peers<9>(d);  // d <= kNoDigit = 256
+    const uint32_t d = (kv[j] >> shift) & 255u;
+    uint32_t peers;
+    if (j & 1) {
+      atomicOr(&sh.match[warp][d], 1u << lane);
+      __syncwarp();
+      peers = sh.match[warp][d];
+    } else {
+      peers = warp_peers<8>(d);
+    }
+    const uint32_t cnt = sh.whist[warp][d];
     const uint32_t before = __popc(peers & lt);
-    const uint32_t cnt = (d != kNoDigit) ? s_whist[warp][d] : 0u;
     __syncwarp();
-    if (d != kNoDigit && before == 0) s_whist[warp][d] = cnt + __popc(peers);
+    if (before == 0) {
+      sh.whist[warp][d] = cnt + __popc(peers);
+      if (j & 1) sh.match[warp][d] = 0u;
+    }
     __syncwarp();
-    rank[j] = cnt + before;
+    at[j] = cnt + before;
   }
   __syncthreads();
 
-  // Per digit: warp prefix inside the tile and the tile total.
+  // Per digit: warp prefix inside the tile and the tile total (the padding of
+  // the last tile taken off the last digit); the tile-local and the global
+  // start of the digit.
   uint32_t total = 0;
+  if (tid < kRadix) {
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const uint32_t c = s_whist[w][tid];
-    s_whist[w][tid] = total;
-    total += c;
+    for (int w = 0; w < kPassWarps; ++w) total += sh.whist[w][tid];
+    if (tid == kRadix - 1) total -= uint32_t(kSortTile) - tile_n;
+    // the tile's count is public as early as possible
+    st_relaxed_u64(lookback + uint64_t(tile) * kRadix + tid, lb_pack(epoch, tile == 0 ? kFlagIncl : kFlagAgg, total));
   }
-  uint32_t tile_sum;
-  const uint32_t excl = block_excl_scan<kThreads>(total, s_scan, tile_sum);
-  s_excl[tid] = excl;
-  // Global start of the digit (exclusive scan of the pass histogram).
-  uint32_t hsum;
-  const uint32_t hbase = block_excl_scan<kThreads>(ctl[pass * kRadix + tid], s_scan, hsum);
-
-  // Scatter into shared memory in digit order (stable) while the look-back
-  // below is still to come: the item registers are free afterwards.
+  uint32_t sum;
+  const uint32_t excl = block_excl_scan<kPassThreads>(total, sh.scan, sum);
+  const uint32_t hbase = block_excl_scan<kPassThreads>(hist, sh.scan, sum);
+  if (tid < kRadix) {
+    uint32_t run = excl;  // each warp's start in the tile
+#pragma unroll
+    for (int w = 0; w < kPassWarps; ++w) {
+      const uint32_t c = sh.whist[w][tid];
+      sh.whist[w][tid] = run;
+      run += c;
+    }
+  }
   __syncthreads();
+
+  // Into shared memory in digit order (stable), values last.
 #pragma unroll
   for (int j = 0; j < kIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    if (p < n) {
-      const uint32_t d = (kv[j] >> shift) & 255u;
-      const uint32_t pos = s_excl[d] + s_whist[warp][d] + rank[j];
-      s_keys[pos] = kv[j];
-      s_vals[pos] = v[j];
-    }
+    const uint32_t d = (kv[j] >> shift) & 255u;
+    at[j] += sh.whist[warp][d];
+    sh.keys[at[j]] = kv[j];
   }
+#pragma unroll
+  for (int j = 0; j < kIPT; ++j) {
+    const uint32_t e = e0 + j * 32;
+    if (e < tile_n) kv[j] = kFirst ? ld.load_val(tile_start + e, kv[j]) : __ldg(in_v + tile_start + e);
+  }
+#pragma unroll
+  for (int j = 0; j < kIPT; ++j) sh.vals[at[j]] = kv[j];
 
-  // Decoupled look-back over the tiles before this one, one digit per
-  // thread, reading kLookbackWindow predecessors per step: the words are
-  // consumed from the nearest tile down until an inclusive prefix is found;
-  // a word not yet published stops the step, which is then retried from
-  // there (bounded in time).
-  uint64_t* my = lookback + uint64_t(tile) * kRadix + tid;
-  uint32_t prefix = 0;
-  if (tile == 0) {
-    st_relaxed_u64(my, lb_pack(epoch, kFlagIncl, total));
-  } else {
-    st_relaxed_u64(my, lb_pack(epoch, kFlagAgg, total));
-    int64_t t = int64_t(tile) - 1;
-    uint64_t t0 = 0;
-    bool done = false;
-    while (!done) {
-      uint64_t w[kLookbackWindow];
+  // Decoupled look-back, one thread per digit, kLookbackWords predecessors
+  // per step: the words are consumed from the nearest tile down until an
+  // inclusive prefix is found; a word not yet published ends the step, which
+  // is then retried from there (bounded in time).
+  if (tid < kRadix) {
+    uint32_t prefix = 0;
+    if (tile) {
+      const uint32_t tag_agg = (epoch << 2) | uint32_t(kFlagAgg), tag_incl = (epoch << 2) | uint32_t(kFlagIncl);
+      int64_t t = int64_t(tile) - 1;  // nearest predecessor not yet consumed
+      uint64_t t0 = 0;
+      for (bool incl = false; !incl;) {
+        uint64_t w[kLookbackWords];
 #pragma unroll
-      for (int i = 0; i < kLookbackWindow; ++i)
-        w[i] = (t - i >= 0) ? ld_relaxed_u64(lookback + uint64_t(t - i) * kRadix + tid) : 0ull;
-      int consumed = 0;
-      bool stall = false;
+        for (int i = 0; i < kLookbackWords; ++i)
+          w[i] = t - i >= 0 ? ld_relaxed_u64(lookback + uint64_t(t - i) * kRadix + tid)
+                            : lb_pack(epoch, kFlagIncl, 0u);
+        int consumed = 0;
+        bool stall = false;
 #pragma unroll
-      for (int i = 0; i < kLookbackWindow; ++i) {
-        if (done || stall) continue;
-        if (t - i < 0) {  // ran past tile 0: the prefix is complete
-          done = true;
-          continue;
+        for (int i = 0; i < kLookbackWords; ++i) {
+          const uint32_t tag = uint32_t(w[i] >> 32);
+          if (!incl && !stall) {
+            incl = tag == tag_incl;
+            stall = !incl && tag != tag_agg;
+            if (!stall) {
+              prefix += uint32_t(w[i]);
+              ++consumed;
+            }
+          }
         }
-        const uint64_t flag = (w[i] >> 32) & 3u;
-        if (uint32_t(w[i] >> 34) != epoch || flag == 0) {
-          stall = true;
-          continue;
-        }
-        prefix += uint32_t(w[i]);
-        ++consumed;
-        if (flag == kFlagIncl) done = true;
+        t -= consumed;
+        if (!incl && consumed == 0 && !spin_continue(t0, kWaitLimitNs, sticky)) break;
+        if (consumed) t0 = 0;
       }
-      t -= consumed;
-      if (!done && consumed == 0 && !spin_continue(t0, kWaitLimitNs, sticky)) break;
+      st_relaxed_u64(lookback + uint64_t(tile) * kRadix + tid, lb_pack(epoch, kFlagIncl, prefix + total));
     }
-    st_relaxed_u64(my, lb_pack(epoch, kFlagIncl, prefix + total));
+    sh.gbase[tid] = hbase - excl + prefix;
   }
-  s_gbase[tid] = hbase + prefix;
   __syncthreads();
 
-  const uint32_t tile_start = tile * kSortTile;
-  const uint32_t tile_n = (n - tile_start) < uint32_t(kSortTile) ? (n - tile_start) : uint32_t(kSortTile);
-  for (uint32_t i = tid; i < tile_n; i += kThreads) {
-    const uint32_t k = s_keys[i];
-    const uint32_t d = (k >> shift) & 255u;
-    const uint32_t dst = s_gbase[d] + (i - s_excl[d]);
+  for (uint32_t i = tid; i < tile_n; i += kPassThreads) {
+    const uint32_t k = sh.keys[i];
+    const uint32_t dst = sh.gbase[(k >> shift) & 255u] + i;
     if (dst < n) {
       out_k[dst] = k;
-      out_v[dst] = s_vals[i];
+      out_v[dst] = sh.vals[i];
     }
   }
 }
@@ -1298,7 +1347,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) 
 }  // namespace
 
 constexpr size_t kBucketSmem = 4 * size_t(kBucketCap) * sizeof(uint32_t) + size_t(kBucketCap) * sizeof(uint16_t);
-PerDeviceFlags g_bucket_attr;
+PerDeviceFlags g_bucket_attr, g_pass_attr[2];
 
 cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status,
                                cudaEvent_t ev) {
@@ -1310,7 +1359,7 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   uint2* runs = reinterpret_cast<uint2*>(ws.tilecnt);
   uint32_t* ctl = ws.ctl + ws.flip * kSortCtlWords;
   uint32_t* next = ws.ctl + (ws.flip ^ 1) * kSortCtlWords;
-  Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, a.n_in, a.n};
+  Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, uint32_t(a.n_in), a.n};
   // a deferred check leaves its verdict in the sort's own control block
   uint32_t* check = a.defer_err ? ctl + kSortCtlStatus : status;
   count_launches(1);
@@ -1335,6 +1384,10 @@ cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, u
   const uint32_t ntiles = (a.n + kSortTile - 1) / kSortTile;
   if (ntiles > ws.max_tiles) return cudaErrorInvalidValue;
   cudaError_t e;
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = set_smem_attr_once(sort_pass<true>, kPassSmem, dev, g_pass_attr[0])) != cudaSuccess) return e;
+  if ((e = set_smem_attr_once(sort_pass<false>, kPassSmem, dev, g_pass_attr[1])) != cudaSuccess) return e;
   if (++ws.epoch >= (1u << 30)) {
     ws.epoch = 1;
     e = cudaMemsetAsync(ws.lookback, 0, sizeof(uint64_t) * kSortPasses * ws.max_tiles * kRadix, st);
@@ -1343,11 +1396,11 @@ cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, u
   uint32_t* ctl = ws.ctl + ws.flip * kSortCtlWords;
   e = cudaMemsetAsync(ctl, 0, sizeof(uint32_t) * kSortCtlWords, st);
   if (e != cudaSuccess) return e;
-  Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, a.n_in, a.n};
-  uint32_t hblocks = (a.n + 255) / 256;
+  Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, uint32_t(a.n_in), a.n};
+  uint32_t hblocks = (a.n + kHistChunk - 1) / kHistChunk;
   if (hblocks > 4 * 152) hblocks = 4 * 152;
   count_launches(1);
-  sort_histogram<<<hblocks, 256, 0, st>>>(ld, ctl, status);
+  sort_histogram<<<hblocks, kPassThreads, 0, st>>>(ld, ctl, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (status && (e = cudaEventRecord(ev, st)) != cudaSuccess) return e;
   // in -> tmp -> out -> tmp -> out
@@ -1355,12 +1408,12 @@ cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, u
   uint32_t* bv[2] = {a.tmp_vals, a.out_vals};
   const size_t lb_stride = size_t(ws.max_tiles) * kRadix;
   count_launches(1);
-  sort_pass<true><<<ntiles, kThreads, 0, st>>>(ld, nullptr, nullptr, bk[0], bv[0], ctl, ws.lookback,
+  sort_pass<true><<<ntiles, kPassThreads, kPassSmem, st>>>(ld, nullptr, nullptr, bk[0], bv[0], ctl, ws.lookback,
                                                 0, ws.epoch, ws.sticky);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (int p = 1; p < kSortPasses; ++p) {
     count_launches(1);
-    sort_pass<false><<<ntiles, kThreads, 0, st>>>(ld, bk[(p - 1) & 1], bv[(p - 1) & 1], bk[p & 1],
+    sort_pass<false><<<ntiles, kPassThreads, kPassSmem, st>>>(ld, bk[(p - 1) & 1], bv[(p - 1) & 1], bk[p & 1],
                                                    bv[p & 1], ctl, ws.lookback + p * lb_stride, p,
                                                    ws.epoch, ws.sticky);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -105,3 +105,10 @@ def test_levels_over_ranges(g, dist, short):
     np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), o1.count(k1, k2))
     assert lsm.device_errors() == 0
     lsm.close()
+
+
+@pytest.mark.parametrize("n", [(1 << 20) + 1, 129 * 8192 - 1, 129 * 8192, 2500001])
+@pytest.mark.parametrize("dist", ["one", "ids", "hot", "zipf"])
+def test_long_sort_over_ranges(g, dist, n):
+    """Above 2^20 elements: the four 8-bit passes, at the edges of their 8192-element tiles."""
+    test_sort_over_ranges(g, dist, n)
