@@ -126,14 +126,18 @@ constexpr int kSortCtlStatus = kSortPasses * 256 + kSortPasses;
 // its buckets' lower bounds in the first pass's histogram, which it does not
 // use.
 constexpr int kSortCtlMap = kSortCtlStatus + 1;
+constexpr int kSortCtlChecked = kSortCtlMap + 2;  // CTAs whose keys have been checked
+static_assert(kSortCtlChecked < kSortCtlWords, "control words");
 constexpr int kSortCtlBounds = 0;
 
-// Enqueues the whole sort.  If `status` is given (a device-visible word,
-// typically mapped pinned host memory), the first kernel stores kErrBadKey
-// there when a key is out of range, and `ev` is recorded right after that
-// kernel, so the host can learn about bad keys before the sort ends.
-cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st,
-                        uint32_t* status, cudaEvent_t ev);
+// Enqueues the whole sort.  If `status` is given (a device-visible word of
+// mapped pinned host memory), the first kernel's last CTA stores there
+// check_word(seq, whether a key is out of range), so the host can learn about
+// bad keys before the sort ends; no event stands between the sort's kernels
+// for it (it would end their launch overlap).
+__host__ __device__ constexpr uint32_t check_word(uint32_t seq, bool bad) { return (seq << 1) | (bad ? 1u : 0u); }
+cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status = nullptr,
+                        uint32_t seq = 0);
 
 // Device key check alone over n keys (multi-batch calls check all first).
 cudaError_t check_keys_launch(const uint32_t* keys, uint64_t n, uint32_t* status,

@@ -518,7 +518,7 @@ struct Run {
     a.tmp_keys = set[2];
     a.tmp_vals = set[3];
     sl.sws.sticky = dict_status_word(s->dict);
-    err = cuda_status(sort_launch(a, sl.sws, rs, nullptr, nullptr));
+    err = cuda_status(sort_launch(a, sl.sws, rs));
     return err == LSM_OK;
   }
 

@@ -97,10 +97,29 @@ struct Loader {
   }
 };
 
+// End of the key check of a sort's first kernel: called by one thread of every
+// CTA with whether the CTA saw a key out of range.  The verdict goes to the
+// control block; with `host`, the last CTA to get here stores it there too.
+struct KeyCheck {
+  uint32_t* host;   // null: a deferred check, or none
+  uint32_t seq;
+  bool on;
+  __device__ __forceinline__ void done(uint32_t* ctl, bool bad) const {
+    if (!on) return;
+    if (bad) {
+      atomicOr(ctl + kSortCtlStatus, kErrBadKey);
+      __threadfence();
+    }
+    if (!host || atomicAdd(ctl + kSortCtlChecked, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    const uint32_t any = atomicOr(ctl + kSortCtlStatus, 0u);
+    *reinterpret_cast<volatile uint32_t*>(host) = check_word(seq, any != 0u);
+  }
+};
+
 // 8 elements a thread at a time, so that as many loads are in flight.
 constexpr uint32_t kHistItems = 8, kHistChunk = kHistItems * kPassThreads;
-__global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32_t* __restrict__ ctl,
-                                                               uint32_t* status) {
+__global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32_t* ctl, KeyCheck check) {
   __shared__ uint32_t s_h[kSortPasses * kRadix];
   for (int i = threadIdx.x; i < kSortPasses * kRadix; i += kPassThreads) s_h[i] = 0;
   __syncthreads();
@@ -127,7 +146,7 @@ __global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32
     const uint32_t c = s_h[i];
     if (c) atomicAdd(ctl + i, c);
   }
-  if (any_bad && threadIdx.x == 0 && status) *reinterpret_cast<volatile uint32_t*>(status) = kErrBadKey;
+  if (threadIdx.x == 0) check.done(ctl, any_bad != 0);
 }
 
 // One 8-bit pass over a tile of 8192 elements, bound by the chain of phases
@@ -437,7 +456,7 @@ __device__ __forceinline__ void rank_block(const uint32_t (&kv)[IPT], uint32_t m
 // writes its (empty) runs.
 __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t* __restrict__ tmp_k,
                                                      uint32_t* __restrict__ tmp_v, uint2* __restrict__ runs,
-                                                     uint32_t* __restrict__ ctl, uint32_t* status) {
+                                                     uint32_t* ctl, KeyCheck check) {
   __shared__ __align__(16) uint32_t s_keys[kMsdTile];
   __shared__ __align__(16) uint32_t s_vals[kMsdTile];
   __shared__ uint32_t s_whist[kScatterWarps][kRadix];
@@ -461,6 +480,8 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
       bad_any |= bad;
     }
   }
+  const int any_bad = __syncthreads_or(bad_any);
+  if (tid == 0) check.done(ctl, any_bad != 0);
   const KeyMap map = sample_map<kScatterThreads>(ld, s_cnt, s_cnt + kScatterWarps);
   if (tile == gridDim.x - 1) {  // the last tile's CTA (the shortest) publishes the map and the buckets' bounds
     if (tid < kRadix) ctl[kSortCtlBounds + tid] = tid ? map.lower(tid) : 0u;
@@ -481,7 +502,7 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
       s_vals[pos] = v[j];
     }
   }
-  const int any_bad = __syncthreads_or(bad_any);  // also orders the writes above before the reads below
+  __syncthreads();
   const uint32_t lo_t = t0 > npad ? t0 : npad, hi_t = (n - t0) < kMsdTile ? n : t0 + kMsdTile;
   const uint32_t tile_n = hi_t > lo_t ? hi_t - lo_t : 0u;  // real elements of the tile
   for (uint32_t i = tid; i < tile_n; i += kScatterThreads) {
@@ -497,7 +518,6 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
     bool bad;
     atomicAdd(ctl + 3 * kRadix + map.bucket(ld.load_key(0, bad)), npad);
   }
-  if (any_bad && tid == 0 && status) *reinterpret_cast<volatile uint32_t*>(status) = kErrBadKey;
 }
 
 // First position i in [0, m) with a[i] >= kv, a sorted.
@@ -1350,7 +1370,7 @@ constexpr size_t kBucketSmem = 4 * size_t(kBucketCap) * sizeof(uint32_t) + size_
 PerDeviceFlags g_bucket_attr, g_pass_attr[2];
 
 cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status,
-                               cudaEvent_t ev) {
+                               uint32_t seq) {
   cudaError_t e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1361,12 +1381,11 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   uint32_t* next = ws.ctl + (ws.flip ^ 1) * kSortCtlWords;
   Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, uint32_t(a.n_in), a.n};
   // a deferred check leaves its verdict in the sort's own control block
-  uint32_t* check = a.defer_err ? ctl + kSortCtlStatus : status;
+  const KeyCheck check{a.defer_err ? nullptr : status, seq, a.defer_err || status};
   count_launches(1);
   if ((e = launch_pdl(msd_tile, dim3(ntiles), dim3(kScatterThreads), 0, st, ld, a.tmp_keys, a.tmp_vals, runs, ctl,
                       check)) != cudaSuccess)
     return e;
-  if (status && !a.defer_err && (e = cudaEventRecord(ev, st)) != cudaSuccess) return e;
   count_launches(1);
   if ((e = launch_pdl(bucket_sort, dim3(kRadix), dim3(kBucketThreads), kBucketSmem, st, ld,
                       static_cast<const uint32_t*>(a.tmp_keys), static_cast<const uint32_t*>(a.tmp_vals),
@@ -1377,10 +1396,9 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   return cudaSuccess;
 }
 
-cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status,
-                        cudaEvent_t ev) {
+cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status, uint32_t seq) {
   if (a.n == 0) return cudaSuccess;
-  if (a.n <= kMsdMaxN && ws.tilecnt) return bucket_sort_launch(a, ws, st, status, ev);
+  if (a.n <= kMsdMaxN && ws.tilecnt) return bucket_sort_launch(a, ws, st, status, seq);
   const uint32_t ntiles = (a.n + kSortTile - 1) / kSortTile;
   if (ntiles > ws.max_tiles) return cudaErrorInvalidValue;
   cudaError_t e;
@@ -1400,9 +1418,8 @@ cudaError_t sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, u
   uint32_t hblocks = (a.n + kHistChunk - 1) / kHistChunk;
   if (hblocks > 4 * 152) hblocks = 4 * 152;
   count_launches(1);
-  sort_histogram<<<hblocks, kPassThreads, 0, st>>>(ld, ctl, status);
+  sort_histogram<<<hblocks, kPassThreads, 0, st>>>(ld, ctl, KeyCheck{status, seq, status != nullptr});
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (status && (e = cudaEventRecord(ev, st)) != cudaSuccess) return e;
   // in -> tmp -> out -> tmp -> out
   uint32_t* bk[2] = {a.tmp_keys, a.out_keys};
   uint32_t* bv[2] = {a.tmp_vals, a.out_vals};
@@ -1561,7 +1578,7 @@ extern "C" lsm_status lsm_sort_pairs_noalloc(const uint32_t* d_keys_in, const ui
   // Each sort leaves the control block of the next one zeroed; the run table
   // and the tile scratch are fully rewritten by every call before they are
   // read, so nothing else needs zeroing.
-  cudaError_t e = sort_launch(a, d.ws, st, nullptr, nullptr);
+  cudaError_t e = sort_launch(a, d.ws, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return LSM_ERR_CUDA;

@@ -112,3 +112,27 @@ def test_levels_over_ranges(g, dist, short):
 def test_long_sort_over_ranges(g, dist, n):
     """Above 2^20 elements: the four 8-bit passes, at the edges of their 8192-element tiles."""
     test_sort_over_ranges(g, dist, n)
+
+
+@pytest.mark.parametrize("b", [64, 5000, (1 << 20) + 5])
+def test_refused_batches_between_folds(g, b):
+    """A batch with a key out of range is refused at every counter value: its fold may have been enqueued, and must
+    leave the levels, the batch kept as level 0 and the later batches alone."""
+    rng = np.random.default_rng(b)
+    lsm, s = g.LSM(b, 16 * b), oracle.StructuralOracle(b)
+    for t in range(9):
+        for _ in range(1 + t % 3):
+            bad = rng.integers(0, TOP, b).astype(np.uint32)
+            bad[rng.integers(0, b)] = TOP + int(rng.integers(0, 3))
+            with pytest.raises(g.LSMError) as e:
+                lsm.insert(bad, np.zeros(b, np.uint32))
+            assert e.value.status == g.LSM_ERR_KEY_RANGE
+            assert lsm.r == s.r == t
+        k, v = rng.integers(0, TOP, b).astype(np.uint32), rng.integers(0, 1 << 31, b).astype(np.uint32)
+        lsm.insert(k, v)
+        s.call("insert", k, v)
+    for i, (kv, vv) in lsm.levels().items():
+        ekv, ev = s.level(i)
+        np.testing.assert_array_equal(kv, ekv)
+        np.testing.assert_array_equal(vv, ev)
+    lsm.close()
