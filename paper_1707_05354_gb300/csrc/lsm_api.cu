@@ -717,7 +717,7 @@ lsm_status lsm_range(lsm_t* h, const uint32_t* d_k1, const uint32_t* d_k2, uint6
   if (total > capacity) return LSM_ERR_CAPACITY;
   if (total && (!d_keys || !d_vals)) return LSM_ERR_ARG;
   ProfScope ps(h, LSM_PROF_EMIT, 8.0 * double(total) + 8.0 * double(nq), st);
-  return cuda_status(range_emit_launch(ls, nq, bounds, d_offsets, d_keys, d_vals, st, nullptr, d_k1, d_k2, wide));
+  return cuda_status(range_emit_launch(ls, nq, bounds, d_offsets, d_keys, d_vals, st, nullptr, wide));
 }
 
 // Rebuild of the levels from sorted sources (rank order: newest first): the

@@ -370,10 +370,9 @@ inline uint64_t scan_tiles(uint64_t n) { return (n + 2047) / 2048; }
 // Range output from the windows of count_launch; with `perm`, thread i
 // serves query perm[i] (neighbouring threads, neighbouring windows).
 // With `wide` (the list count_launch left), the wide queries are emitted by
-// a warp each, from their bounds k1 / k2.
+// a warp each.
 cudaError_t range_emit_launch(const LevelSet& ls, uint64_t nq, const uint32_t* bounds,
                               const uint64_t* offsets, uint32_t* keys, uint32_t* vals,
-                              cudaStream_t st, const uint32_t* perm = nullptr, const uint32_t* k1 = nullptr,
-                              const uint32_t* k2 = nullptr, const uint32_t* wide = nullptr);
+                              cudaStream_t st, const uint32_t* perm = nullptr, const uint32_t* wide = nullptr);
 
 }  // namespace gpulsm

@@ -324,69 +324,213 @@ __global__ void __launch_bounds__(kThreads) range_emit(LevelSet ls, uint64_t nq,
   }
 }
 
-// Wide queries, one warp each: the key interval [k1, k2] is cut into 32
-// equal key sub-intervals, one per lane; every lane takes its windows in
-// each level and merges them as the one-thread path does (all versions of
-// a key fall in one lane's sub-interval, so the lanes' results are
-// disjoint).  The count is the warp's sum; the range output of a lane goes
-// after the lanes before it (a warp scan of their counts).
-template <int L>
-__device__ __forceinline__ uint32_t lane_windows(const LevelSet& ls, uint32_t a, uint32_t z, uint32_t (&lo)[L],
-                                                 uint32_t (&hi)[L]) {
-  const uint64_t w = (uint64_t(z) - a + 32) / 32;  // ceil((z - a + 1) / 32)
-  const uint64_t s0 = uint64_t(a) + lane_id() * w;
-  const uint64_t s1 = s0 + w - 1 < z ? s0 + w - 1 : uint64_t(z);
-  const bool empty = s0 > z;
-#pragma unroll
-  for (int l = 0; l < L; ++l) {
-    lo[l] = hi[l] = 0;
-    if (l < ls.count && !empty) level_window(ls, l, uint32_t(s0) << 1, (uint32_t(s1) + 1u) << 1, lo[l], hi[l]);
+// Wide queries, one warp each.  The warp stages the windows of all levels,
+// newest level first, in shared memory (coalesced reads, all in flight).
+// Every element then looks for its key in the windows of the older levels:
+// levels double, so that these searches are few (each element once per older
+// level: about as many as elements in all), while looking from the old
+// levels, which hold most elements, into the newer ones takes some four times
+// as many.  An element found has a newer version and loses its status bit; what
+// is still regular, and the first of its key in its level, is live.  For the
+// output order the same searches give every element's place in the merged
+// order: c elements of the older level come before the one that searches, and
+// that one comes before the older level's elements from c on (a histogram of
+// c, summed up).  The places of the live elements are marked in a bitmap
+// whose prefix counts give the output positions.
+// Windows above kWideCap elements in all are taken in pieces: the keys below
+// the smallest of the levels' (kWideCap / levels)-th keys, which at most
+// kWideCap elements have; a key that fills a level's share alone is decided by
+// itself.
+// (2 10^5 queries of about 107 elements in six levels, count_wide + range_wide:
+// one lane per 1/32 of the key interval, merging its own windows step by step,
+// 618 + 1151 us; searches into the newer levels 499 + 748; this 258 +
+// 365 us.  Bound by its instructions.)
+constexpr uint32_t kWideCap = 512, kPlaceBits = 9;
+static_assert(kWideCap == 1u << kPlaceBits && kMaxLevels <= 64, "a place and its level fit 16 bits");
+struct WideCount {
+  uint32_t kv[kWideCap];
+};
+struct WideEmit {
+  uint32_t kv[kWideCap], hist[kWideCap];
+  uint16_t place[kWideCap];
+  uint32_t bits[kWideCap / 32], before[kWideCap / 32];
+};
+
+// First of the n elements of the sorted run a whose key variable is >= x.
+__device__ __forceinline__ uint32_t lower_bound_smem(const uint32_t* a, uint32_t n, uint32_t x) {
+  uint32_t lo = 0;
+  while (n) {
+    const uint32_t h = n >> 1;
+    const bool less = a[lo + h] < x;
+    lo = less ? lo + h + 1 : lo;
+    n = less ? n - h - 1 : h;
   }
-  return empty ? 0u : merge_windows<false, L>(ls, lo, hi, nullptr, nullptr, 0);
+  return lo;
 }
 
-template <int L>
+// Live keys of the windows [pos, end) (lane l holds level l's), emitted to
+// out_k/out_v in key order when kEmit (at most `room`); returns their number.
+template <class Shared>
+__device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos, uint32_t end, Shared& sh,
+                                               uint32_t* out_k, uint32_t* out_v, uint64_t room) {
+  constexpr bool kEmit = sizeof(Shared) == sizeof(WideEmit);
+  const uint32_t lane = lane_id();
+  const int nl = ls.count;
+  const bool act = lane < uint32_t(nl);
+  const uint32_t* keys = act ? ls.keys[lane] : nullptr;
+  uint32_t done = 0;
+  for (;;) {
+    const uint32_t left = act ? end - pos : 0u;
+    const uint32_t total = warp_sum(left);
+    if (total == 0) return done;
+    // this piece: [pos, pos + n) of every level
+    uint32_t n = left;
+    if (total > kWideCap) {
+      const uint32_t share = kWideCap / uint32_t(nl);
+      const uint32_t lim = __reduce_min_sync(0xffffffffu, left > share ? key_of(__ldg(keys + pos + share)) : 0xFFFFFFFFu);
+      n = left ? lower_bound_kv(keys, pos, pos + min(left, share), lim << 1) - pos : 0u;
+      if (!__any_sync(0xffffffffu, n != 0u)) {
+        // every next element has a key >= lim, and one level starts with more
+        // than its share of copies of it
+        const uint32_t first = left ? __ldg(keys + pos) : 0xFFFFFFFFu;
+        const uint32_t has = __ballot_sync(0xffffffffu, left && key_of(first) == lim);
+        const int newest = __ffs(int(has)) - 1;
+        const bool live = (__shfl_sync(0xffffffffu, first, newest) & 1u) != 0u;
+        if (live) {
+          if (kEmit && int(lane) == newest && done < room) {
+            out_k[done] = lim;
+            out_v[done] = __ldg(ls.vals[lane] + pos);
+          }
+          ++done;
+        }
+        if (left && key_of(first) == lim) pos = upper_bound_key(keys, pos, end, lim);
+        continue;
+      }
+    }
+    const uint32_t off = warp_incl_scan(n) - n;
+    __syncwarp();
+    for (int l = 0; l < nl; ++l) {
+      const uint32_t m = __shfl_sync(0xffffffffu, n, l), o = __shfl_sync(0xffffffffu, off, l),
+                     p = __shfl_sync(0xffffffffu, pos, l);
+      const uint32_t* from = ls.keys[l] + p;
+      for (uint32_t i = lane; i < m; i += 32) {
+        cp_async4(sh.kv + o + i, from + i);
+        if constexpr (kEmit) {
+          sh.hist[o + i] = 0u;
+          sh.place[o + i] = uint16_t(l << kPlaceBits);
+        }
+      }
+    }
+    const uint32_t all = warp_sum(n);
+    if constexpr (kEmit) {
+      if (lane < kWideCap / 32) sh.bits[lane] = 0u;
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    for (int l = 1; l < nl; ++l) {  // the elements of the newer levels, [0, o), look into level l
+      const uint32_t m = __shfl_sync(0xffffffffu, n, l), o = __shfl_sync(0xffffffffu, off, l);
+      if (m == 0) continue;
+      for (uint32_t t = lane; t < o; t += 32) {
+        const uint32_t x = sh.kv[t] & ~1u, c = lower_bound_smem(sh.kv + o, m, x);
+        if (c < m) {
+          if ((sh.kv[o + c] & ~1u) == x) sh.kv[o + c] = x;  // (the key and the order stay)
+          if constexpr (kEmit) atomicAdd(&sh.hist[o + c], 1u);
+        }
+        if constexpr (kEmit) sh.place[t] += uint16_t(c);     // this lane's alone; the sum is below kWideCap
+      }
+    }
+    __syncwarp();
+    uint32_t live = 0;
+    if constexpr (!kEmit) {
+      // (at a level's start the element before is a newer level's: one with
+      // the same key has taken the status bit)
+      for (uint32_t t = lane; t < all; t += 32)
+        live += (sh.kv[t] & 1u) && (t == 0 || key_of(sh.kv[t - 1]) != key_of(sh.kv[t])) ? 1u : 0u;
+      live = warp_sum(live);
+    } else {
+      uint32_t sum = 0;
+      for (uint32_t t0 = 0; t0 < all; t0 += 32) {  // running sums of the histogram, over all levels
+        const uint32_t t = t0 + lane;
+        const uint32_t h = sum + warp_incl_scan(t < all ? sh.hist[t] : 0u);
+        if (t < all) sh.hist[t] = h;
+        sum = __shfl_sync(0xffffffffu, h, 31);
+      }
+      __syncwarp();
+      for (uint32_t t0 = 0; t0 < all; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        const uint32_t own = t < all ? sh.place[t] : 0u, l = own >> kPlaceBits;
+        const uint32_t o = __shfl_sync(0xffffffffu, off, int(l));  // the level's first element here
+        if (t < all) {
+          const bool ok = (sh.kv[t] & 1u) && (t == 0 || key_of(sh.kv[t - 1]) != key_of(sh.kv[t]));
+          const uint32_t place = t - o + (own & (kWideCap - 1)) + sh.hist[t] - (o ? sh.hist[o - 1] : 0u);
+          sh.place[t] = ok ? uint16_t((l << kPlaceBits) | place) : uint16_t(0xFFFFu);
+          if (ok) atomicOr(&sh.bits[place >> 5], 1u << (place & 31u));
+        }
+      }
+      __syncwarp();
+      const uint32_t b = lane < kWideCap / 32 ? uint32_t(__popc(sh.bits[lane])) : 0u;
+      const uint32_t incl = warp_incl_scan(b);
+      if (lane < kWideCap / 32) sh.before[lane] = incl - b;
+      live = __shfl_sync(0xffffffffu, incl, 31);
+      __syncwarp();
+      for (uint32_t t0 = 0; t0 < all; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        const uint32_t own = t < all ? sh.place[t] : 0xFFFFu, l = own == 0xFFFFu ? 0u : own >> kPlaceBits;
+        const uint32_t from = __shfl_sync(0xffffffffu, pos - off, int(l));  // (may wrap)
+        if (own == 0xFFFFu) continue;
+        const uint32_t place = own & (kWideCap - 1), w = place >> 5;
+        const uint32_t at = done + sh.before[w] + __popc(sh.bits[w] & ((1u << (place & 31u)) - 1u));
+        if (at < room) {
+          out_k[at] = key_of(sh.kv[t]);
+          out_v[at] = __ldg(ls.vals[l] + (from + t));
+        }
+      }
+    }
+    done += live;
+    pos += n;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) count_wide(LevelSet ls, const uint32_t* __restrict__ k1,
                                                        const uint32_t* __restrict__ k2, uint64_t nq,
                                                        uint32_t* __restrict__ out_count,
                                                        const uint32_t* __restrict__ perm,
                                                        const uint32_t* __restrict__ wide) {
+  __shared__ WideCount s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
   const uint32_t lane = lane_id();
   for (uint32_t w = (blockIdx.x * kThreads + threadIdx.x) >> 5; w < nw; w += (gridDim.x * kThreads) >> 5) {
     const uint32_t i0 = wide[1 + w];
     const uint64_t i = perm ? __ldg(perm + i0) : i0;
     if (i >= nq) continue;  // whole warp
-    const uint32_t a = __ldg(k1 + i0);
-    uint32_t z = __ldg(k2 + i);
-    if (z > kMaxUserKey) z = kMaxUserKey;
-    uint32_t lo[L], hi[L];
-    const uint32_t c = warp_sum(lane_windows<L>(ls, a, z, lo, hi));
+    const uint32_t a = __ldg(k1 + i0), z = min(__ldg(k2 + i), kMaxUserKey);
+    uint32_t lo = 0, hi = 0;
+    if (lane < uint32_t(ls.count) && a <= z) level_window(ls, int(lane), a << 1, (z + 1u) << 1, lo, hi);
+    const uint32_t c = wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], nullptr, nullptr, 0);
     if (lane == 0) out_count[i] = c;
   }
 }
 
-template <int L>
-__global__ void __launch_bounds__(kThreads) range_wide(LevelSet ls, const uint32_t* __restrict__ k1,
-                                                       const uint32_t* __restrict__ k2, uint64_t nq,
+// The windows are those that the count pass stored.
+__global__ void __launch_bounds__(kThreads) range_wide(LevelSet ls, uint64_t nq, const uint32_t* __restrict__ bounds,
                                                        const uint64_t* __restrict__ offsets,
                                                        uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                        const uint32_t* __restrict__ perm,
                                                        const uint32_t* __restrict__ wide) {
+  __shared__ WideEmit s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
+  const uint32_t lane = lane_id();
   for (uint32_t w = (blockIdx.x * kThreads + threadIdx.x) >> 5; w < nw; w += (gridDim.x * kThreads) >> 5) {
     const uint32_t i0 = wide[1 + w];
     const uint64_t i = perm ? __ldg(perm + i0) : i0;
     if (i >= nq) continue;  // whole warp
-    const uint32_t a = __ldg(k1 + i0);
-    uint32_t z = __ldg(k2 + i);
-    if (z > kMaxUserKey) z = kMaxUserKey;
-    uint32_t lo[L], hi[L];
-    const uint32_t c = lane_windows<L>(ls, a, z, lo, hi);
-    const uint32_t before = warp_incl_scan(c) - c;
-    const uint64_t o = offsets[i], room = offsets[i + 1] - o;
-    if (c && before < room)
-      merge_windows<true, L>(ls, lo, hi, keys + o + before, vals + o + before, room - before);
+    uint32_t lo = 0, hi = 0;
+    if (lane < uint32_t(ls.count)) {
+      lo = __ldg(bounds + (i * ls.count + lane) * 2);
+      hi = __ldg(bounds + (i * ls.count + lane) * 2 + 1);
+    }
+    const uint64_t o = offsets[i];
+    wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], keys + o, vals + o, offsets[i + 1] - o);
   }
 }
 
@@ -620,12 +764,7 @@ cudaError_t count_launch(const LevelSet& ls, const uint32_t* k1, const uint32_t*
   // all are wide; an empty list ends at once)
   const unsigned wgrid = persistent_grid(nq * 32, kThreads, 152 * 8);
   count_launches(1);
-  if (ls.count <= 1) count_wide<1><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
-  else if (ls.count <= 2) count_wide<2><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
-  else if (ls.count <= 4) count_wide<4><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
-  else if (ls.count <= 8) count_wide<8><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
-  else if (ls.count <= 16) count_wide<16><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
-  else count_wide<kMaxLevels><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
+  count_wide<<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
   return cudaGetLastError();
 }
 
@@ -643,7 +782,7 @@ cudaError_t scan_launch(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t*
 
 cudaError_t range_emit_launch(const LevelSet& ls, uint64_t nq, const uint32_t* bounds, const uint64_t* offsets,
                               uint32_t* keys, uint32_t* vals, cudaStream_t st, const uint32_t* perm,
-                              const uint32_t* k1, const uint32_t* k2, const uint32_t* wide) {
+                              const uint32_t* wide) {
   if (nq == 0) return cudaSuccess;
   cudaError_t e;
   const bool w = wide != nullptr;
@@ -658,12 +797,7 @@ cudaError_t range_emit_launch(const LevelSet& ls, uint64_t nq, const uint32_t* b
   if ((e = cudaGetLastError()) != cudaSuccess || !w) return e;
   const unsigned wgrid = persistent_grid(nq * 32, kThreads, 152 * 8);
   count_launches(1);
-  if (ls.count <= 1) range_wide<1><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
-  else if (ls.count <= 2) range_wide<2><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
-  else if (ls.count <= 4) range_wide<4><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
-  else if (ls.count <= 8) range_wide<8><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
-  else if (ls.count <= 16) range_wide<16><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
-  else range_wide<kMaxLevels><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, offsets, keys, vals, perm, wide);
+  range_wide<<<wgrid, kThreads, 0, st>>>(ls, nq, bounds, offsets, keys, vals, perm, wide);
   return cudaGetLastError();
 }
 
