@@ -141,7 +141,11 @@ lsm_status lsm_update_batch_ordered(lsm_t* h, const uint32_t* d_keys, const uint
  *   d_found   nq outputs: 1 when the key is present, else 0.
  * Full levels are searched from the newest (smallest) to the oldest; the first
  * element of the key found decides: regular -> found, tombstone -> absent.
- * nq = 0 is a no-op.  Asynchronous.
+ * nq = 0 is a no-op.  Asynchronous.  Many queries (from several 10^5 on,
+ * depending on the levels) are grouped by key range first, in about 7.3 bytes
+ * per query of the handle's query scratch (grown on demand; growing it
+ * synchronises the device); without that memory, and on a stream that is
+ * being captured, they are searched in input order.
  */
 lsm_status lsm_lookup(lsm_t* h, const uint32_t* d_q, uint64_t nq, uint32_t* d_val,
                       uint8_t* d_found, void* stream);
@@ -316,7 +320,8 @@ lsm_status lsm_sort_pairs_noalloc(const uint32_t* d_keys_in, const uint32_t* d_v
 /*
  * lsm_set_option / lsm_get_option - tuning knobs (integers):
  *   LSM_OPT_LOOKUP_MODE  0 = automatic, 1 = one search per query in input
- *                        order, 2 = sort the queries first (§IV-B "bulk").
+ *                        order, 2 = group the queries by key range first
+ *                        (§IV-B "bulk").
  *   LSM_OPT_DEVICE_ERROR read-only: sticky device error bits seen so far
  *                        (1 = bad key, 2 = wait timeout, 4 = misaligned
  *                        copy avoided); synchronises; reading clears them.

@@ -259,6 +259,24 @@ cudaError_t ensure_q(lsm_t* h, size_t bytes) {
   return e;
 }
 
+// Whether many lookups are worth grouping by key range (lookup_bulk_launch).
+// Measured over 1 to 7 full levels, 4 thousand to 264 million elements and 2^14
+// to 2^24 queries, half of them hits, a query costs about
+//   in input order  4 + 10 levels + 40 min(1.2, elements / 10^8)   ps
+//   grouped         18 + 3 levels + 8 min(1.2, elements / 10^8)    ps
+// and the grouping some 45 us, so it pays from 6 10^5 queries (seven levels of
+// 133 million: 2^20 lookups 150 -> 120 us, 2^24 2197 -> 835), 1.4 10^6 (one level
+// of 2^27: 2^21 115 and 115 us, 2^24 866 -> 469), 6 10^6 (three small levels:
+// 2^23 255 -> 225 us) on, and never for one or two levels that L2 holds (one of
+// 2^24: 2^24 lookups 278 against 371 us).
+bool bulk_pays(const LevelSet& ls, uint64_t nq) {
+  uint64_t n = 0;
+  for (int l = 0; l < ls.count; ++l) n += ls.n[l];
+  const double big = double(n) / 1e8;
+  const double ps = 7.0 * ls.count + 32.0 * (big < 1.2 ? big : 1.2) - 14.0;
+  return double(nq) * ps > 45e6;
+}
+
 // Stable sort of (keys[i], i) for i < n into the query scratch (grown on
 // demand, `extra` more words kept after the four sort arrays); returns the
 // sorted keys and positions.
@@ -630,14 +648,19 @@ lsm_status lsm_lookup(lsm_t* h, const uint32_t* d_q, uint64_t nq, uint32_t* d_va
     LSM_TRY(cudaMemsetAsync(d_found, 0, nq, st));
     return LSM_OK;
   }
-  const bool sorted = h->lookup_mode == 2 && nq <= 0xFFFFFFFFull;
+  bool bulk = nq <= kBulkMaxQueries && (h->lookup_mode == 2 || (h->lookup_mode == 0 && bulk_pays(ls, nq)));
+  if (bulk) {
+    // Without the scratch (no memory, or a stream being captured, whose graph
+    // would keep a pointer that a later call may free) the queries are
+    // searched in input order.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bulk = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+           ensure_q(h, lookup_bulk_bytes(nq)) == cudaSuccess;
+    if (!bulk) cudaGetLastError();
+  }
   ProfScope ps(h, LSM_PROF_LOOKUP, double(nq) * (9.0 + 32.0 * ls.count), st);
-  if (!sorted) return cuda_status(lookup_launch(ls, d_q, nq, d_val, d_found, st));
-  // Sorted mode: radix sort (key, position), then warp-cooperative search.
-  uint32_t* sk = nullptr;
-  uint32_t* sv = nullptr;
-  LSM_TRY(sort_positions(h, d_q, nq, 0, st, &sk, &sv));
-  return cuda_status(lookup_sorted_launch(ls, sk, sv, nq, d_val, d_found, st));
+  if (!bulk) return cuda_status(lookup_launch(ls, d_q, nq, d_val, d_found, st));
+  return cuda_status(lookup_bulk_launch(ls, d_q, nq, d_val, d_found, h->d_q, st));
 }
 
 static lsm_status neighbor_call(lsm_t* h, const uint32_t* d_q, uint64_t nq, bool successor, uint32_t* d_key,

@@ -341,6 +341,13 @@ cudaError_t build_fence_launch(const uint32_t* keys, uint32_t n, uint32_t* fence
 cudaError_t lookup_launch(const LevelSet& ls, const uint32_t* q, uint64_t nq,
                           uint32_t* val, uint8_t* found, cudaStream_t st);
 
+// The same for many queries (at most kBulkMaxQueries), grouped by key range
+// first; scratch: lookup_bulk_bytes(nq) bytes, 16-byte aligned.
+constexpr uint64_t kBulkMaxQueries = 1ull << 31;
+size_t lookup_bulk_bytes(uint64_t nq);
+cudaError_t lookup_bulk_launch(const LevelSet& ls, const uint32_t* q, uint64_t nq, uint32_t* val, uint8_t* found,
+                               void* scratch, cudaStream_t st);
+
 // Lookup of queries already sorted by key (kSortQueries output): results go
 // to positions idx[i] of the output arrays.
 cudaError_t lookup_sorted_launch(const LevelSet& ls, const uint32_t* sq, const uint32_t* idx,

@@ -49,3 +49,30 @@ def test_wide_windows(g, r, space):
         lsm.cleanup()                          # the second time over what a cleanup leaves
     assert lsm.device_errors() == 0
     lsm.close()
+
+
+@pytest.mark.parametrize("nq", [1, 8191, 8192, 8193, 70000, (1 << 20) + 77])
+@pytest.mark.parametrize("qdist", ["mixed", "one", "narrow"])
+def test_bulk_lookups_agree(g, nq, qdist):
+    """Lookups grouped by key range against the same ones in input order: ragged tiles, all queries in one part of
+    the range, keys outside the levels' range and above the user keys."""
+    rng = np.random.default_rng(nq)
+    lsm = g.LSM(5000, 32 * 5000)
+    keys = (1 << 27) + rng.integers(0, 1 << 26, 11 * 5000)
+    for t in range(11):
+        k = keys[t * 5000:(t + 1) * 5000].astype(np.uint32)
+        lsm.update(k, rng.integers(0, 1 << 32, 5000, dtype=np.uint64).astype(np.uint32), (rng.random(5000) < 0.2).astype(np.uint8))
+    q = np.where(rng.random(nq) < 0.5, rng.choice(keys, nq), rng.integers(0, 1 << 32, nq))
+    if qdist == "one":
+        q = np.full(nq, keys[77])
+    elif qdist == "narrow":
+        q = keys[5] + rng.integers(0, 9, nq)
+    q = g.as_device_u32(q.astype(np.uint32), 0)
+    out = []
+    for mode in (g.LOOKUP_DIRECT, g.LOOKUP_SORTED, g.LOOKUP_AUTO):
+        lsm.set_lookup_mode(mode)
+        out.append(lsm.lookup(q))
+    for val, found in out[1:]:
+        assert torch.equal(val, out[0][0]) and torch.equal(found, out[0][1])
+    assert int(out[0][1].sum()) > 0 or nq == 1 or qdist != "mixed"
+    lsm.close()
