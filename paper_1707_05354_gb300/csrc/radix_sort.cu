@@ -44,29 +44,53 @@ struct Loader {
   uint32_t n_in;  // ops in the input, 1 .. n
   uint32_t n;
 
-  // Element p of the logical sequence.  Batch modes: position p of the
-  // reversed padded batch, i.e. op min(n - 1 - p, n_in - 1).
-  __device__ __forceinline__ void load(uint32_t p, uint32_t& kv, uint32_t& v, bool& bad) const {
-    bad = false;
-    if (mode == kSortPairs) {
-      kv = __ldg(keys + p);
-      v = __ldg(vals + p);
-      return;
+  // Calls f with the mode as a compile-time constant: a loop over elements
+  // inside f has no branch on it, so that all its loads are issued before the
+  // first is waited for.
+  template <class F>
+  __device__ __forceinline__ void with_mode(const F& f) const {
+    switch (mode) {
+      case kSortPairs: return f(Mode<kSortPairs>{});
+      case kSortInsert: return f(Mode<kSortInsert>{});
+      case kSortDelete: return f(Mode<kSortDelete>{});
+      case kSortUpdate: return f(Mode<kSortUpdate>{});
+      default: return f(Mode<kSortQueries>{});
     }
-    if (mode == kSortQueries) {
-      kv = __ldg(keys + p);
-      v = p;
-      return;
-    }
-    const uint32_t s = min(n - 1 - p, n_in - 1);
-    // the key, delete flag and value loads are independent (insert and
-    // update calls always pass values), so they are in flight together
-    const uint32_t k = __ldg(keys + s);
-    const uint32_t v0 = mode != kSortDelete ? __ldg(vals + s) : 0u;
-    const bool is_del = (mode == kSortDelete) || (mode == kSortUpdate && __ldg(del + s) != 0);
-    bad = k > kMaxUserKey;
-    kv = bad ? kPlaceboKv : ((k << 1) | (is_del ? 0u : 1u));
-    v = (is_del || bad) ? 0u : v0;
+  }
+  template <int M>
+  struct Mode {
+    static constexpr int value = M;
+    static constexpr bool batch = M != kSortPairs && M != kSortQueries;
+  };
+
+  // Where element p of the logical sequence comes from.  Batch modes:
+  // position p of the reversed padded batch, i.e. op min(n - 1 - p, n_in - 1).
+  template <int M>
+  __device__ __forceinline__ uint32_t src(uint32_t p) const {
+    return Mode<M>::batch ? min(n - 1 - p, n_in - 1) : p;
+  }
+  // Delete flag of input s (as loaded: any value but 0 deletes).
+  template <int M>
+  __device__ __forceinline__ uint32_t flag(uint32_t s) const {
+    return M == kSortUpdate ? uint32_t(__ldg(del + s)) : uint32_t(M == kSortDelete);
+  }
+  // Key variable of an input key with its flag; bad: a key above the user
+  // range, which becomes a placebo tombstone.
+  template <int M>
+  static __device__ __forceinline__ uint32_t encode(uint32_t k, uint32_t fl, bool& bad) {
+    if (!Mode<M>::batch) return k;
+    const bool b = k > kMaxUserKey;
+    bad |= b;
+    return b ? kPlaceboKv : ((k << 1) | (fl ? 0u : 1u));
+  }
+  // Value of element p, as loaded; tombstones (and so bad keys) carry 0.
+  template <int M>
+  __device__ __forceinline__ uint32_t raw_val(uint32_t p) const {
+    return M == kSortQueries ? p : (M == kSortDelete ? 0u : __ldg(vals + src<M>(p)));
+  }
+  template <int M>
+  static __device__ __forceinline__ uint32_t val_of(uint32_t kv, uint32_t raw) {
+    return Mode<M>::batch && !(kv & 1u) ? 0u : raw;
   }
 
   // Leading positions of the reversed padded batch that are padding (copies
@@ -76,24 +100,82 @@ struct Loader {
     return n - n_in;
   }
 
-  // The value of element p, whose key variable is kv.
-  __device__ __forceinline__ uint32_t load_val(uint32_t p, uint32_t kv) const {
-    if (mode == kSortPairs) return __ldg(vals + p);
-    if (mode == kSortQueries) return p;
-    if (mode == kSortDelete || !(kv & 1u)) return 0u;  // tombstones (bad keys are placebo tombstones) carry 0
-    const uint32_t s = min(n - 1 - p, n_in - 1);
-    return __ldg(vals + s);
+  // One element.
+  __device__ __forceinline__ void load(uint32_t p, uint32_t& kv, uint32_t& v, bool& bad) const {
+    bad = false;
+    with_mode([&](auto m) {
+      constexpr int M = decltype(m)::value;
+      kv = encode<M>(__ldg(keys + src<M>(p)), flag<M>(src<M>(p)), bad);
+      v = val_of<M>(kv, raw_val<M>(p));
+    });
+  }
+  __device__ __forceinline__ uint32_t load_key(uint32_t p, bool& bad) const {
+    uint32_t kv = 0;
+    bad = false;
+    with_mode([&](auto m) {
+      constexpr int M = decltype(m)::value;
+      kv = encode<M>(__ldg(keys + src<M>(p)), flag<M>(src<M>(p)), bad);
+    });
+    return kv;
   }
 
-  // Key variable only (the histogram needs no values).
-  __device__ __forceinline__ uint32_t load_key(uint32_t p, bool& bad) const {
-    bad = false;
-    if (mode == kSortPairs || mode == kSortQueries) return __ldg(keys + p);
-    const uint32_t s = min(n - 1 - p, n_in - 1);
-    const uint32_t k = __ldg(keys + s);
-    const bool is_del = (mode == kSortDelete) || (mode == kSortUpdate && __ldg(del + s) != 0);
-    bad = k > kMaxUserKey;
-    return bad ? kPlaceboKv : ((k << 1) | (is_del ? 0u : 1u));
+  // Elements p0 + step j of a thread, j < N, that pass `in(p)`: all loads
+  // first.  Elements outside keep kv = `none` and v = 0.
+  template <int N, class In>
+  __device__ __forceinline__ void load_keys(uint32_t p0, uint32_t step, const In& in, uint32_t none, uint32_t (&kv)[N],
+                                            bool& bad) const {
+    with_mode([&](auto m) {
+      constexpr int M = decltype(m)::value;
+      uint32_t fl[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const uint32_t p = p0 + j * step;
+        if (in(p)) {
+          kv[j] = __ldg(keys + src<M>(p));
+          fl[j] = flag<M>(src<M>(p));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < N; ++j) kv[j] = in(p0 + j * step) ? encode<M>(kv[j], fl[j], bad) : none;
+    });
+  }
+  template <int N, class In>
+  __device__ __forceinline__ void load_vals(uint32_t p0, uint32_t step, const In& in, const uint32_t (&kv)[N],
+                                            uint32_t (&v)[N]) const {
+    with_mode([&](auto m) {
+      constexpr int M = decltype(m)::value;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const uint32_t p = p0 + j * step;
+        const uint32_t x = kv[j];
+        v[j] = in(p) ? raw_val<M>(p) : 0u;
+        v[j] = val_of<M>(x, v[j]);
+      }
+    });
+  }
+  template <int N, class In>
+  __device__ __forceinline__ void load_items(uint32_t p0, uint32_t step, const In& in, uint32_t (&kv)[N],
+                                             uint32_t (&v)[N], bool& bad) const {
+    with_mode([&](auto m) {
+      constexpr int M = decltype(m)::value;
+      uint32_t fl[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const uint32_t p = p0 + j * step;
+        kv[j] = v[j] = fl[j] = 0u;
+        if (in(p)) {
+          kv[j] = __ldg(keys + src<M>(p));
+          fl[j] = flag<M>(src<M>(p));
+          v[j] = raw_val<M>(p);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        if (!in(p0 + j * step)) continue;
+        kv[j] = encode<M>(kv[j], fl[j], bad);
+        v[j] = val_of<M>(kv[j], v[j]);
+      }
+    });
   }
 };
 
@@ -126,16 +208,12 @@ __global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32
   bool bad_any = false;
   for (uint64_t p0 = uint64_t(blockIdx.x) * kHistChunk; p0 < ld.n; p0 += uint64_t(gridDim.x) * kHistChunk) {
     uint32_t kv[kHistItems];
+    const uint32_t left = uint32_t(ld.n - p0 < kHistChunk ? ld.n - p0 : kHistChunk);
+    ld.load_keys(uint32_t(p0) + threadIdx.x, uint32_t(kPassThreads),
+                 [&](uint32_t p) { return p - uint32_t(p0) < left; }, 0u, kv, bad_any);
 #pragma unroll
     for (uint32_t j = 0; j < kHistItems; ++j) {
-      const uint64_t p = p0 + j * kPassThreads + threadIdx.x;
-      bool bad = false;
-      kv[j] = p < ld.n ? ld.load_key(uint32_t(p), bad) : 0u;
-      bad_any |= bad;
-    }
-#pragma unroll
-    for (uint32_t j = 0; j < kHistItems; ++j) {
-      if (p0 + j * kPassThreads + threadIdx.x < ld.n) {
+      if (j * kPassThreads + threadIdx.x < left) {
 #pragma unroll
         for (int d = 0; d < kSortPasses; ++d) atomicAdd(&s_h[d * kRadix + ((kv[j] >> (8 * d)) & 255u)], 1u);
       }
@@ -192,13 +270,16 @@ __global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const ui
   const uint32_t tile_n = (n - tile_start) < uint32_t(kSortTile) ? (n - tile_start) : uint32_t(kSortTile);
   const uint32_t e0 = warp * (32 * kIPT) + lane;  // item j: element e0 + 32 j of the tile
 
+  // past the end: the last digit, after every element of it
   uint32_t kv[kIPT], at[kIPT];
+  const auto inside = [&](uint32_t p) { return p - tile_start < tile_n; };
+  if (kFirst) {
+    bool bad = false;
+    ld.load_keys(tile_start + e0, 32u, inside, 0xFFFFFFFFu, kv, bad);
+  } else {
 #pragma unroll
-  for (int j = 0; j < kIPT; ++j) {
-    const uint32_t e = e0 + j * 32;
-    bool bad;
-    kv[j] = 0xFFFFFFFFu;  // past the end: the last digit, after every element of it
-    if (e < tile_n) kv[j] = kFirst ? ld.load_key(tile_start + e, bad) : __ldg(in_k + tile_start + e);
+    for (int j = 0; j < kIPT; ++j)
+      kv[j] = inside(tile_start + e0 + j * 32) ? __ldg(in_k + tile_start + e0 + j * 32) : 0xFFFFFFFFu;
   }
   const uint32_t hist = tid < kRadix ? ctl[pass * kRadix + tid] : 0u;
 
@@ -263,10 +344,12 @@ __global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const ui
     at[j] += sh.whist[warp][d];
     sh.keys[at[j]] = kv[j];
   }
+  if (kFirst) {
+    ld.load_vals(tile_start + e0, 32u, inside, kv, kv);
+  } else {
 #pragma unroll
-  for (int j = 0; j < kIPT; ++j) {
-    const uint32_t e = e0 + j * 32;
-    if (e < tile_n) kv[j] = kFirst ? ld.load_val(tile_start + e, kv[j]) : __ldg(in_v + tile_start + e);
+    for (int j = 0; j < kIPT; ++j)
+      if (inside(tile_start + e0 + j * 32)) kv[j] = __ldg(in_v + tile_start + e0 + j * 32);
   }
 #pragma unroll
   for (int j = 0; j < kIPT; ++j) sh.vals[at[j]] = kv[j];
@@ -469,17 +552,7 @@ __global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t*
   const uint32_t base = t0 + warp * (32 * kScatterIPT);
   uint32_t kv[kScatterIPT], v[kScatterIPT], rank[kScatterIPT];
   bool bad_any = false;
-#pragma unroll
-  for (int j = 0; j < kScatterIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    kv[j] = 0;
-    v[j] = 0;
-    if (p < n && p >= npad) {
-      bool bad;
-      ld.load(p, kv[j], v[j], bad);
-      bad_any |= bad;
-    }
-  }
+  ld.load_items(base + lane, 32u, [&](uint32_t p) { return p < n && p >= npad; }, kv, v, bad_any);
   const int any_bad = __syncthreads_or(bad_any);
   if (tid == 0) check.done(ctl, any_bad != 0);
   const KeyMap map = sample_map<kScatterThreads>(ld, s_cnt, s_cnt + kScatterWarps);
