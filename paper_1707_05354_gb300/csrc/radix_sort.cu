@@ -717,8 +717,9 @@ struct BucketShared {
 };
 
 // Sorts m <= kBucketCap elements stably by the key variable (all in
-// [range.lo, range.hi]) and hands each to emit(position, kv, value).  With
-// kGather the elements are read from the source, otherwise bsm holds them in
+// [range.lo, range.hi]) and hands each to emit(position, kv, value).
+// load(kv, v) fills a thread's elements threadIdx.x + j kBucketThreads (< m) of
+// the stable order; with kHeld they come from bsm, which holds all of them in
 // order (kBucketCap words of keys, then the values).
 //   Fast path (no sub-bin above kSubBinMax): one counting pass places every
 //   element in its sub-bin (about one element each for spread keys), at an
@@ -729,25 +730,16 @@ struct BucketShared {
 //   Otherwise stable 8-bit passes over the bits in which the range differs.
 // bsm holds 4 kBucketCap words plus kBucketCap 16-bit indexes.  The view
 // returned stays valid until bsm or sh.whist change.
-template <bool kGather, class Src, class Emit>
-__device__ __forceinline__ SortedView sort_resident(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
-                                                    uint32_t m, const BucketRange& range, uint32_t* bsm,
-                                                    BucketShared& sh, const Emit& emit) {
+template <bool kHeld, class Load, class Emit>
+__device__ __forceinline__ SortedView sort_resident(const Load& load, uint32_t m, const BucketRange& range,
+                                                    uint32_t* bsm, BucketShared& sh, const Emit& emit) {
   static_assert(kSubBins == kBucketWarps * kRadix, "the counters reuse the per-warp histograms");
   uint32_t *ak = bsm, *av = bsm + kBucketCap, *bk = bsm + 2 * kBucketCap, *bv = bsm + 3 * kBucketCap;
   uint16_t* bi = reinterpret_cast<uint16_t*>(bsm + 4 * kBucketCap);
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   uint32_t* cnt = &sh.whist[0][0];
   uint32_t kv[kBucketIPT], v[kBucketIPT];
-#pragma unroll
-  for (int j = 0; j < kBucketIPT; ++j) {
-    const uint32_t i = tid + j * kBucketThreads;
-    if (i < m) {
-      const uint32_t at = kGather ? src.at(i) : i;
-      kv[j] = kGather ? src_k[at] : ak[at];
-      v[j] = kGather ? src_v[at] : av[at];
-    }
-  }
+  load(kv, v);
   for (uint32_t i = tid; i < kSubBins; i += kBucketThreads) cnt[i] = 0u;
   if (tid == 0) sh.max = 0u;
   __syncthreads();
@@ -830,7 +822,7 @@ __device__ __forceinline__ SortedView sort_resident(const uint32_t* src_k, const
   __syncthreads();
   // Many copies of one key, or a cluster.  The block is laid out with as many
   // items a thread as m needs, so that a small bucket's passes are short.
-  if (kGather) {
+  if (!kHeld) {
 #pragma unroll
     for (int j = 0; j < kBucketIPT; ++j) {
       const uint32_t i = tid + j * kBucketThreads;
@@ -1094,7 +1086,17 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
     __syncthreads();
     if (kept) {
       const BucketRange part{mn, mx, SubMap::of(mn, float(mx - mn) + 1.0f)};
-      sort_resident<false>(src_k, src_v, src, kept, part, bsm, sh, [&](uint32_t i, uint32_t kk, uint32_t vv) {
+      const auto load = [&](uint32_t (&kv)[kBucketIPT], uint32_t (&v)[kBucketIPT]) {
+#pragma unroll
+        for (int j = 0; j < kBucketIPT; ++j) {
+          const uint32_t i = tid + j * kBucketThreads;
+          if (i < kept) {
+            kv[j] = ak[i];
+            v[j] = av[i];
+          }
+        }
+      };
+      sort_resident<true>(load, kept, part, bsm, sh, [&](uint32_t i, uint32_t kk, uint32_t vv) {
         const uint32_t dst = start + done + i + (copies && key_of(kk) > hot ? copies : 0u) + shift(kk);
         out_k[dst] = kk;
         out_v[dst] = vv;
@@ -1107,61 +1109,160 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
   __syncthreads();  // the caller reads the output back
 }
 
+// Prefix-index entries `bins` of a bucket at `start`: the elements in `view`
+// and the padding run.  `ends`: bit 0 when the bucket holds the first element
+// of the output, bit 1 the last; its entries are then written inside the
+// populated bin range only, whose bound is recorded.
+__device__ __forceinline__ void write_bins(const SortedView& view, uint32_t start, const PadRun& pad, BinRange bins,
+                                           int ends) {
+  if (!bins.fence) return;
+  if (ends) {
+    const uint32_t nb = fence_bins(bins.fshift);
+    if (ends & 1) {
+      const uint32_t kv = min(view.m ? view.smallest() : pad.kv, pad.n ? pad.kv : 0xFFFFFFFFu);
+      bins.bin0 = max(bins.bin0, fence_bin(kv, bins.fshift) + 1);
+      if (threadIdx.x == 0) bins.fence[nb + 2] = fence_bin(kv, bins.fshift);
+    }
+    if (ends & 2) {
+      const uint32_t kv = max(view.m ? view.largest() : pad.kv, pad.n ? pad.kv : 0u);
+      bins.bin1 = min(bins.bin1, fence_bin(kv, bins.fshift) + 1);
+      if (threadIdx.x == 0) {
+        bins.fence[nb + 3] = fence_bin(kv, bins.fshift);
+        bins.fence[nb] = start + view.m + pad.n;
+      }
+    }
+  }
+  for (uint32_t P = bins.bin0 + threadIdx.x; P < bins.bin1; P += blockDim.x) {
+    const uint32_t kv = P << bins.fshift;
+    bins.fence[P] = start + (view.m ? view.less(kv) : 0u) + (pad.n && kv > pad.kv ? pad.n : 0u);
+  }
+}
+
+// A bucket that fits shared memory: the elements given by `load` (see
+// sort_resident), with the padding run at its sorted place, to out[start ..)
+// and its prefix-index entries.
+template <class Load>
+__device__ __forceinline__ void resident_body(const Load& load, uint32_t* out_k, uint32_t* out_v, uint32_t start,
+                                              uint32_t m, const BucketRange& range, const PadRun& pad,
+                                              const BinRange& bins, int ends, uint32_t* bsm, BucketShared& sh) {
+  SortedView view{bsm, 0u, nullptr, range.map};
+  if (m)
+    view = sort_resident<false>(load, m, range, bsm, sh, [&](uint32_t i, uint32_t k, uint32_t v) {
+      const uint32_t dst = start + i + (pad.n && k >= pad.kv ? pad.n : 0u);
+      out_k[dst] = k;
+      out_v[dst] = v;
+    });
+  if (pad.n) {
+    const uint32_t L = m ? view.less(pad.kv) : 0u;
+    for (uint32_t j = threadIdx.x; j < pad.n; j += blockDim.x) {
+      out_k[start + L + j] = pad.kv;
+      out_v[start + L + j] = pad.v;
+    }
+  }
+  write_bins(view, start, pad, bins, ends);
+}
+
 // One bucket, one CTA of kBucketThreads: sorts the m elements src.at(0 ..
 // m - 1) of (src_k, src_v) stably by the key variable into out[start, start +
 // m + pad.n) and writes the prefix-index entries `bins` of the result.  The
 // padding run (a short batch's, which comes first among equal key variables
-// in the stable order) is written at its sorted place.  `ends`: bit 0 when
-// the bucket holds the first element of the output, bit 1 the last; its
-// entries are then written inside the populated bin range only, whose bound
-// is recorded.
+// in the stable order) is written at its sorted place.
 template <class Src>
 __device__ __forceinline__ void bucket_body(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
                                             uint32_t* out_k, uint32_t* out_v, uint32_t start, uint32_t m,
                                             const BucketRange& range, const PadRun& pad, BinRange bins, int ends,
                                             uint32_t* bsm, BucketShared& sh) {
   SortedView view{out_k + start, m + pad.n, nullptr, range.map};
-  uint32_t extra = 0;  // padding elements that the view does not hold
   if (m > kBucketCap) {
     sort_big(src_k, src_v, src, out_k, out_v, start, m, range, pad, bsm, sh);
-  } else {
-    if (m)
-      view = sort_resident<true>(src_k, src_v, src, m, range, bsm, sh, [&](uint32_t i, uint32_t k, uint32_t v) {
-        const uint32_t dst = start + i + (pad.n && k >= pad.kv ? pad.n : 0u);
-        out_k[dst] = k;
-        out_v[dst] = v;
-      });
-    view.m = m;
-    extra = pad.n;
-    if (pad.n) {
-      const uint32_t L = m ? view.less(pad.kv) : 0u;
-      for (uint32_t j = threadIdx.x; j < pad.n; j += blockDim.x) {
-        out_k[start + L + j] = pad.kv;
-        out_v[start + L + j] = pad.v;
+    write_bins(view, start, PadRun{0u, 0u, 0u}, bins, ends);
+    return;
+  }
+  const auto load = [&](uint32_t (&kv)[kBucketIPT], uint32_t (&v)[kBucketIPT]) {
+#pragma unroll
+    for (int j = 0; j < kBucketIPT; ++j) {
+      const uint32_t i = threadIdx.x + j * kBucketThreads;
+      if (i < m) {
+        const uint32_t at = src.at(i);
+        kv[j] = src_k[at];
+        v[j] = src_v[at];
       }
     }
+  };
+  resident_body(load, out_k, out_v, start, m, range, pad, bins, ends, bsm, sh);
+}
+
+// A batch whose deferred key check failed becomes n placebo tombstones (the
+// key 2^31 - 1 that no query sees), all in the last bin.  CTA d of `ctas`.
+__device__ __forceinline__ void write_placebos(uint32_t* out_k, uint32_t* out_v, uint32_t n, uint32_t* fence,
+                                               int fshift, uint32_t d, uint32_t ctas) {
+  const uint32_t at = d * blockDim.x + threadIdx.x, step = ctas * blockDim.x;
+  for (uint32_t i = at; i < n; i += step) {
+    out_k[i] = kPlaceboKv;
+    out_v[i] = 0u;
   }
-  if (!bins.fence) return;
-  if (ends) {
-    const uint32_t nb = fence_bins(bins.fshift);
-    if (ends & 1) {
-      const uint32_t kv = min(view.m ? view.smallest() : pad.kv, extra ? pad.kv : 0xFFFFFFFFu);
-      bins.bin0 = max(bins.bin0, fence_bin(kv, bins.fshift) + 1);
-      if (threadIdx.x == 0) bins.fence[nb + 2] = fence_bin(kv, bins.fshift);
+  if (fence) {
+    const uint32_t nb = fence_bins(fshift);
+    for (uint32_t i = at; i < nb; i += step) fence[i] = 0u;
+    if (at == 0) {
+      fence[nb] = n;
+      fence[nb + 2] = 0u;
+      fence[nb + 3] = nb - 1;
     }
-    if (ends & 2) {
-      const uint32_t kv = max(view.m ? view.largest() : pad.kv, extra ? pad.kv : 0u);
-      bins.bin1 = min(bins.bin1, fence_bin(kv, bins.fshift) + 1);
-      if (threadIdx.x == 0) {
-        bins.fence[nb + 3] = fence_bin(kv, bins.fshift);
-        bins.fence[nb] = start + m + pad.n;
-      }
+  }
+}
+
+// The whole sort of at most kBucketCap elements in one CTA and one launch:
+// bound by the chain of its barriers, 4.1 us where the two kernels took
+// 12.2 (lsm_sort_pairs of 2^10 pairs, back to back).
+__global__ void __launch_bounds__(kBucketThreads) small_sort(Loader ld, uint32_t* out_k, uint32_t* out_v,
+                                                             uint32_t* fence, int fshift, uint32_t* host,
+                                                             uint32_t seq, uint32_t* defer_err) {
+  extern __shared__ __align__(16) uint32_t bsm[];
+  __shared__ BucketShared sh;
+  pdl_trigger();
+  pdl_wait();
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t npad = ld.npad(), m = ld.n - npad;
+  uint32_t kv[kBucketIPT], v[kBucketIPT];
+  bool bad = false;
+  ld.load_items(npad + tid, uint32_t(kBucketThreads), [&](uint32_t p) { return p < ld.n; }, kv, v, bad);
+  uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+#pragma unroll
+  for (int j = 0; j < kBucketIPT; ++j) {
+    if (tid + j * kBucketThreads < m) {
+      mn = min(mn, kv[j]);
+      mx = max(mx, kv[j]);
     }
   }
-  for (uint32_t P = bins.bin0 + threadIdx.x; P < bins.bin1; P += blockDim.x) {
-    const uint32_t kv = P << bins.fshift;
-    bins.fence[P] = start + (view.m ? view.less(kv) : 0u) + (extra && kv > pad.kv ? extra : 0u);
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) {
+    sh.cand[warp] = mn;
+    sh.votes[warp] = mx;
   }
+  const int any_bad = __syncthreads_or(bad);
+  if (tid == 0 && host) *reinterpret_cast<volatile uint32_t*>(host) = check_word(seq, any_bad != 0);
+  if (any_bad && defer_err) {
+    write_placebos(out_k, out_v, ld.n, fence, fshift, 0u, 1u);
+    if (tid == 0) atomicOr(defer_err, kErrBadKey);
+    return;
+  }
+  const uint32_t w = lane & uint32_t(kBucketWarps - 1);
+  mn = __reduce_min_sync(0xffffffffu, sh.cand[w]);
+  mx = __reduce_max_sync(0xffffffffu, sh.votes[w]);
+  PadRun pad{npad, 0u, 0u};
+  if (npad) ld.load(0, pad.kv, pad.v, bad);
+  const BinRange bins{fence, fshift, 0u, fence ? fence_bins(fshift) : 0u};
+  const BucketRange range{mn, mx, SubMap::of(mn, float(mx - mn) + 1.0f)};
+  const auto load = [&](uint32_t (&k)[kBucketIPT], uint32_t (&x)[kBucketIPT]) {
+#pragma unroll
+    for (int j = 0; j < kBucketIPT; ++j) {
+      k[j] = kv[j];
+      x[j] = v[j];
+    }
+  };
+  resident_body(load, out_k, out_v, 0u, m, range, pad, bins, 3, bsm, sh);
 }
 
 __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, const uint32_t* __restrict__ tmp_k,
@@ -1183,23 +1284,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
   if (d == 0)
     for (uint32_t i = tid; i < uint32_t(kSortCtlWords); i += kBucketThreads) next_ctl[i] = 0u;
   if (defer_err && ctl[kSortCtlStatus]) {
-    // Deferred key check failed: the batch becomes n placebo tombstones (the
-    // key 2^31 - 1 that no query sees), all in the last bin.
-    const uint32_t chunk = (n + kRadix - 1) / kRadix;
-    const uint32_t lo = d * chunk, hi = (lo + chunk) < n ? lo + chunk : n;
-    for (uint32_t i = lo + tid; i < hi; i += kBucketThreads) {
-      out_k[i] = kPlaceboKv;
-      out_v[i] = 0u;
-    }
-    if (fence) {
-      const uint32_t per = 1u << (24 - fshift);
-      for (uint32_t i = tid; i < per; i += kBucketThreads) fence[d * per + i] = 0u;
-      if (d == kRadix - 1 && tid == 0) {
-        fence[fence_bins(fshift)] = n;
-        fence[fence_bins(fshift) + 2] = 0u;
-        fence[fence_bins(fshift) + 3] = fence_bins(fshift) - 1;
-      }
-    }
+    write_placebos(out_k, out_v, n, fence, fshift, d, kRadix);
     if (d == 0 && tid == 0) atomicOr(defer_err, kErrBadKey);
     return;
   }
@@ -1440,14 +1525,14 @@ __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) 
 }  // namespace
 
 constexpr size_t kBucketSmem = 4 * size_t(kBucketCap) * sizeof(uint32_t) + size_t(kBucketCap) * sizeof(uint16_t);
-PerDeviceFlags g_bucket_attr, g_pass_attr[2];
+PerDeviceFlags g_bucket_attr[2], g_pass_attr[2];
 
 cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_t st, uint32_t* status,
                                uint32_t seq) {
   cudaError_t e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = set_smem_attr_once(bucket_sort, kBucketSmem, dev, g_bucket_attr)) != cudaSuccess) return e;
+  if ((e = set_smem_attr_once(bucket_sort, kBucketSmem, dev, g_bucket_attr[0])) != cudaSuccess) return e;
   const uint32_t ntiles = (a.n + kMsdTile - 1) / kMsdTile;
   uint2* runs = reinterpret_cast<uint2*>(ws.tilecnt);
   uint32_t* ctl = ws.ctl + ws.flip * kSortCtlWords;
@@ -1455,6 +1540,12 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
   Loader ld{a.mode, a.in_keys, a.in_vals, a.in_del, uint32_t(a.n_in), a.n};
   // a deferred check leaves its verdict in the sort's own control block
   const KeyCheck check{a.defer_err ? nullptr : status, seq, a.defer_err || status};
+  if (a.n <= kBucketCap) {
+    if ((e = set_smem_attr_once(small_sort, kBucketSmem, dev, g_bucket_attr[1])) != cudaSuccess) return e;
+    count_launches(1);  // (the control block stays as it is)
+    return launch_pdl(small_sort, dim3(1), dim3(kBucketThreads), kBucketSmem, st, ld, a.out_keys, a.out_vals, a.fence,
+                      a.fshift, a.defer_err ? nullptr : status, seq, a.defer_err);
+  }
   count_launches(1);
   if ((e = launch_pdl(msd_tile, dim3(ntiles), dim3(kScatterThreads), 0, st, ld, a.tmp_keys, a.tmp_vals, runs, ctl,
                       check)) != cudaSuccess)

@@ -136,3 +136,37 @@ def test_refused_batches_between_folds(g, b):
         np.testing.assert_array_equal(kv, ekv)
         np.testing.assert_array_equal(vv, ev)
     lsm.close()
+
+
+@pytest.mark.parametrize("b", [1, 33, 5119, 5120, 5121])
+@pytest.mark.parametrize("dist", ["one", "ids", "hot", "zipf"])
+def test_small_batches(g, dist, b):
+    """Batches at the edge of the one-kernel sort, full and short, with the key check waited for and deferred (a bad
+    batch then becomes placebos that no query sees)."""
+    rng = np.random.default_rng(b)
+    lsm, s, o1 = g.LSM(b, 32 * b), oracle.StructuralOracle(b), oracle.MapOracle(b)
+    seen = []
+    for t in range(9):
+        n = b if t % 3 else max(1, b - b // 3)
+        k, v = draw(dist, n, rng), rng.integers(0, 1 << 31, n).astype(np.uint32)
+        d = (rng.random(n) < 0.3).astype(np.uint8)
+        for x in (lsm, s, o1):
+            x.call("update", k, v, d)
+        seen.append(k)
+    for i, (kv, vv) in lsm.levels().items():
+        ekv, ev = s.level(i)
+        np.testing.assert_array_equal(kv, ekv)
+        np.testing.assert_array_equal(vv, ev)
+    bad = draw(dist, b, rng)
+    bad[-1] = TOP
+    with pytest.raises(g.LSMError):
+        lsm.insert(bad, np.zeros(b, np.uint32))
+    g.lsm_set_option(lsm.h, g.LSM_OPT_KEY_CHECK, 1)
+    lsm.insert(bad, np.zeros(b, np.uint32))
+    assert lsm.r == 10 and lsm.device_errors() & 1
+    q = np.concatenate(seen + [np.arange(50)]).astype(np.uint32)
+    val, found = lsm.lookup(q)
+    ev, ef = o1.lookup(q)
+    np.testing.assert_array_equal(found.cpu().numpy(), ef)
+    np.testing.assert_array_equal(g.to_numpy_u32(val), ev)
+    lsm.close()
