@@ -625,6 +625,35 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
   const bool act = lane < uint32_t(nl);
   const uint32_t* keys = act ? ls.keys[lane] : nullptr;
   uint32_t done = 0;
+  if (nl == 1) {  // nothing to look for in other levels: the window is read through, in order
+    const uint32_t last = __shfl_sync(0xffffffffu, end, 0), lt = lanemask_lt();
+    uint32_t before = 0xFFFFFFFFu;  // key before the chunk
+    for (uint32_t i0 = __shfl_sync(0xffffffffu, pos, 0); i0 < last;) {
+      uint32_t kv[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i = i0 + 32 * j + lane;
+        kv[j] = i < last ? __ldg(ls.keys[0] + i) : 0xFFFFFFFEu;  // (no regular element)
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t k = key_of(kv[j]), up = __shfl_up_sync(0xffffffffu, k, 1);
+        const bool ok = (kv[j] & 1u) && k != (lane ? up : before);
+        before = __shfl_sync(0xffffffffu, k, 31);
+        const uint32_t m = __ballot_sync(0xffffffffu, ok), at = done + __popc(m & lt);
+        if (kEmit && ok && at < room) {
+          out_k[at] = k;
+          out_v[at] = __ldg(ls.vals[0] + (i0 + 32 * j + lane));
+        }
+        done += __popc(m);
+      }
+      i0 += 128;
+      // a long run of one key (a short batch's padding): past its end
+      if (i0 < last && __shfl_sync(0xffffffffu, key_of(kv[0]), 0) == before)
+        i0 = upper_bound_key(ls.keys[0], i0, last, before);
+    }
+    return done;
+  }
   for (;;) {
     const uint32_t left = act ? end - pos : 0u;
     const uint32_t total = warp_sum(left);
