@@ -208,8 +208,9 @@ lsm_status lsm_cleanup(lsm_t* h, void* stream);
  * last occurrence of a key wins), laid out as a cleanup leaves the levels
  * (the live pairs sorted, filling the set bits of r = ceil(n'/b), placebos
  * after them).  One stable sort of all n pairs (the paper's bulk build, §V)
- * and the cleanup's compaction; needs temporary device memory of about
- * 18 bytes per pair.  Synchronises.
+ * and the cleanup's compaction; uses the cleanup's scratch and a quarter of a
+ * byte per pair and pass beside it, allocated on first use and kept.
+ * Synchronises.
  * Errors: LSM_ERR_ARG (not empty), LSM_ERR_FULL (n > capacity),
  * LSM_ERR_KEY_RANGE, LSM_ERR_OOM, LSM_ERR_CUDA.
  */

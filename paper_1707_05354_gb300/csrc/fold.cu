@@ -1015,9 +1015,102 @@ __global__ void __launch_bounds__(256) distribute(DistributeArgs a) {
   }
 }
 
+// Cleanup of one sorted run (a bulk build's sorted pairs, or a single full
+// level): nothing is merged, so the run is read twice instead, once for the
+// number of kept elements per tile (keys alone), once to write them at their
+// final places, which the scanned counts give: bound by HBM (12 B read and 8 B
+// written per pair).
+constexpr int kPlaceTile = 4096, kPlaceChunks = kPlaceTile / (4 * kThreads);
+
+// Bits e of the elements i0 + e, e < 4, of the run that are kept: the first
+// element of a key, when regular.
+__device__ __forceinline__ uint32_t keep_bits(const uint32_t* keys, uint64_t i0, uint64_t n, uint4& w) {
+  if (i0 >= n) return 0u;
+  w = __ldg(reinterpret_cast<const uint4*>(keys + i0));  // (slack is readable)
+  const uint32_t kv[4] = {w.x, w.y, w.z, w.w};
+  uint32_t prev = i0 ? key_of(__ldg(keys + i0 - 1)) : 0xFFFFFFFFu, bits = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if (i0 + e < n && (kv[e] & 1u) && key_of(kv[e]) != prev) bits |= 1u << e;
+    prev = key_of(kv[e]);
+  }
+  return bits;
+}
+
+__global__ void __launch_bounds__(kThreads) place_count(const uint32_t* __restrict__ keys, uint64_t n,
+                                                        uint32_t* __restrict__ tile_keep) {
+  __shared__ uint32_t s_scan[kThreads / 32];
+  const uint64_t t0 = uint64_t(blockIdx.x) * kPlaceTile + threadIdx.x * 4;
+  uint32_t c = 0;
+#pragma unroll
+  for (int j = 0; j < kPlaceChunks; ++j) {
+    uint4 w;
+    c += uint32_t(__popc(keep_bits(keys, t0 + j * 4 * kThreads, n, w)));
+  }
+  uint32_t all;
+  block_excl_scan<kThreads>(c, s_scan, all);
+  if (threadIdx.x == 0) tile_keep[blockIdx.x] = all;
+}
+
+// Writes the kept elements (offset[t] of them before tile t) and the
+// placebos to the places that `a` gives.
+__global__ void __launch_bounds__(kThreads) place_write(const uint32_t* __restrict__ keys,
+                                                        const uint32_t* __restrict__ vals, uint64_t n,
+                                                        const uint64_t* __restrict__ offset, DistributeArgs a) {
+  __shared__ uint32_t s_k[kPlaceTile], s_v[kPlaceTile];
+  __shared__ uint64_t s_scan[kThreads / 32];
+  const uint32_t tid = threadIdx.x;
+  const uint64_t t0 = uint64_t(blockIdx.x) * kPlaceTile + tid * 4;
+  uint4 k[kPlaceChunks], v[kPlaceChunks];
+  uint32_t bits[kPlaceChunks];
+  uint64_t mine = 0;  // kept elements per chunk, 16 bits each
+  static_assert(kPlaceChunks == 4 && 4 * kThreads < 65536, "four chunk counts in a word");
+#pragma unroll
+  for (int j = 0; j < kPlaceChunks; ++j) {
+    const uint64_t i0 = t0 + j * 4 * kThreads;
+    bits[j] = keep_bits(keys, i0, n, k[j]);
+    if (bits[j]) v[j] = __ldg(reinterpret_cast<const uint4*>(vals + i0));
+    mine += uint64_t(__popc(bits[j])) << (16 * j);
+  }
+  uint64_t all;
+  const uint64_t before = block_excl_scan<kThreads, uint64_t>(mine, s_scan, all);
+  uint32_t kept = 0;
+#pragma unroll
+  for (int j = 0; j < kPlaceChunks; ++j) {
+    uint32_t at = kept + (uint32_t(before >> (16 * j)) & 0xFFFFu);
+    const uint32_t kk[4] = {k[j].x, k[j].y, k[j].z, k[j].w}, vv[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if ((bits[j] >> e) & 1u) {
+        s_k[at] = kk[e];
+        s_v[at++] = vv[e];
+      }
+    }
+    kept += uint32_t(all >> (16 * j)) & 0xFFFFu;
+  }
+  __syncthreads();
+  const uint64_t first = offset[blockIdx.x];
+  int l = 0;
+  for (uint32_t i = tid; i < kept; i += kThreads) {
+    const uint64_t g = first + i;
+    while (l + 1 < a.nlevels && g >= a.level_start[l + 1]) ++l;
+    const uint64_t dst = a.level_off[l] + (g - a.level_start[l]);
+    a.keys[dst] = s_k[i];
+    a.vals[dst] = s_v[i];
+  }
+  l = 0;
+  for (uint64_t g = a.n_live + uint64_t(blockIdx.x) * kThreads + tid; g < a.total; g += uint64_t(gridDim.x) * kThreads) {
+    while (l + 1 < a.nlevels && g >= a.level_start[l + 1]) ++l;
+    const uint64_t dst = a.level_off[l] + (g - a.level_start[l]);
+    a.keys[dst] = kPlaceboKv;
+    a.vals[dst] = 0u;
+  }
+}
+
 // Prefix index of a sorted run: the element at position i owns the entries
 // between the bin of element i - 1 and its own; the first and last elements
-// record the populated bin range.
+// record the populated bin range.  Four elements a thread from one 16-byte
+// load (n = 32 million: 101 -> 74 us).
 __global__ void __launch_bounds__(256) build_fence(const uint32_t* __restrict__ keys, uint32_t n,
                                                    uint32_t* __restrict__ fence, int fshift) {
   __shared__ uint32_t s_ngap;
@@ -1025,15 +1118,20 @@ __global__ void __launch_bounds__(256) build_fence(const uint32_t* __restrict__ 
   if (threadIdx.x == 0) s_ngap = 0;
   __syncthreads();
   const uint32_t nb = fence_bins(fshift);
-  for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < n; i += uint64_t(gridDim.x) * 256ull) {
-    const uint32_t bin = fence_bin(__ldg(keys + i), fshift);
-    if (i == 0) {
-      fence[nb + 2] = bin;
-    } else {
-      const uint32_t pb = fence_bin(__ldg(keys + i - 1), fshift);
-      if (bin > pb) fence_write_gap(fence, pb, bin, uint32_t(i), s_gaps, &s_ngap);
+  for (uint64_t i0 = (blockIdx.x * 256ull + threadIdx.x) * 4; i0 < n; i0 += uint64_t(gridDim.x) * 1024ull) {
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(keys + i0));  // (slack is readable)
+    const uint32_t kv[4] = {w.x, w.y, w.z, w.w};
+    uint32_t pb = i0 ? fence_bin(__ldg(keys + i0 - 1), fshift) : fence_bin(kv[0], fshift);
+    if (i0 == 0) fence[nb + 2] = pb;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (i0 + e < n) {
+        const uint32_t bin = fence_bin(kv[e], fshift);
+        if (bin > pb) fence_write_gap(fence, pb, bin, uint32_t(i0) + e, s_gaps, &s_ngap);
+        pb = bin;
+        if (i0 + e + 1 == n) fence[nb + 3] = bin;
+      }
     }
-    if (i + 1 == n) fence[nb + 3] = bin;
   }
   __syncthreads();
   fence_fill_gaps(fence, s_gaps, s_ngap);
@@ -1148,8 +1246,25 @@ cudaError_t distribute_launch(const DistributeArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+uint64_t place_tiles(uint64_t n) { return (n + kPlaceTile - 1) / kPlaceTile; }
+
+cudaError_t place_count_launch(const uint32_t* keys, uint64_t n, uint32_t* tile_keep, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  count_launches(1);
+  place_count<<<unsigned(place_tiles(n)), kThreads, 0, st>>>(keys, n, tile_keep);
+  return cudaGetLastError();
+}
+
+cudaError_t place_write_launch(const uint32_t* keys, const uint32_t* vals, uint64_t n, const uint64_t* offset,
+                               const DistributeArgs& a, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  count_launches(1);
+  place_write<<<unsigned(place_tiles(n)), kThreads, 0, st>>>(keys, vals, n, offset, a);
+  return cudaGetLastError();
+}
+
 cudaError_t build_fence_launch(const uint32_t* keys, uint32_t n, uint32_t* fence, int fshift, cudaStream_t st) {
-  uint64_t blocks = (uint64_t(n) + 1 + 255) / 256;
+  uint64_t blocks = (uint64_t(n) + 1023) / 1024;
   if (blocks > 152 * 8) blocks = 152 * 8;
   count_launches(1);
   build_fence<<<unsigned(blocks), 256, 0, st>>>(keys, n, fence, fshift);

@@ -99,6 +99,10 @@ struct lsm_t {
   uint32_t* d_cv = nullptr;
   uint64_t* d_clb = nullptr;
   uint64_t clean_cap = 0;
+  // bulk build's look-back words (allocated by the first one, kept)
+  uint64_t* d_blb = nullptr;
+  uint64_t blb_tiles = 0;
+  uint32_t blb_epoch = 0;
   // query scratch (grown on demand)
   unsigned char* d_q = nullptr;
   size_t q_bytes = 0;
@@ -164,7 +168,7 @@ cudaError_t dalloc(T** p, uint64_t count) {
 
 void free_all(lsm_t* h) {
   void* dptrs[] = {h->d_keys, h->d_vals, h->d_bk, h->d_bv, h->d_tk, h->d_tv, h->sws.ctl, h->sws.lookback,
-                   h->sws.tilecnt, h->d_part, h->d_fence, h->d_misc, h->d_u64, h->d_ck, h->d_cv, h->d_clb,
+                   h->sws.tilecnt, h->d_part, h->d_fence, h->d_misc, h->d_u64, h->d_ck, h->d_cv, h->d_clb, h->d_blb,
                    h->d_q, h->qsws.lookback, h->qsws.tilecnt, h->d_qctl};
   for (void* p : dptrs)
     if (p) cudaFree(p);
@@ -549,7 +553,10 @@ lsm_status lsm_create(lsm_t** out, uint32_t b, uint64_t max_elements, int device
   h->capacity = off[L];
   const uint64_t bpad = round_up(b, kLevelAlign) + kSlack;
   const uint32_t sort_tiles = (b + kSortTile - 1) / kSortTile;
+  // co-ranks of a fold, or a single run's offsets and counts (rebuild)
   h->part_words = (fold_tiles(h->capacity) + 2) * (L + 1);
+  const uint64_t pt = place_tiles(h->capacity), place_words = 2 * (pt + 1) + 2 * scan_tiles(pt) + pt;
+  if (h->part_words < place_words) h->part_words = place_words;
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = dalloc(&h->d_keys, h->capacity + kSlack);
   if (e == cudaSuccess) e = dalloc(&h->d_vals, h->capacity + kSlack);
@@ -743,49 +750,28 @@ lsm_status lsm_range(lsm_t* h, const uint32_t* d_k1, const uint32_t* d_k2, uint6
   return cuda_status(range_emit_launch(ls, nq, bounds, d_offsets, d_keys, d_vals, st, nullptr, wide));
 }
 
-// Rebuild of the levels from sorted sources (rank order: newest first): the
-// fold keeps the first element of every key when it is regular and compacts
-// the survivors; the n' live pairs then fill the set bits of r' = ceil(n'/b)
-// in ascending level order, with placebo tombstones after the last one
-// (§IV-E).  Synchronises with `st` (the host must learn n').
-static lsm_status rebuild(lsm_t* h, const FoldSources& src, uint64_t total, cudaStream_t st) {
-  if (h->clean_cap < total) {
-    if (h->d_ck) cudaFree(h->d_ck);
-    if (h->d_cv) cudaFree(h->d_cv);
-    if (h->d_clb) cudaFree(h->d_clb);
-    h->d_ck = h->d_cv = nullptr;
-    h->d_clb = nullptr;
-    h->clean_cap = 0;
-    const uint64_t cap = h->capacity;  // enough for any later cleanup too
-    LSM_TRY(dalloc(&h->d_ck, cap + kSlack));
-    LSM_TRY(dalloc(&h->d_cv, cap + kSlack));
-    LSM_TRY(dalloc(&h->d_clb, fold_tiles(cap) + 1));
-    h->clean_cap = cap;
-  }
-  FoldArgs f{};
-  f.src = src;
-  f.total = total;
-  f.out_keys = h->d_ck;
-  f.out_vals = h->d_cv;
-  f.part = h->d_part;
-  f.status = h->d_misc + kMiscSticky;
-  f.cleanup = true;
-  f.lookback = h->d_clb;
-  f.tile_ctr = h->d_misc + kMiscCtrA;
-  f.out_count = h->d_u64;
-  {
-    ProfScope ps(h, LSM_PROF_CLEANUP, 8.0 * double(total), st);
-    LSM_TRY(fold_launch(f, st));
-  }
-  LSM_TRY(cudaMemcpyAsync(h->h_u64, h->d_u64, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-  LSM_TRY(cudaStreamSynchronize(st));
-  const uint64_t n_live = *h->h_u64;
-  if (n_live > total) return LSM_ERR_CUDA;
+// Cleanup scratch for every run the handle can hold, kept once allocated.
+static cudaError_t ensure_clean(lsm_t* h) {
+  if (h->clean_cap >= h->capacity) return cudaSuccess;
+  if (h->d_ck) cudaFree(h->d_ck);
+  if (h->d_cv) cudaFree(h->d_cv);
+  if (h->d_clb) cudaFree(h->d_clb);
+  h->d_ck = h->d_cv = nullptr;
+  h->d_clb = nullptr;
+  h->clean_cap = 0;
+  const uint64_t cap = h->capacity;
+  cudaError_t e = dalloc(&h->d_ck, cap + kSlack);
+  if (e == cudaSuccess) e = dalloc(&h->d_cv, cap + kSlack);
+  if (e == cudaSuccess) e = dalloc(&h->d_clb, fold_tiles(cap) + 1);
+  if (e == cudaSuccess) h->clean_cap = cap;
+  return e;
+}
+
+// Where n' live pairs and the placebos after them go: the set bits of r' =
+// ceil(n'/b) in ascending level order (§IV-E).
+static DistributeArgs level_places(const lsm_t* h, uint64_t n_live) {
   const uint64_t r2 = (n_live + h->b - 1) / h->b;
-  h->l0_buf = -1;  // every level is rewritten in the level array
   DistributeArgs d{};
-  d.src_keys = h->d_ck;
-  d.src_vals = h->d_cv;
   d.n_live = n_live;
   d.keys = h->d_keys;
   d.vals = h->d_vals;
@@ -797,9 +783,69 @@ static lsm_status rebuild(lsm_t* h, const FoldSources& src, uint64_t total, cuda
     d.level_size[d.nlevels] = uint64_t(h->b) << i;
     ++d.nlevels;
   }
+  return d;
+}
+
+// Rebuild of the levels from sorted sources (rank order: newest first): the
+// first element of every key is kept when it is regular; the n' live pairs
+// then fill the set bits of r' in ascending level order, with placebo
+// tombstones after the last one (§IV-E).  Several sources are folded into the
+// cleanup scratch and copied from there; a single one is counted and written
+// at once, to the levels themselves when it lies in the scratch (a bulk
+// build's sorted pairs), else by way of the scratch (it is a level).
+// Synchronises with `st` (the host must learn n').
+static lsm_status rebuild(lsm_t* h, const FoldSources& src, uint64_t total, cudaStream_t st) {
+  const bool single = src.count == 1, direct = single && src.keys[0] == h->d_ck;
+  LSM_TRY(ensure_clean(h));
+  // a single source's offsets and counts per tile, in the co-rank table
+  const uint64_t tiles = place_tiles(total);
+  uint64_t* offset = reinterpret_cast<uint64_t*>(h->d_part);
+  uint64_t* lookback = offset + tiles + 1;
+  uint32_t* tile_keep = reinterpret_cast<uint32_t*>(lookback + scan_tiles(tiles));
+  {
+    ProfScope ps(h, LSM_PROF_CLEANUP, 8.0 * double(total), st);
+    if (single) {
+      LSM_TRY(place_count_launch(src.keys[0], total, tile_keep, st));
+      LSM_TRY(scan_launch(tile_keep, tiles, offset, lookback, h->d_misc + kMiscCtrB, h->d_misc + kMiscSticky, st));
+    } else {
+      FoldArgs f{};
+      f.src = src;
+      f.total = total;
+      f.out_keys = h->d_ck;
+      f.out_vals = h->d_cv;
+      f.part = h->d_part;
+      f.status = h->d_misc + kMiscSticky;
+      f.cleanup = true;
+      f.lookback = h->d_clb;
+      f.tile_ctr = h->d_misc + kMiscCtrA;
+      f.out_count = h->d_u64;
+      LSM_TRY(fold_launch(f, st));
+    }
+  }
+  LSM_TRY(cudaMemcpyAsync(h->h_u64, single ? offset + tiles : h->d_u64, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+  LSM_TRY(cudaStreamSynchronize(st));
+  const uint64_t n_live = *h->h_u64;
+  if (n_live > total) return LSM_ERR_CUDA;
+  const uint64_t r2 = (n_live + h->b - 1) / h->b;
+  h->l0_buf = -1;  // every level is rewritten in the level array
+  DistributeArgs d = level_places(h, n_live);
+  d.src_keys = h->d_ck;
+  d.src_vals = h->d_cv;
   {
     ProfScope ps(h, LSM_PROF_CLEANUP, 8.0 * double(d.total), st);
-    LSM_TRY(distribute_launch(d, st));
+    if (direct) {
+      LSM_TRY(place_write_launch(src.keys[0], src.vals[0], total, offset, d, st));
+    } else {
+      if (single) {
+        DistributeArgs flat{};
+        flat.n_live = flat.total = n_live;
+        flat.keys = h->d_ck;
+        flat.vals = h->d_cv;
+        flat.nlevels = 1;
+        LSM_TRY(place_write_launch(src.keys[0], src.vals[0], total, offset, flat, st));
+      }
+      LSM_TRY(distribute_launch(d, st));
+    }
     for (uint32_t i = 0; i < h->L; ++i)
       if ((r2 >> i) & 1u)
         LSM_TRY(build_fence_launch(level_keys(h, i), h->b << i, level_fence(h, i), h->fshift[i], st));
@@ -835,62 +881,48 @@ lsm_status lsm_bulk_build(lsm_t* h, const uint32_t* d_keys, const uint32_t* d_va
   DeviceGuard g(h->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   LSM_TRY(join_side(h, st));
-  // one stable sort of the whole reversed input (the last occurrence of a key
-  // first), with its prefix index, into temporary buffers
-  const uint64_t npad = round_up(n, kLevelAlign) + kSlack;
+  // One stable sort of the whole reversed input (the last occurrence of a key
+  // first) into the cleanup scratch, with the empty levels' memory as its
+  // other half; nothing is allocated once scratch and look-back words are.
+  LSM_TRY(ensure_clean(h));
   const uint64_t tiles = (n + kSortTile - 1) / kSortTile;
-  const int fs = fence_shift_for(n);
-  uint32_t *buf = nullptr, *ctl = nullptr, *tilecnt = nullptr;
-  uint64_t* lookback = nullptr;
-  lsm_status result = LSM_OK;
-  cudaError_t e = dalloc(&buf, 4 * npad + fence_words(fs));
-  if (e == cudaSuccess) e = dalloc(&ctl, 2 * kSortCtlWords);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 0, 4ull * 2 * kSortCtlWords, st);
-  if (e == cudaSuccess) e = dalloc(&tilecnt, kMsdRunWords);
-  if (e == cudaSuccess) e = dalloc(&lookback, uint64_t(kSortPasses) * tiles * 256);
-  if (e == cudaSuccess) e = cudaMemsetAsync(lookback, 0, 8ull * kSortPasses * tiles * 256, st);
-  if (e == cudaSuccess) {
-    SortWorkspace ws{};
-    ws.ctl = ctl;
-    ws.flip = 0;
-    ws.lookback = lookback;
-    ws.max_tiles = uint32_t(tiles);
-    ws.epoch = 0;
-    ws.sticky = h->d_misc + kMiscSticky;
-    ws.tilecnt = tilecnt;
-    SortArgs a{};
-    a.mode = kSortInsert;
-    a.in_keys = d_keys;
-    a.in_vals = d_vals;
-    a.n_in = n;
-    a.n = uint32_t(n);
-    a.out_keys = buf;
-    a.out_vals = buf + npad;
-    a.tmp_keys = buf + 2 * npad;
-    a.tmp_vals = buf + 3 * npad;
-    a.fence = buf + 4 * npad;
-    a.fshift = fs;
-    const uint32_t seq = next_check(h);
-    e = sort_launch(a, ws, st, h->d_status_map, seq);
-    if (e == cudaSuccess) result = wait_check(h, seq, st);
-    if (e == cudaSuccess && result == LSM_OK) {
-      FoldSources src{};
-      src.count = 1;
-      src.keys[0] = a.out_keys;
-      src.vals[0] = a.out_vals;
-      src.fence[0] = a.fence;
-      src.fshift[0] = fs;
-      src.n[0] = uint32_t(n);
-      result = rebuild(h, src, n, st);
-    }
+  if (!h->d_blb || h->blb_tiles < tiles) {
+    if (h->d_blb) cudaFree(h->d_blb);
+    h->d_blb = nullptr;
+    h->blb_tiles = 0;
+    LSM_TRY(dalloc(&h->d_blb, uint64_t(kSortPasses) * tiles * 256));
+    h->blb_tiles = tiles;
+    h->blb_epoch = 0;
+    LSM_TRY(cudaMemsetAsync(h->d_blb, 0, 8ull * kSortPasses * tiles * 256, st));
   }
-  cudaStreamSynchronize(st);
-  if (buf) cudaFree(buf);
-  if (ctl) cudaFree(ctl);
-  if (tilecnt) cudaFree(tilecnt);
-  if (lookback) cudaFree(lookback);
-  if (e != cudaSuccess) return cuda_status(e);
-  return result;
+  // the batch sort's control words and run table, with look-back words for n
+  SortWorkspace ws = h->sws;
+  ws.lookback = h->d_blb;
+  ws.max_tiles = uint32_t(h->blb_tiles);
+  ws.epoch = h->blb_epoch;
+  SortArgs a{};
+  a.mode = kSortInsert;
+  a.in_keys = d_keys;
+  a.in_vals = d_vals;
+  a.n_in = n;
+  a.n = uint32_t(n);
+  a.out_keys = h->d_ck;
+  a.out_vals = h->d_cv;
+  a.tmp_keys = h->d_keys;
+  a.tmp_vals = h->d_vals;
+  const uint32_t seq = next_check(h);
+  const cudaError_t e = sort_launch(a, ws, st, h->d_status_map, seq);
+  h->sws.flip = ws.flip;
+  h->blb_epoch = ws.epoch;
+  LSM_TRY(e);
+  const lsm_status s = wait_check(h, seq, st);
+  if (s != LSM_OK) return s;
+  FoldSources src{};
+  src.count = 1;
+  src.keys[0] = a.out_keys;
+  src.vals[0] = a.out_vals;
+  src.n[0] = uint32_t(n);
+  return rebuild(h, src, n, st);
 }
 
 lsm_status lsm_stats(const lsm_t* h, uint64_t* r, uint64_t* resident, uint32_t* b, uint32_t* levels) {

@@ -211,6 +211,15 @@ struct DistributeArgs {
 };
 cudaError_t distribute_launch(const DistributeArgs& a, cudaStream_t st);
 
+// The cleanup of one sorted run (16-byte aligned, readable slack after it):
+// kept elements per tile, to be scanned into offset[0 .. place_tiles(n)], and
+// the kept elements with the placebos to the places that `a` gives (its source
+// pointers are not used).
+uint64_t place_tiles(uint64_t n);
+cudaError_t place_count_launch(const uint32_t* keys, uint64_t n, uint32_t* tile_keep, cudaStream_t st);
+cudaError_t place_write_launch(const uint32_t* keys, const uint32_t* vals, uint64_t n, const uint64_t* offset,
+                               const DistributeArgs& a, cudaStream_t st);
+
 // ------------------------------------------------------ many dictionaries ---
 // The batched form: n independent dictionaries, each with its own batch size
 // b_i and levels b_i * 2^l, advanced together.  A round gives every instance

@@ -170,3 +170,40 @@ def test_small_batches(g, dist, b):
     np.testing.assert_array_equal(found.cpu().numpy(), ef)
     np.testing.assert_array_equal(g.to_numpy_u32(val), ev)
     lsm.close()
+
+
+@pytest.mark.parametrize("n", [1, 4095, 4096, 4097, 13 * 4096 + 5, (1 << 20) + 3])
+@pytest.mark.parametrize("dist", ["one", "ids", "zipf"])
+def test_one_run_rebuilds(g, dist, n):
+    """Bulk builds (twice, the second with the kept scratch) and cleanups of a single full level: the run is counted
+    and written tile by tile.  Levels against the structural oracle."""
+    b, rng = max(1, n // 5), np.random.default_rng(n)
+    lsm = g.LSM(b, 8 * b + n)
+    for _ in range(2):
+        g.lsm_reset(lsm.h)
+        k, v = draw(dist, n, rng), rng.integers(0, 1 << 31, n).astype(np.uint32)
+        lsm.bulk_build(k, v)
+        s = oracle.StructuralOracle(b)
+        s.call("insert", k, v)
+        s.cleanup()
+        assert lsm.r == s.r
+        for i, (kv, vv) in lsm.levels().items():
+            ekv, ev = s.level(i)
+            np.testing.assert_array_equal(kv, ekv)
+            np.testing.assert_array_equal(vv, ev)
+    g.lsm_reset(lsm.h)
+    s = oracle.StructuralOracle(b)
+    for t in range(2):   # two batches: one full level with deletes and old versions
+        k, v = draw(dist, b, rng), rng.integers(0, 1 << 31, b).astype(np.uint32)
+        d = (rng.random(b) < 0.4).astype(np.uint8)
+        lsm.update(k, v, d)
+        s.call("update", k, v, d)
+    lsm.cleanup()
+    s.cleanup()
+    assert lsm.r == s.r
+    for i, (kv, vv) in lsm.levels().items():
+        ekv, ev = s.level(i)
+        np.testing.assert_array_equal(kv, ekv)
+        np.testing.assert_array_equal(vv, ev)
+    assert lsm.device_errors() == 0
+    lsm.close()
