@@ -156,9 +156,16 @@ struct Loader {
   template <int N, class In>
   __device__ __forceinline__ void load_items(uint32_t p0, uint32_t step, const In& in, uint32_t (&kv)[N],
                                              uint32_t (&v)[N], bool& bad) const {
+    uint32_t none;
+    load_items<false>(p0, step, in, kv, v, bad, 0u, none);
+  }
+  // The same, and the key variable of element `at`, asked for behind them.
+  template <bool kProbe, int N, class In>
+  __device__ __forceinline__ void load_items(uint32_t p0, uint32_t step, const In& in, uint32_t (&kv)[N],
+                                             uint32_t (&v)[N], bool& bad, uint32_t at, uint32_t& probe) const {
     with_mode([&](auto m) {
       constexpr int M = decltype(m)::value;
-      uint32_t fl[N];
+      uint32_t fl[N], probe_fl = 0u;
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         const uint32_t p = p0 + j * step;
@@ -169,6 +176,12 @@ struct Loader {
           v[j] = raw_val<M>(p);
         }
       }
+      if (kProbe) {
+        probe = __ldg(keys + src<M>(at));
+        probe_fl = flag<M>(src<M>(at));
+      }
+      bool b = false;  // (of another thread's element)
+      if (kProbe) probe = encode<M>(probe, probe_fl, b);
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         if (!in(p0 + j * step)) continue;
@@ -424,7 +437,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const ui
 //                CTA in parts that fit.
 // The buckets split the range of the keys that the batch holds (KeyMap), not
 // the 32 bits of the key variable: ids below 2^25 would otherwise fall in
-// four buckets and be sorted by four CTAs.
+// four buckets and be sorted by four CTAs; hot keys have buckets of their own.
 // ---------------------------------------------------------------------------
 constexpr int kBucketThreads = 512;
 constexpr int kBucketWarps = kBucketThreads / 32;
@@ -441,47 +454,134 @@ constexpr int kScatterIPT = int(kMsdTile) / kScatterThreads;  // 8
 static_assert(kScatterIPT * kScatterThreads == int(kMsdTile), "tile");
 static_assert(kMsdMaxTiles <= uint32_t(kBucketThreads), "one thread per tile run in the bucket kernel");
 
-// The buckets of one sort: bucket(kv) = floor((kv - lo) * mul / 2^32), kept
-// within [0, 255]; monotone, so bucket d holds the key variables of
-// [lower(d), lower(d + 1)).  lo and mul come from the smallest and largest of
-// 512 elements taken at even distances (every CTA of the tile kernel reads
-// the same ones), the range widened by 1/128 at both ends: for evenly spread
-// keys the widened range misses elements with a probability of about e^-5 at
-// either end, and those then fall in the first or last bucket.
+// The buckets of one sort: `parts` equal parts of the key range, part(kv) =
+// floor((kv - lo) * mul / 2^32), and, of every hot key variable, a bucket of its
+// own, which splits the part that holds it in two: 256 in all, in key order.
+// lo, mul and the hot ones come from 512 elements taken at even distances
+// (every CTA of the tile kernel reads the same ones): the range is the one
+// they span, widened by 1/128 at both ends (for evenly spread keys it then
+// misses elements with a probability of about e^-10 at either end, and those
+// fall in the first or last bucket); hot is what comes up kHotSamples times or
+// more, about 0.8 % of the batch, and would overflow a bucket of 2^20 / 256
+// elements.
 // With the top byte as the bucket, batches of 2^18 ids below 2^25 took 553 us
-// in bucket_sort and 2^20 keys below 2^30 154 us; now 21.7 and 21.3 us.
+// in bucket_sort and 2^20 keys below 2^30 154 us; now 21.7 and 21.3 us.  Without
+// buckets for the hot keys a sort of 2^18 Zipf(1.1) pairs took 63 us, of 2^20
+// 167; now 34 and 79.
+constexpr uint32_t kHotSamples = 4, kMaxHot = 32, kSamples = 512;
+constexpr uint32_t kMaxSampledHot = kSamples / kHotSamples;
+constexpr int kSampleTableLog = 10, kSampleCellsLog = 12;
+constexpr uint32_t kSampleTable = 1u << kSampleTableLog, kSampleCells = 1u << kSampleCellsLog;
 struct KeyMap {
-  uint32_t lo, mul;
-  __device__ __forceinline__ uint32_t bucket(uint32_t kv) const {
-    return min(__umulhi(max(kv, lo) - lo, mul), uint32_t(kRadix - 1));
+  uint32_t lo, mul, parts, nhot;
+  const uint32_t* hot;  // ascending, in shared memory
+  __device__ __forceinline__ uint32_t part(uint32_t kv) const {
+    return min(__umulhi(max(kv, lo) - lo, mul), parts - 1);
   }
-  // smallest key variable of bucket d in 1 .. 255 (2^32 - 1 for a bucket the
+  __device__ __forceinline__ uint32_t bucket(uint32_t kv) const {
+    uint32_t d = part(kv);
+    for (uint32_t h = 0; h < nhot; ++h) d += (kv >= hot[h] ? 1u : 0u) + (kv > hot[h] ? 1u : 0u);
+    return d;
+  }
+  // smallest key variable of part p in 1 .. parts - 1 (2^32 - 1 for a part the
   // 32 bits do not reach: key variables are below it)
-  __device__ __forceinline__ uint32_t lower(uint32_t d) const {
-    return uint32_t(min(lo + ((uint64_t(d) << 32) + mul - 1) / mul, uint64_t(0xFFFFFFFFu)));
+  __device__ __forceinline__ uint32_t lower(uint32_t p) const {
+    return uint32_t(min(lo + ((uint64_t(p) << 32) + mul - 1) / mul, uint64_t(0xFFFFFFFFu)));
+  }
+  // Stores the smallest key variable of every bucket (threads 0 .. 255).
+  __device__ __forceinline__ void bounds(uint32_t* out) const {
+    const uint32_t t = threadIdx.x;
+    if (t < parts) {
+      const uint32_t kv = t ? lower(t) : 0u;
+      uint32_t d = t;
+      for (uint32_t h = 0; h < nhot; ++h) d += hot[h] < kv ? 2u : 0u;
+      out[d] = kv;
+    }
+    if (t < nhot) {
+      const uint32_t d = part(hot[t]) + 2u * t;
+      out[d + 1] = hot[t];
+      out[d + 2] = hot[t] + 1u;
+    }
   }
 };
+static_assert(kRadix == 256 && 2 * kMaxHot < kRadix, "the hot keys' buckets leave parts over");
+static_assert(kSamples == uint32_t(kScatterThreads), "one sample a thread");
+static_assert(kSampleTable == 2 * kSamples && 2 * kSampleTable == 4 * uint32_t(kScatterThreads) &&
+                  2 * kSampleTable <= kSampleCells && kSampleCells <= uint32_t(kMsdTile), "room to count in");
 
-// Key map of the batch (every thread of a CTA of NT threads gets it).
-template <int NT>
-__device__ __forceinline__ KeyMap sample_map(const Loader& ld, uint32_t* s_min, uint32_t* s_max) {
-  static_assert(NT == 512, "one sample a thread");
-  const uint32_t npad = ld.npad(), cnt = ld.n - npad;
-  bool bad;
-  const uint32_t kv = ld.load_key(npad + uint32_t(uint64_t(threadIdx.x) * cnt / NT), bad);
+struct SampleShared {
+  uint32_t mn[kScatterWarps], mx[kScatterWarps], hot[kMaxHot], n_hot;
+};
+// Key map of the batch of cnt elements (every thread of the CTA gets it); kv:
+// the thread's sample.  First the samples are counted by a hash of theirs: for
+// most batches no cell fills up (with 4096 cells a batch of different keys
+// fills one in 30 times; 1024 would be filled nearly every time, for 1.3 us).
+// Otherwise those in a full cell are counted by key variable, in an open hash
+// table half full at most (keys in `cells`, 0 where empty, counts behind
+// them).  cells: kSampleCells words of shared memory, 16-byte aligned; list:
+// kMaxSampledHot words.  sample_begin comes first, with a barrier between.
+__device__ __forceinline__ void sample_begin(const uint32_t kv, uint32_t* cells, SampleShared& sh) {
+  const uint32_t tid = threadIdx.x, warp = tid >> 5;
+  for (uint32_t i = tid; i < kSampleCells / 4; i += kScatterThreads)
+    reinterpret_cast<uint4*>(cells)[i] = make_uint4(0u, 0u, 0u, 0u);
   const uint32_t mn = __reduce_min_sync(0xffffffffu, kv), mx = __reduce_max_sync(0xffffffffu, kv);
   if (lane_id() == 0) {
-    s_min[threadIdx.x >> 5] = mn;
-    s_max[threadIdx.x >> 5] = mx;
+    sh.mn[warp] = mn;
+    sh.mx[warp] = mx;
   }
-  __syncthreads();
-  const uint32_t w = lane_id() & uint32_t(NT / 32 - 1);
-  const uint32_t lo = __reduce_min_sync(0xffffffffu, s_min[w]), hi = __reduce_max_sync(0xffffffffu, s_max[w]);
-  const uint32_t ext = (hi - lo) / 128 + 1;
+  if (tid == 0) sh.n_hot = 0u;
+}
+__device__ __forceinline__ KeyMap sample_map(const uint32_t kv, uint32_t cnt, uint32_t* cells, uint32_t* list,
+                                             SampleShared& sh) {
+  const uint32_t tid = threadIdx.x;
+  const bool seek_hot = cnt >= 8 * kSamples;  // (else elements are sampled twice)
+  const uint32_t w = lane_id() & uint32_t(kScatterWarps - 1);
+  const uint32_t lo = __reduce_min_sync(0xffffffffu, sh.mn[w]), hi = __reduce_max_sync(0xffffffffu, sh.mx[w]);
+  uint32_t nhot = 0;
+  if (seek_hot) {
+    const uint32_t hash = kv * 0x9E3779B1u, cell = hash >> (32 - kSampleCellsLog);
+    atomicAdd(&cells[cell], 1u);
+    __syncthreads();
+    // (0 has nothing below it, 2^32 - 1 nothing above)
+    const bool may = cells[cell] >= kHotSamples && kv != 0u && kv != 0xFFFFFFFFu;
+    if (__syncthreads_or(may)) {
+      uint32_t *table = cells, *count = cells + kSampleTable, at = hash >> (32 - kSampleTableLog);
+      reinterpret_cast<uint4*>(cells)[tid] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+      bool first = false;  // the sample that entered its key variable
+      if (may) {
+        for (;;) {
+          uint32_t was = reinterpret_cast<volatile uint32_t*>(table)[at];
+          if (was == 0u) {
+            was = atomicCAS(&table[at], 0u, kv);
+            first = was == 0u;
+          }
+          if (first || was == kv) break;
+          at = (at + 1u) & (kSampleTable - 1u);
+        }
+        atomicAdd(&count[at], 1u);
+      }
+      __syncthreads();
+      if (first && count[at] >= kHotSamples) list[atomicAdd(&sh.n_hot, 1u)] = kv;
+      __syncthreads();
+      // at most kMaxSampledHot of them, of which the kMaxHot lowest are taken, in order
+      nhot = sh.n_hot;
+      if (tid < nhot) {
+        const uint32_t x = list[tid];
+        uint32_t r = 0;
+        for (uint32_t i = 0; i < nhot; ++i) r += list[i] < x ? 1u : 0u;
+        if (r < kMaxHot) sh.hot[r] = x;
+      }
+      nhot = min(nhot, kMaxHot);
+      __syncthreads();
+    }
+  }
+  const uint32_t ext = (hi - lo) / 128 + 1, parts = uint32_t(kRadix) - 2u * nhot;
   const uint32_t l = lo > ext ? lo - ext : 0u, h = hi < ~ext ? hi + ext : 0xFFFFFFFFu;
-  // (a float quotient: any factor near 2^40 / range does, the same in every
-  // CTA; the conversion saturates)
-  return KeyMap{l, max(1u, __float2uint_rd(__fdividef(1099511627776.0f, float(h - l) + 1.0f)))};
+  // (a float quotient: any factor near parts * 2^32 / range does, the same in
+  // every CTA; the conversion saturates)
+  const float q = __fdividef(float(parts) * 4294967296.0f, float(h - l) + 1.0f);
+  return KeyMap{l, max(1u, __float2uint_rd(q)), parts, nhot, sh.hot};
 }
 
 // Stable in-shared-memory rank of up to IPT items per thread of a warp-striped
@@ -537,43 +637,67 @@ __device__ __forceinline__ void rank_block(const uint32_t (&kv)[IPT], uint32_t m
 // one run of equal elements, added to its bucket's total here and written by
 // that bucket's sort at its sorted place.  A tile of padding only still
 // writes its (empty) runs.
-__global__ void __launch_bounds__(kScatterThreads) msd_tile(Loader ld, uint32_t* __restrict__ tmp_k,
+// 48 registers (a few spills): with the 62 that the compiler would take, fewer
+// CTAs find room beside those of the fold before them, and 128 inserts of
+// 2^20 took 1 to 2 % longer.
+__global__ void __maxnreg__(48) msd_tile(Loader ld, uint32_t* __restrict__ tmp_k,
                                                      uint32_t* __restrict__ tmp_v, uint2* __restrict__ runs,
                                                      uint32_t* ctl, KeyCheck check) {
   __shared__ __align__(16) uint32_t s_keys[kMsdTile];
   __shared__ __align__(16) uint32_t s_vals[kMsdTile];
   __shared__ uint32_t s_whist[kScatterWarps][kRadix];
   __shared__ uint32_t s_excl[kRadix], s_cnt[kRadix], s_scan[kScatterWarps];
+  __shared__ SampleShared s_sample;
   pdl_trigger();
   pdl_wait();
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, tile = blockIdx.x;
   const uint32_t n = ld.n, npad = ld.npad();
   const uint32_t t0 = tile * kMsdTile;
   const uint32_t base = t0 + warp * (32 * kScatterIPT);
-  uint32_t kv[kScatterIPT], v[kScatterIPT], rank[kScatterIPT];
+  uint32_t kv[kScatterIPT], v[kScatterIPT];
   bool bad_any = false;
-  ld.load_items(base + lane, 32u, [&](uint32_t p) { return p < n && p >= npad; }, kv, v, bad_any);
+  uint32_t sample;
+  ld.load_items<true>(base + lane, 32u, [&](uint32_t p) { return p < n && p >= npad; }, kv, v, bad_any,
+                      npad + uint32_t(uint64_t(tid) * (n - npad) / kSamples), sample);
+  sample_begin(sample, s_keys, s_sample);
   const int any_bad = __syncthreads_or(bad_any);
   if (tid == 0) check.done(ctl, any_bad != 0);
-  const KeyMap map = sample_map<kScatterThreads>(ld, s_cnt, s_cnt + kScatterWarps);
-  if (tile == gridDim.x - 1) {  // the last tile's CTA (the shortest) publishes the map and the buckets' bounds
-    if (tid < kRadix) ctl[kSortCtlBounds + tid] = tid ? map.lower(tid) : 0u;
+  const KeyMap map = sample_map(sample, n - npad, s_keys, s_vals, s_sample);
+  if (tile == gridDim.x - 1) {  // the last tile's CTA (the shortest) publishes the buckets' bounds
+    map.bounds(ctl + kSortCtlBounds);
     if (tid == kRadix) {
       ctl[kSortCtlMap] = map.lo;
       ctl[kSortCtlMap + 1] = map.mul;
     }
   }
-  rank_block<kScatterThreads, kScatterIPT>(kv, n, base, [&](uint32_t k) { return map.bucket(k); }, rank, s_whist,
-                                           s_excl, s_scan, s_cnt, npad);
+  // ranked and put in order in shared memory; digit(x[j]) is element j's bucket
+  const auto place = [&](const uint32_t (&x)[kScatterIPT], const auto& digit) {
+    uint32_t rank[kScatterIPT];
+    rank_block<kScatterThreads, kScatterIPT>(x, n, base, digit, rank, s_whist, s_excl, s_scan, s_cnt, npad);
 #pragma unroll
-  for (int j = 0; j < kScatterIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    if (p < n && p >= npad) {
-      const uint32_t d = map.bucket(kv[j]);
-      const uint32_t pos = s_excl[d] + s_whist[warp][d] + rank[j];
-      s_keys[pos] = kv[j];
-      s_vals[pos] = v[j];
+    for (int j = 0; j < kScatterIPT; ++j) {
+      const uint32_t p = base + j * 32 + lane;
+      if (p < n && p >= npad) {
+        const uint32_t d = digit(x[j]);
+        const uint32_t pos = s_excl[d] + s_whist[warp][d] + rank[j];
+        s_keys[pos] = kv[j];
+        s_vals[pos] = v[j];
+      }
     }
+  };
+  if (map.nhot == 0) {
+    place(kv, [&](uint32_t k) { return map.part(k); });
+  } else {
+    uint32_t dig[kScatterIPT];
+#pragma unroll
+    for (int j = 0; j < kScatterIPT; ++j) dig[j] = map.part(kv[j]);
+#pragma unroll 1
+    for (uint32_t h = 0; h < map.nhot; ++h) {
+      const uint32_t x = map.hot[h];
+#pragma unroll
+      for (int j = 0; j < kScatterIPT; ++j) dig[j] += (kv[j] >= x ? 1u : 0u) + (kv[j] > x ? 1u : 0u);
+    }
+    place(dig, [](uint32_t d) { return d; });
   }
   __syncthreads();
   const uint32_t lo_t = t0 > npad ? t0 : npad, hi_t = (n - t0) < kMsdTile ? n : t0 + kMsdTile;
@@ -885,6 +1009,33 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
                                       const PadRun pad, uint32_t* bsm, BucketShared& sh) {
   constexpr uint32_t kItems = 8, kChunk = kItems * kBucketThreads;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  if (range.lo == range.hi) {  // a hot key's bucket: its elements in order, after the padding if that is of the key
+    const uint32_t base = start + pad.n;
+    for (uint32_t j = tid; j < pad.n; j += kBucketThreads) {
+      out_k[start + j] = pad.kv;
+      out_v[start + j] = pad.v;
+    }
+    constexpr uint32_t kFar = 24;  // loads in flight (one CTA copies 3.3 elements a nanosecond)
+    uint32_t t = 0;
+    for (uint32_t i0 = 0; i0 < m; i0 += kFar * kBucketThreads) {
+      uint32_t v[kFar];
+#pragma unroll
+      for (uint32_t j = 0; j < kFar; ++j) {
+        const uint32_t i = i0 + j * kBucketThreads + tid;
+        v[j] = i < m ? src_v[src.seek(i, t)] : 0u;
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < kFar; ++j) {
+        const uint32_t i = i0 + j * kBucketThreads + tid;
+        if (i < m) {
+          out_k[base + i] = range.lo;
+          out_v[base + i] = v[j];
+        }
+      }
+    }
+    __syncthreads();  // the caller reads the output back
+    return;
+  }
   uint32_t* cnt = &sh.whist[0][0];
   const auto shift = [&](uint32_t kv) { return pad.n && kv >= pad.kv ? pad.n : 0u; };
   // f(kv, valid) for every element, whole warps at a time, in no order
@@ -1293,7 +1444,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
   // before the bucket, its start in the output
   const uint2 run = tid < ntiles ? runs[d * kMsdMaxTiles + tid] : make_uint2(0u, 0u);
   const uint32_t before = tid < d ? ctl[3 * kRadix + tid] : 0u;
-  const KeyMap map{ctl[kSortCtlMap], ctl[kSortCtlMap + 1]};
+  const uint32_t map_lo = ctl[kSortCtlMap], map_mul = ctl[kSortCtlMap + 1];
   const bool top = d == kRadix - 1;
   const uint32_t lo = ctl[kSortCtlBounds + d], next = top ? 0xFFFFFFFFu : ctl[kSortCtlBounds + d + 1];
   const uint32_t hi = next == 0xFFFFFFFFu ? next : next - 1;
@@ -1314,7 +1465,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
   if (pad.n) {
     bool bad;
     ld.load(0, pad.kv, pad.v, bad);
-    if (map.bucket(pad.kv) != d) pad.n = 0;
+    if (pad.kv < lo || pad.kv > hi || hi < lo) pad.n = 0;
   }
   const uint32_t total = m + pad.n;
   // An empty bucket writes its bins too (they share the next element's
@@ -1327,7 +1478,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, cons
   }
   // keys below the sampled range (bucket 0) and above it (bucket 255) share
   // the sub-bins at that end
-  const BucketRange range{lo, hi, SubMap::of(d ? lo : map.lo, __fdividef(4294967296.0f, float(map.mul)) + 1.0f)};
+  const BucketRange range{lo, hi, SubMap::of(d ? lo : map_lo, __fdividef(4294967296.0f, float(map_mul)) + 1.0f)};
   const int ends = (total && start == 0 ? 1 : 0) | (total && start + total == n ? 2 : 0);
   const RunSrc src{s_rstart, s_rbase, s_chunk, ntiles};
   bucket_body(tmp_k, tmp_v, src, out_k, out_v, start, m, range, pad, bins, ends, bsm, sh);

@@ -207,3 +207,25 @@ def test_one_run_rebuilds(g, dist, n):
         np.testing.assert_array_equal(vv, ev)
     assert lsm.device_errors() == 0
     lsm.close()
+@pytest.mark.parametrize("n", [4095, 4096, 30000, 1 << 18, 1 << 20])
+@pytest.mark.parametrize("words", ["many", "ends", "runs", "pair"])
+def test_hot_words(g, words, n):
+    """Words that a sort puts in buckets of their own: more of them than it has room for, the smallest and largest
+    32-bit words, neighbours, and hot words with nothing else in the batch."""
+    rng = np.random.default_rng(n + len(words))
+    hot = {"many": 1 + rng.permutation(1 << 20)[:60] * 4093, "ends": [0, 1, 2, (1 << 32) - 3, (1 << 32) - 2, (1 << 32) - 1],
+           "runs": list(range(1 << 31, (1 << 31) + 20)), "pair": [77, 3 << 30]}[words]
+    keys = rng.choice(np.asarray(hot, np.int64), n)
+    if words != "pair":
+        keys = np.where(rng.random(n) < 0.3, rng.integers(0, 1 << 32, n), keys)
+    keys = keys.astype(np.uint32)
+    lsm = g.LSM(n, n)
+    kd, vd = g.as_device_u32(keys, 0), g.as_device_u32(np.arange(n, dtype=np.uint32), 0)
+    ko, vo = torch.zeros_like(kd), torch.zeros_like(vd)
+    g.lsm_sort_pairs(lsm.h, kd.data_ptr(), vd.data_ptr(), ko.data_ptr(), vo.data_ptr(), n,
+                     torch.cuda.current_stream().cuda_stream)
+    order = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(g.to_numpy_u32(ko), keys[order])
+    np.testing.assert_array_equal(g.to_numpy_u32(vo), order.astype(np.uint32))
+    assert lsm.device_errors() == 0
+    lsm.close()
