@@ -1501,33 +1501,53 @@ __global__ void __launch_bounds__(256) check_keys(const uint32_t* __restrict__ k
 // or refused by the prep kernel) leave at once.
 // ---------------------------------------------------------------------------
 constexpr int kMultiIPT = int(kMultiSortTile) / kThreads;  // 16
-static_assert(kMultiIPT * kThreads == int(kMultiSortTile), "tile");
+static_assert(kMultiIPT * kThreads == int(kMultiSortTile) && kScatterIPT * kScatterThreads == int(kMultiSortTile), "tile");
 
 __device__ __forceinline__ uint32_t multi_ops(const MultiBatch& in, const MultiInst& d, uint32_t i) {
   return in.counts ? __ldg(in.counts + i) : d.b;
 }
 
-// Element p (< b) of instance d's reversed padded batch: op min(b-1-p, n-1).
-__device__ __forceinline__ uint32_t multi_load_key(const MultiBatch& in, const MultiInst& d, uint32_t nops,
-                                                   uint32_t p, bool& bad) {
-  uint64_t s = uint64_t(d.b) - 1 - p;
-  if (s >= nops) s = nops - 1;
-  s += d.in_off;
-  const uint32_t k = __ldg(in.keys + s);
-  const bool is_del = in.del && __ldg(in.del + s) != 0;
-  bad = k > kMaxUserKey;
-  return bad ? kPlaceboKv : ((k << 1) | (is_del ? 0u : 1u));
-}
-__device__ __forceinline__ void multi_load(const MultiBatch& in, const MultiInst& d, uint32_t nops, uint32_t p,
-                                           uint32_t& kv, uint32_t& v) {
-  uint64_t s = uint64_t(d.b) - 1 - p;
-  if (s >= nops) s = nops - 1;
-  s += d.in_off;
-  const uint32_t k = __ldg(in.keys + s);
-  const bool is_del = in.del && __ldg(in.del + s) != 0;
-  const bool bad = k > kMaxUserKey;
-  kv = bad ? kPlaceboKv : ((k << 1) | (is_del ? 0u : 1u));
-  v = (is_del || bad || !in.vals) ? 0u : __ldg(in.vals + s);
+// Elements p0 + step j, j < N, below m of the tile at t0 of an instance's
+// reversed padded batch (element p is op min(b - 1 - p, nops - 1)): all loads
+// are issued before the first is used.  Elements outside keep kv = v = 0.
+// (One element after another, its value once its key had come, and 16 a thread
+// in mseg_scatter instead of 8: eight rounds of 128 dictionaries, 2^10 to 2^18
+// operations each, took 4042 us; now 3617.)
+template <bool kVals, int N>
+__device__ __forceinline__ void multi_load_items(const MultiBatch& in, const MultiInst& d, uint32_t nops, uint32_t t0,
+                                                 uint32_t m, uint32_t p0, uint32_t step, uint32_t (&kv)[N],
+                                                 uint32_t (&v)[N], bool& bad) {
+  const uint32_t last = d.b - 1 - t0;
+  const uint32_t* keys = in.keys + d.in_off;
+  const uint32_t* vals = in.vals + d.in_off;
+  const uint8_t* del = in.del + d.in_off;
+  uint32_t fl[N];
+  const auto load = [&](auto with_del, auto with_vals) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const uint32_t p = p0 + j * step;
+      kv[j] = v[j] = fl[j] = 0u;
+      if (p < m) {
+        const uint32_t s = min(last - p, nops - 1);
+        kv[j] = __ldg(keys + s);
+        if (decltype(with_del)::value) fl[j] = __ldg(del + s);
+        if (decltype(with_vals)::value) v[j] = __ldg(vals + s);
+      }
+    }
+  };
+  const bool has_vals = kVals && in.vals;
+  if (in.del && has_vals) load(std::true_type{}, std::true_type{});
+  else if (in.del) load(std::true_type{}, std::false_type{});
+  else if (has_vals) load(std::false_type{}, std::true_type{});
+  else load(std::false_type{}, std::false_type{});
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (p0 + j * step >= m) continue;
+    const bool b = kv[j] > kMaxUserKey;
+    bad |= b;
+    kv[j] = b ? kPlaceboKv : ((kv[j] << 1) | (fl[j] ? 0u : 1u));
+    if (!(kv[j] & 1u)) v[j] = 0u;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads) mseg_count(MultiArena ar, MultiBatch in) {
@@ -1543,16 +1563,11 @@ __global__ void __launch_bounds__(kThreads) mseg_count(MultiArena ar, MultiBatch
   const uint32_t m = (d.b - t0) < kMultiSortTile ? (d.b - t0) : kMultiSortTile;
   const int shift = 32 - int(d.msd_bits);
   bool bad_any = false;
-#pragma unroll 4
-  for (int j = 0; j < kMultiIPT; ++j) {
-    const uint32_t p = j * kThreads + tid;
-    if (p < m) {
-      bool bad;
-      const uint32_t kv = multi_load_key(in, d, nops, t0 + p, bad);
-      bad_any |= bad;
-      atomicAdd(&s_h[kv >> shift], 1u);
-    }
-  }
+  uint32_t kv[kMultiIPT], v[kMultiIPT];
+  multi_load_items<false>(in, d, nops, t0, m, tid, uint32_t(kThreads), kv, v, bad_any);
+#pragma unroll
+  for (int j = 0; j < kMultiIPT; ++j)
+    if (j * kThreads + tid < m) atomicAdd(&s_h[kv[j] >> shift], 1u);
   const int any_bad = __syncthreads_or(bad_any);
   ar.tilecnt[uint64_t(gt) * 512 + tid] = s_h[tid];
   if (any_bad && tid == 0) atomicOr(ar.badkey + i, 1u);
@@ -1585,11 +1600,11 @@ __global__ void __launch_bounds__(kThreads) mseg_offsets(MultiArena ar) {
   }
 }
 
-__global__ void __launch_bounds__(kThreads) mseg_scatter(MultiArena ar, MultiBatch in) {
+__global__ void __launch_bounds__(kScatterThreads) mseg_scatter(MultiArena ar, MultiBatch in) {
   __shared__ __align__(16) uint32_t s_keys[kMultiSortTile];
   __shared__ __align__(16) uint32_t s_vals[kMultiSortTile];
-  __shared__ uint32_t s_whist[kWarps][kRadix];
-  __shared__ uint32_t s_excl[kRadix], s_gbase[kRadix], s_scan[kWarps];
+  __shared__ uint32_t s_whist[kScatterWarps][kRadix];
+  __shared__ uint32_t s_excl[kRadix], s_gbase[kRadix], s_scan[kScatterWarps];
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, gt = blockIdx.x;
   const uint32_t i = find_instance(ar.stile_prefix, ar.n, gt);
   if (ar.k[i] < 0) return;  // whole CTA
@@ -1598,19 +1613,15 @@ __global__ void __launch_bounds__(kThreads) mseg_scatter(MultiArena ar, MultiBat
   const uint32_t t0 = (gt - d.stile0) * kMultiSortTile;
   const uint32_t m = (d.b - t0) < kMultiSortTile ? (d.b - t0) : kMultiSortTile;
   const int shift = 32 - int(d.msd_bits);
-  const uint32_t base = warp * (32 * kMultiIPT);
-  uint32_t kv[kMultiIPT], v[kMultiIPT], rank[kMultiIPT];
+  const uint32_t base = warp * (32 * kScatterIPT);
+  uint32_t kv[kScatterIPT], v[kScatterIPT], rank[kScatterIPT];
+  bool bad_any = false;  // (mseg_count has seen them)
+  multi_load_items<true>(in, d, nops, t0, m, base + lane, 32u, kv, v, bad_any);
+  if (tid < kRadix) s_gbase[tid] = ar.tilecnt[uint64_t(gt) * 512 + 256 + tid];
+  rank_block<kScatterThreads, kScatterIPT>(kv, m, base, [&](uint32_t k) { return k >> shift; }, rank, s_whist,
+                                           s_excl, s_scan, nullptr);
 #pragma unroll
-  for (int j = 0; j < kMultiIPT; ++j) {
-    const uint32_t p = base + j * 32 + lane;
-    kv[j] = 0;
-    v[j] = 0;
-    if (p < m) multi_load(in, d, nops, t0 + p, kv[j], v[j]);
-  }
-  s_gbase[tid] = ar.tilecnt[uint64_t(gt) * 512 + 256 + tid];
-  rank_block<kThreads, kMultiIPT>(kv, m, base, [&](uint32_t k) { return k >> shift; }, rank, s_whist, s_excl, s_scan, nullptr);
-#pragma unroll
-  for (int j = 0; j < kMultiIPT; ++j) {
+  for (int j = 0; j < kScatterIPT; ++j) {
     const uint32_t p = base + j * 32 + lane;
     if (p < m) {
       const uint32_t dg = kv[j] >> shift;
@@ -1622,7 +1633,7 @@ __global__ void __launch_bounds__(kThreads) mseg_scatter(MultiArena ar, MultiBat
   __syncthreads();
   uint32_t* tk = ar.tkeys + d.boff;
   uint32_t* tv = ar.tvals + d.boff;
-  for (uint32_t e = tid; e < m; e += kThreads) {
+  for (uint32_t e = tid; e < m; e += kScatterThreads) {
     const uint32_t k = s_keys[e];
     const uint32_t dg = k >> shift;
     const uint32_t dst = s_gbase[dg] + (e - s_excl[dg]);
@@ -1786,7 +1797,7 @@ cudaError_t multi_sort_launch(const MultiArena& ar, const MultiBatch& in, cudaSt
   mseg_offsets<<<ar.n, kThreads, 0, st>>>(ar);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   count_launches(1);
-  mseg_scatter<<<unsigned(ar.total_stiles), kThreads, 0, st>>>(ar, in);
+  mseg_scatter<<<unsigned(ar.total_stiles), kScatterThreads, 0, st>>>(ar, in);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   count_launches(1);
   mseg_bucket<<<unsigned(ar.total_buckets), kBucketThreads, kBucketSmem, st>>>(ar);

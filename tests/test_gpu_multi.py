@@ -236,3 +236,32 @@ def test_multi_config_full_size(g):
         ev, ef = o2.lookup(q[s])
         np.testing.assert_array_equal(found[s], ef)
         np.testing.assert_array_equal(val[s], ev)
+
+
+@pytest.mark.parametrize("with_vals", [False, True])
+@pytest.mark.parametrize("with_del", [False, True])
+def test_multi_optional_inputs(g, with_vals, with_del):
+    """Values and delete flags left out, at batch sizes around a sort tile."""
+    sizes = np.array([1, 31, 4095, 4096, 4097, 8193], np.int64)
+    n, off = len(sizes), np.concatenate([[0], np.cumsum(sizes)])
+    m = g.MultiLSM(list(sizes), max_batches=3)
+    s_or = [oracle.StructuralOracle(int(b)) for b in sizes]
+    rs = np.random.default_rng(2 * with_vals + with_del)
+    stream = torch.cuda.current_stream().cuda_stream
+    for t in range(3):
+        keys = rs.integers(0, 1 << 31, size=off[-1]).astype(np.uint32)
+        keys[keys == 0x7FFFFFFF] = 0
+        keys[::7] %= 50
+        vals = rs.integers(0, 1 << 32, size=off[-1], dtype=np.uint64).astype(np.uint32) * np.uint32(with_vals)
+        dele = (rs.random(off[-1]) < 0.3).astype(np.uint8) * np.uint8(with_del)
+        counts = np.array([rs.integers(1, b + 1) for b in sizes], np.uint32) if t == 1 else sizes.astype(np.uint32)
+        dev = [g.as_device_u32(keys, 0), g.as_device_u32(vals, 0), g.as_device_u8(dele, 0), g.as_device_u32(counts, 0)]
+        g.lsm_multi_update(m.h, dev[0].data_ptr(), dev[1].data_ptr() if with_vals else None,
+                           dev[2].data_ptr() if with_del else None, dev[3].data_ptr(), stream)
+        status, flags = m.sync()
+        assert status == g.LSM_OK and flags == [0] * n
+        for i in range(n):
+            c = slice(int(off[i]), int(off[i]) + int(counts[i]))
+            s_or[i].call("update", keys[c], vals[c], dele[c])
+        check_levels(m, s_or, range(n))
+    m.close()
