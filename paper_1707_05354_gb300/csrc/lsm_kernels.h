@@ -240,7 +240,7 @@ struct MultiInst {           // fixed at creation
   uint64_t boff;             // its sorted batch / sort scratch start (a multiple of kLevelAlign)
   uint32_t b;                // batch size
   uint32_t levels;           // allocated levels: a batch is refused once ffz(r) >= levels
-  uint32_t msd_bits;         // d: the batch sort's buckets are the top d bits of the key variable
+  uint32_t msd_bits;         // d: the batch sort has 2^d buckets, equal parts of the batch's key range
   uint32_t tile;             // merge tile: 1024 or 2048 output elements
   uint32_t stile0;           // first global sort tile
   uint32_t bucket0;          // first global bucket
@@ -268,6 +268,8 @@ struct MultiArena {
   uint32_t* tilecnt;         // per sort tile 256 bucket counts, then 256 output offsets
   uint32_t* bstart;          // per global bucket: start in the instance's batch
   uint32_t* bcnt;            // per global bucket: element count
+  uint32_t* blo;             // per global bucket: its smallest key variable
+  uint32_t* map;             // per instance: start and factor of its buckets' key range
   // device state
   uint32_t* r;               // batches applied per instance
   int32_t* k;                // this round's fold target level, -1 when the instance has no batch

@@ -224,7 +224,7 @@ lsm_status lsm_multi_create(lsm_multi_t** out, uint32_t n_inst, const uint32_t* 
   const uint64_t stiles = stp[n_inst], buckets = bkp[n_inst];
   const uint64_t state_words = 4ull * n_inst + 8;
   h->device_bytes = sizeof(MultiInst) * n_inst + 32ull * (n_inst + 1) + 8 * loff + 16 * boff + 4 * foff +
-                    4 * stiles * 512 + 8 * buckets + 4 * part_words * kMultiPartStride + 4 * state_words;
+                    4 * stiles * 512 + 12 * buckets + 8 * n_inst + 4 * part_words * kMultiPartStride + 4 * state_words;
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = dalloc(&h->d_inst, n_inst);
   if (e == cudaSuccess) e = dalloc(&h->d_prefix, 4ull * (n_inst + 1));
@@ -236,7 +236,7 @@ lsm_status lsm_multi_create(lsm_multi_t** out, uint32_t n_inst, const uint32_t* 
   if (e == cudaSuccess) e = dalloc(&h->d_tv, boff);
   if (e == cudaSuccess) e = dalloc(&h->d_fence, foff);
   if (e == cudaSuccess) e = dalloc(&h->d_tilecnt, stiles * 512);
-  if (e == cudaSuccess) e = dalloc(&h->d_bucket, 2 * buckets);
+  if (e == cudaSuccess) e = dalloc(&h->d_bucket, 3 * buckets + 2 * n_inst);
   if (e == cudaSuccess) e = dalloc(&h->d_part, part_words * kMultiPartStride);
   if (e == cudaSuccess) e = dalloc(&h->d_state, state_words);
   if (e == cudaSuccess) e = cudaMemcpy(h->d_inst, inst.data(), sizeof(MultiInst) * n_inst, cudaMemcpyHostToDevice);
@@ -276,6 +276,8 @@ lsm_status lsm_multi_create(lsm_multi_t** out, uint32_t n_inst, const uint32_t* 
   a.tilecnt = h->d_tilecnt;
   a.bstart = h->d_bucket;
   a.bcnt = h->d_bucket + buckets;
+  a.blo = h->d_bucket + 2 * buckets;
+  a.map = h->d_bucket + 3 * buckets;
   a.r = h->d_state;
   a.k = reinterpret_cast<int32_t*>(h->d_state + n_inst);
   a.badkey = h->d_state + 2 * n_inst;

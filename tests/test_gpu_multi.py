@@ -265,3 +265,39 @@ def test_multi_optional_inputs(g, with_vals, with_del):
             s_or[i].call("update", keys[c], vals[c], dele[c])
         check_levels(m, s_or, range(n))
     m.close()
+
+
+@pytest.mark.parametrize("keys_of", ["low", "high", "one", "wide", "hot"])
+def test_multi_key_ranges(g, keys_of):
+    """Batches over narrow, distant and repeated keys: the sort splits the range that each instance's batch spans."""
+    sizes = np.array([1, 300, 4096, 5121, 12000, 40000], np.int64)
+    n, off = len(sizes), np.concatenate([[0], np.cumsum(sizes)])
+    m = g.MultiLSM(list(sizes), max_batches=3)
+    s_or = [oracle.StructuralOracle(int(b)) for b in sizes]
+    o1 = [oracle.MapOracle(int(b)) for b in sizes]
+    rs = np.random.default_rng(len(keys_of))
+    top = (1 << 31) - 1
+    for t in range(3):
+        u = rs.integers(0, top, size=off[-1])
+        keys = {"low": u % 30000, "high": top - 1 - u % 9000, "one": np.full(off[-1], 1 << 29), "wide": u,
+                "hot": np.where(u % 3 == 0, 77777, u % (1 << 20))}[keys_of].astype(np.uint32)
+        vals = rs.integers(0, 1 << 32, size=off[-1], dtype=np.uint64).astype(np.uint32)
+        dele = (rs.random(off[-1]) < 0.3).astype(np.uint8)
+        counts = np.array([rs.integers(1, b + 1) for b in sizes], np.uint32) if t == 1 else None
+        m.update(keys, vals, dele, counts)
+        status, flags = m.sync()
+        assert status == g.LSM_OK and flags == [0] * n
+        for i in range(n):
+            c = slice(int(off[i]), int(off[i]) + int(sizes[i] if counts is None else counts[i]))
+            for o in (s_or[i], o1[i]):
+                o.call("update", keys[c], vals[c], dele[c])
+        check_levels(m, s_or, range(n))
+    qoff = np.arange(n + 1, dtype=np.int64) * 500
+    q = rs.choice(keys, int(qoff[-1])).astype(np.uint32)
+    val, found = m.lookup(q, qoff)
+    torch.cuda.synchronize()
+    for i in range(n):
+        ev, ef = o1[i].lookup(q[qoff[i]:qoff[i + 1]])
+        np.testing.assert_array_equal(found.cpu().numpy()[qoff[i]:qoff[i + 1]], ef)
+        np.testing.assert_array_equal(u32(val)[qoff[i]:qoff[i + 1]], ev)
+    m.close()
