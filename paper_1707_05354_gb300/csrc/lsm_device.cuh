@@ -126,6 +126,18 @@ __device__ __forceinline__ uint32_t find_instance(const uint64_t* prefix, uint32
   return lo;
 }
 
+// The same by a whole warp: 32 probes a round.
+__device__ __forceinline__ uint32_t find_instance_warp(const uint64_t* prefix, uint32_t n, uint64_t w) {
+  uint32_t lo = 0, hi = n;  // answer in [lo, hi)
+  while (hi - lo > 1) {
+    const uint32_t step = (hi - lo + 31) / 32, at = lo + lane_id() * step;
+    const uint32_t le = __ballot_sync(0xffffffffu, at < hi && __ldg(prefix + at) <= w);
+    lo += (uint32_t(__popc(le)) - 1) * step;  // (prefix[lo] <= w: lane 0 is among them)
+    hi = min(lo + step, hi);
+  }
+  return lo;
+}
+
 // Lanes of the warp whose value equals this lane's (values below 2^kBits):
 // the intersection, over the bits, of the lanes that agree with this lane on
 // that bit -- one ballot per bit, a fixed cost however many distinct values
