@@ -1,7 +1,9 @@
-// Batch sort of the GPU LSM: a stable least-significant-digit radix sort of
-// (key variable, value) pairs over all 32 bits, 8 bits per pass (§IV-A sorts
-// every batch with a radix sort over the whole key variable, status bit
-// included, so a tombstone precedes a regular element of the same key).
+// Batch sort of the GPU LSM: a stable radix sort of (key variable, value) pairs
+// over all 32 bits (§IV-A sorts every batch with a radix sort over the whole
+// key variable, status bit included, so a tombstone precedes a regular element
+// of the same key).  Up to 5120 elements one CTA sorts the batch (small_sort),
+// up to 2^20 msd_tile and bucket_sort do, whose comments are further down; what
+// follows is the least-significant-digit sort above that, 8 bits per pass.
 //
 // Structure (one histogram kernel, then one kernel per digit):
 //   * sort_histogram reads the input once and counts all four digits; in the
@@ -1561,7 +1563,7 @@ __device__ __forceinline__ void multi_load_items(const MultiBatch& in, const Mul
 __global__ void __launch_bounds__(kThreads) mseg_count(MultiArena ar, MultiBatch in) {
   __shared__ uint32_t s_h[kRadix], s_mn[kWarps], s_mx[kWarps];
   const uint32_t tid = threadIdx.x, gt = blockIdx.x;
-  const uint32_t i = find_instance(ar.stile_prefix, ar.n, gt);
+  const uint32_t i = find_instance_warp(ar.stile_prefix, ar.n, gt);
   const MultiInst& d = ar.inst[i];
   const uint32_t nops = multi_ops(in, d, i);
   if (nops == 0 || nops > d.b) return;  // whole CTA: no batch, or refused
@@ -1634,7 +1636,7 @@ __global__ void __launch_bounds__(kScatterThreads) mseg_scatter(MultiArena ar, M
   __shared__ uint32_t s_whist[kScatterWarps][kRadix];
   __shared__ uint32_t s_excl[kRadix], s_gbase[kRadix], s_scan[kScatterWarps];
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, gt = blockIdx.x;
-  const uint32_t i = find_instance(ar.stile_prefix, ar.n, gt);
+  const uint32_t i = find_instance_warp(ar.stile_prefix, ar.n, gt);
   if (ar.k[i] < 0) return;  // whole CTA
   const MultiInst& d = ar.inst[i];
   const uint32_t nops = multi_ops(in, d, i);
@@ -1683,7 +1685,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) 
   extern __shared__ __align__(16) uint32_t bsm[];
   __shared__ BucketShared sh;
   const uint32_t gb = blockIdx.x;
-  const uint32_t i = find_instance(ar.bucket_prefix, ar.n, gb);
+  const uint32_t i = find_instance_warp(ar.bucket_prefix, ar.n, gb);
   const int k = ar.k[i];
   if (k < 0) return;  // whole CTA
   const MultiInst& d = ar.inst[i];
