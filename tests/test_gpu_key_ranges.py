@@ -229,3 +229,32 @@ def test_hot_words(g, words, n):
     np.testing.assert_array_equal(g.to_numpy_u32(vo), order.astype(np.uint32))
     assert lsm.device_errors() == 0
     lsm.close()
+
+
+@pytest.mark.parametrize("b", [1, 33, 1051, 5119, 5120, 5121])
+@pytest.mark.parametrize("dist", ["two", "ids", "outliers", "hot"])
+def test_small_batches_over_ranges(g, dist, b):
+    """Batches around the largest that one CTA sorts, whose prefix-index entries several CTAs write: levels, and
+    lookups and counts across the whole key range."""
+    rng = np.random.default_rng(b + DISTS.index(dist))
+    lsm, s, o1 = g.LSM(b, 8 * b), oracle.StructuralOracle(b), oracle.MapOracle(b)
+    for t in range(5):
+        n = b if t != 2 else max(1, b // 3)
+        k, v = draw(dist, n, rng), rng.integers(0, 1 << 31, n).astype(np.uint32)
+        d = (rng.random(n) < 0.2).astype(np.uint8)
+        for x in (lsm, s, o1):
+            x.call("update", k, v, d)
+        for i, (kv, vv) in lsm.levels().items():
+            ekv, ev = s.level(i)
+            np.testing.assert_array_equal(kv, ekv)
+            np.testing.assert_array_equal(vv, ev)
+        q = np.concatenate([k, np.minimum(k + 1, TOP), np.linspace(0, TOP - 1, 3000).astype(np.uint32)]).astype(np.uint32)
+        val, found = lsm.lookup(q)
+        ev, ef = o1.lookup(q)
+        np.testing.assert_array_equal(found.cpu().numpy(), ef)
+        np.testing.assert_array_equal(g.to_numpy_u32(val), ev)
+        k1 = np.sort(q)[:-1]
+        k2 = np.sort(q)[1:]
+        np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), o1.count(k1, k2))
+    assert lsm.device_errors() == 0
+    lsm.close()
