@@ -358,8 +358,9 @@ lsm_status lsm_get_option(lsm_t* h, lsm_option opt, int64_t* value);
  * group, the number of launches, their total device time and the ALGORITHMIC
  * bytes they had to move (the bytes an ideal implementation reads and writes
  * in HBM; scratch traffic excluded):
- *   LSM_PROF_SORT       batch sort (two kernels up to 2^20 elements, else a
- *                       histogram and four passes), 16 B per element
+ *   LSM_PROF_SORT       batch sort (one kernel up to 5120 elements, two up to
+ *                       2^20, else a histogram and four passes), 16 B per
+ *                       element
  *   LSM_PROF_PARTITION  fold co-rank search, 0 B (pure overhead)
  *   LSM_PROF_MERGE      fold merge into level k, 16 * 2^k * b B
  *   LSM_PROF_LOOKUP     lookup kernels, 9 B per query + 32 B per level probed

@@ -5,7 +5,7 @@
 // where the interface says so (the key check of an update, the totals of
 // range and cleanup).
 //
-// Two streams.  A batch is sorted on the caller's stream into one of three
+// Two streams.  A batch is sorted on the caller's stream into one of six
 // sorted-batch buffers; its fold into level k runs on the handle's internal
 // stream, so the next batch's sort overlaps it.  A batch that lands in level
 // 0 (k = 0) is not copied: its buffer becomes level 0 until the next fold
