@@ -1118,15 +1118,20 @@ __global__ void __launch_bounds__(kThreads) place_write(const uint32_t* __restri
 // Prefix index of a sorted run: the element at position i owns the entries
 // between the bin of element i - 1 and its own; the first and last elements
 // record the populated bin range.  Four elements a thread from one 16-byte
-// load (n = 32 million: 101 -> 74 us).
+// load (n = 32 million: 101 -> 74 us), `per` elements a CTA: 1024, or of a
+// sparse run as many as share about kFencePer entries, which the CTA fills in
+// together (one CTA alone wrote all 2^16 entries of a run of 1000: its cleanup
+// 75 us, now 43).
+constexpr uint32_t kFencePer = 2048;
 __global__ void __launch_bounds__(256) build_fence(const uint32_t* __restrict__ keys, uint32_t n,
-                                                   uint32_t* __restrict__ fence, int fshift) {
+                                                   uint32_t* __restrict__ fence, int fshift, uint32_t per) {
   __shared__ uint32_t s_ngap;
   __shared__ FenceGap s_gaps[kFenceGapSlots];
   if (threadIdx.x == 0) s_ngap = 0;
   __syncthreads();
   const uint32_t nb = fence_bins(fshift);
-  for (uint64_t i0 = (blockIdx.x * 256ull + threadIdx.x) * 4; i0 < n; i0 += uint64_t(gridDim.x) * 1024ull) {
+  for (uint64_t i0 = uint64_t(blockIdx.x) * per + threadIdx.x * 4; threadIdx.x * 4 < per && i0 < n;
+       i0 += uint64_t(gridDim.x) * per) {
     const uint4 w = __ldg(reinterpret_cast<const uint4*>(keys + i0));  // (slack is readable)
     const uint32_t kv[4] = {w.x, w.y, w.z, w.w};
     uint32_t pb = i0 ? fence_bin(__ldg(keys + i0 - 1), fshift) : fence_bin(kv[0], fshift);
@@ -1272,10 +1277,12 @@ cudaError_t place_write_launch(const uint32_t* keys, const uint32_t* vals, uint6
 }
 
 cudaError_t build_fence_launch(const uint32_t* keys, uint32_t n, uint32_t* fence, int fshift, cudaStream_t st) {
-  uint64_t blocks = (uint64_t(n) + 1023) / 1024;
+  const uint64_t share = uint64_t(n) * kFencePer / fence_bins(fshift) / 4 * 4;
+  const uint32_t per = uint32_t(share < 4 ? 4 : (share > 1024 ? 1024 : share));
+  uint64_t blocks = (uint64_t(n) + per - 1) / per;
   if (blocks > 152 * 8) blocks = 152 * 8;
   count_launches(1);
-  build_fence<<<unsigned(blocks), 256, 0, st>>>(keys, n, fence, fshift);
+  build_fence<<<unsigned(blocks), 256, 0, st>>>(keys, n, fence, fshift, per);
   return cudaGetLastError();
 }
 

@@ -791,11 +791,11 @@ static DistributeArgs level_places(const lsm_t* h, uint64_t n_live) {
 // then fill the set bits of r' in ascending level order, with placebo
 // tombstones after the last one (§IV-E).  Several sources are folded into the
 // cleanup scratch and copied from there; a single one is counted and written
-// at once, to the levels themselves when it lies in the scratch (a bulk
-// build's sorted pairs), else by way of the scratch (it is a level).
+// at once, to the levels themselves unless one of them is the source, else by
+// way of the scratch.
 // Synchronises with `st` (the host must learn n').
 static lsm_status rebuild(lsm_t* h, const FoldSources& src, uint64_t total, cudaStream_t st) {
-  const bool single = src.count == 1, direct = single && src.keys[0] == h->d_ck;
+  const bool single = src.count == 1;
   LSM_TRY(ensure_clean(h));
   // a single source's offsets and counts per tile, in the co-rank table
   const uint64_t tiles = place_tiles(total);
@@ -828,6 +828,9 @@ static lsm_status rebuild(lsm_t* h, const FoldSources& src, uint64_t total, cuda
   if (n_live > total) return LSM_ERR_CUDA;
   const uint64_t r2 = (n_live + h->b - 1) / h->b;
   h->l0_buf = -1;  // every level is rewritten in the level array
+  bool direct = single;
+  for (uint32_t i = 0; i < h->L; ++i)
+    if (((r2 >> i) & 1u) && src.keys[0] == level_keys(h, i)) direct = false;
   DistributeArgs d = level_places(h, n_live);
   d.src_keys = h->d_ck;
   d.src_vals = h->d_cv;

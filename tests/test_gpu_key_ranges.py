@@ -258,3 +258,32 @@ def test_small_batches_over_ranges(g, dist, b):
         np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), o1.count(k1, k2))
     assert lsm.device_errors() == 0
     lsm.close()
+
+
+@pytest.mark.parametrize("deletes", [0.0, 0.7, 1.0])
+@pytest.mark.parametrize("batches", [1, 2, 4])
+@pytest.mark.parametrize("b", [1, 5, 1000, 5200])
+def test_cleanup_of_one_level(g, b, batches, deletes):
+    """A single full level cleaned up into itself, into smaller levels or into nothing, and its prefix index."""
+    rng = np.random.default_rng(b + batches)
+    lsm, s, o1 = g.LSM(b, 8 * b), oracle.StructuralOracle(b), oracle.MapOracle(b)
+    keys = draw("outliers" if b > 100 else "ids", b, rng)
+    for t in range(batches):
+        k = np.where(rng.random(b) < 0.5, keys, rng.integers(0, TOP, b)).astype(np.uint32)
+        v, d = rng.integers(0, 1 << 31, b).astype(np.uint32), (rng.random(b) < deletes).astype(np.uint8)
+        for x in (lsm, s, o1):
+            x.call("update", k, v, d)
+    lsm.cleanup()
+    s.cleanup()
+    assert lsm.r == s.r
+    for i, (kv, vv) in lsm.levels().items():
+        ekv, ev = s.level(i)
+        np.testing.assert_array_equal(kv, ekv)
+        np.testing.assert_array_equal(vv, ev)
+    q = np.concatenate([keys, k, np.linspace(0, TOP - 1, 2000).astype(np.uint32)]).astype(np.uint32)
+    val, found = lsm.lookup(q)
+    ev, ef = o1.lookup(q)
+    np.testing.assert_array_equal(found.cpu().numpy(), ef)
+    np.testing.assert_array_equal(g.to_numpy_u32(val), ev)
+    assert lsm.device_errors() == 0
+    lsm.close()
