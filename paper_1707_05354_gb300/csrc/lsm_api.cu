@@ -917,15 +917,21 @@ lsm_status lsm_bulk_build(lsm_t* h, const uint32_t* d_keys, const uint32_t* d_va
   const cudaError_t e = sort_launch(a, ws, st, h->d_status_map, seq);
   h->sws.flip = ws.flip;
   h->blb_epoch = ws.epoch;
-  LSM_TRY(e);
-  const lsm_status s = wait_check(h, seq, st);
-  if (s != LSM_OK) return s;
-  FoldSources src{};
-  src.count = 1;
-  src.keys[0] = a.out_keys;
-  src.vals[0] = a.out_vals;
-  src.n[0] = uint32_t(n);
-  return rebuild(h, src, n, st);
+  lsm_status s = cuda_status(e);
+  if (s == LSM_OK) s = wait_check(h, seq, st);
+  if (s == LSM_OK) {
+    FoldSources src{};
+    src.count = 1;
+    src.keys[0] = a.out_keys;
+    src.vals[0] = a.out_vals;
+    src.n[0] = uint32_t(n);
+    s = rebuild(h, src, n, st);
+  }
+  // The sort reads the caller's pairs after the verdict of the key check, and
+  // the levels are written after the wait for n': no later call is ordered
+  // after either, so both have ended when this one returns.
+  const lsm_status end = cuda_status(cudaStreamSynchronize(st));
+  return s != LSM_OK ? s : end;
 }
 
 lsm_status lsm_stats(const lsm_t* h, uint64_t* r, uint64_t* resident, uint32_t* b, uint32_t* levels) {
