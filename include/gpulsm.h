@@ -143,9 +143,10 @@ lsm_status lsm_update_batch_ordered(lsm_t* h, const uint32_t* d_keys, const uint
  * element of the key found decides: regular -> found, tombstone -> absent.
  * nq = 0 is a no-op.  Asynchronous.  Many queries (from several 10^5 on,
  * depending on the levels) are grouped by key range first, in about 7.3 bytes
- * per query of the handle's query scratch (grown on demand; growing it
- * synchronises the device); without that memory, and on a stream that is
- * being captured, they are searched in input order.
+ * per query of scratch that only lookups use (grown on demand; growing it
+ * synchronises the device; grouped lookups on several streams take turns);
+ * without that memory, and on a stream that is being captured, they are
+ * searched in input order.
  */
 lsm_status lsm_lookup(lsm_t* h, const uint32_t* d_q, uint64_t nq, uint32_t* d_val,
                       uint8_t* d_found, void* stream);

@@ -106,6 +106,12 @@ struct lsm_t {
   // query scratch (grown on demand)
   unsigned char* d_q = nullptr;
   size_t q_bytes = 0;
+  // Scratch of the grouped lookups (grown on demand), and the event after the
+  // latest of them: the next one, on whichever stream, waits for it.  Apart
+  // from d_q, so that a lookup never moves what a captured count points to.
+  unsigned char* d_lk = nullptr;
+  size_t lk_bytes = 0;
+  cudaEvent_t ev_lk = nullptr;
   // sorted-lookup workspace (grown on demand)
   SortWorkspace qsws{};
   uint32_t* d_qctl = nullptr;
@@ -169,11 +175,12 @@ cudaError_t dalloc(T** p, uint64_t count) {
 void free_all(lsm_t* h) {
   void* dptrs[] = {h->d_keys, h->d_vals, h->d_bk, h->d_bv, h->d_tk, h->d_tv, h->sws.ctl, h->sws.lookback,
                    h->sws.tilecnt, h->d_part, h->d_fence, h->d_misc, h->d_u64, h->d_ck, h->d_cv, h->d_clb, h->d_blb,
-                   h->d_q, h->qsws.lookback, h->qsws.tilecnt, h->d_qctl};
+                   h->d_q, h->d_lk, h->qsws.lookback, h->qsws.tilecnt, h->d_qctl};
   for (void* p : dptrs)
     if (p) cudaFree(p);
   if (h->side) cudaStreamDestroy(h->side);
   if (h->ev_sorted) cudaEventDestroy(h->ev_sorted);
+  if (h->ev_lk) cudaEventDestroy(h->ev_lk);
   for (cudaEvent_t e : h->ev_fold)
     if (e) cudaEventDestroy(e);
   if (h->h_status) cudaFreeHost(h->h_status);
@@ -248,20 +255,22 @@ LevelSet full_levels(lsm_t* h) {
   return ls;
 }
 
-cudaError_t ensure_q(lsm_t* h, size_t bytes) {
-  if (bytes <= h->q_bytes) return cudaSuccess;
-  if (h->d_q) {
-    cudaError_t e = cudaFree(h->d_q);
-    h->d_q = nullptr;
-    h->q_bytes = 0;
+cudaError_t grow(unsigned char** p, size_t* have, size_t bytes) {
+  if (bytes <= *have) return cudaSuccess;
+  if (*p) {
+    cudaError_t e = cudaFree(*p);
+    *p = nullptr;
+    *have = 0;
     if (e != cudaSuccess) return e;
   }
   const size_t want = round_up(bytes + bytes / 4, 1 << 20);
   cudaError_t e = alloc_gate();
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&h->d_q), want);
-  if (e == cudaSuccess) h->q_bytes = want;
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(p), want);
+  if (e == cudaSuccess) *have = want;
   return e;
 }
+
+cudaError_t ensure_q(lsm_t* h, size_t bytes) { return grow(&h->d_q, &h->q_bytes, bytes); }
 
 // Whether many lookups are worth grouping by key range (lookup_bulk_launch).
 // Measured over 1 to 7 full levels, 4 thousand to 264 million elements and 2^14
@@ -589,6 +598,7 @@ lsm_status lsm_create(lsm_t** out, uint32_t b, uint64_t max_elements, int device
   if (e == cudaSuccess) e = cudaMemset(h->d_bv, 0, sizeof(uint32_t) * kBatchBufs * bpad);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_sorted, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_lk, cudaEventDisableTiming);
   for (cudaEvent_t& ev : h->ev_fold)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   if (e == cudaSuccess)
@@ -659,15 +669,23 @@ lsm_status lsm_lookup(lsm_t* h, const uint32_t* d_q, uint64_t nq, uint32_t* d_va
   if (bulk) {
     // Without the scratch (no memory, or a stream being captured, whose graph
     // would keep a pointer that a later call may free) the queries are
-    // searched in input order.
+    // searched in input order.  (The scratch may grow while another stream is
+    // being captured: it is no part of that graph.)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     bulk = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-           ensure_q(h, lookup_bulk_bytes(nq)) == cudaSuccess;
+           cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    if (bulk) {
+      bulk = grow(&h->d_lk, &h->lk_bytes, lookup_bulk_bytes(nq)) == cudaSuccess;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
     if (!bulk) cudaGetLastError();
   }
   ProfScope ps(h, LSM_PROF_LOOKUP, double(nq) * (9.0 + 32.0 * ls.count), st);
   if (!bulk) return cuda_status(lookup_launch(ls, d_q, nq, d_val, d_found, st));
-  return cuda_status(lookup_bulk_launch(ls, d_q, nq, d_val, d_found, h->d_q, st));
+  LSM_TRY(cudaStreamWaitEvent(st, h->ev_lk, 0));  // (at once before the first record)
+  LSM_TRY(lookup_bulk_launch(ls, d_q, nq, d_val, d_found, h->d_lk, st));
+  return cuda_status(cudaEventRecord(h->ev_lk, st));
 }
 
 static lsm_status neighbor_call(lsm_t* h, const uint32_t* d_q, uint64_t nq, bool successor, uint32_t* d_key,
