@@ -998,6 +998,109 @@ __device__ __forceinline__ SortedView sort_resident(const Load& load, uint32_t m
   return SortedView{ak, m, nullptr, range.map};
 }
 
+// A bucket above kBucketCap elements of many different keys in clusters: stable
+// 8-bit passes over the bits in which the keys [mn, mx] differ, kBucketCap
+// elements at a time, between the bucket's places in the scratch and out[0 .. m)
+// (every element is read and written once per pass, whatever the keys; pass 0
+// reads the scratch).  The last pass leaves room for the padding run.  Bound by
+// the one CTA's instructions, about 9 us a chunk.
+template <class Src>
+__device__ __noinline__ void sort_digits(uint32_t* src_k, uint32_t* src_v, const Src src, uint32_t* out_k,
+                                         uint32_t* out_v, uint32_t m, uint32_t mn, uint32_t mx, const PadRun pad,
+                                         uint32_t* bsm, BucketShared& sh) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  uint32_t *to = bsm, *tot = to + kSortPasses * kRadix;  // next place of a digit per pass, its count in the chunk
+  uint32_t *sk = tot + kRadix, *sv = sk + kBucketCap;
+  static_assert((kSortPasses + 1) * kRadix <= kBucketCap, "fits the bucket's shared memory");
+  const int passes = (32 - __clz(int(mx - mn)) + 7) / 8;
+  const auto room = [&](uint32_t kv) { return pad.n && kv >= pad.kv ? pad.n : 0u; };
+  for (uint32_t i = tid; i < uint32_t(kSortPasses * kRadix); i += kBucketThreads) to[i] = 0u;
+  __syncthreads();
+  constexpr uint32_t kItems = 8;
+  for (uint32_t i0 = 0, t = 0; i0 < m; i0 += kItems * kBucketThreads) {
+    uint32_t k[kItems];
+#pragma unroll
+    for (uint32_t j = 0; j < kItems; ++j) {
+      const uint32_t i = i0 + j * kBucketThreads + tid;
+      k[j] = i < m ? src_k[src.seek(i, t)] - mn : 0u;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kItems; ++j)
+      if (i0 + j * kBucketThreads + tid < m)
+        for (int p = 0; p < passes; ++p) atomicAdd(&to[p * kRadix + ((k[j] >> (8 * p)) & 255u)], 1u);
+  }
+  __syncthreads();
+  for (int p = 0; p < passes; ++p) {
+    uint32_t all;
+    const uint32_t first = block_excl_scan<kBucketThreads>(tid < kRadix ? to[p * kRadix + tid] : 0u, sh.scan, all);
+    if (tid < kRadix) to[p * kRadix + tid] = first;
+  }
+  __syncthreads();
+  const uint32_t wbase = warp * (32 * kBucketIPT);
+  for (int p = 0; p < passes; ++p) {
+    const bool back = p & 1;  // out -> scratch
+    const auto digit = [&](uint32_t k) { return ((k - mn) >> (8 * p)) & 255u; };
+    for (uint32_t c0 = 0, t = 0; c0 < m; c0 += kBucketCap) {
+      const uint32_t cm = min(m - c0, kBucketCap);
+      uint32_t kv[kBucketIPT], v[kBucketIPT], rank[kBucketIPT];
+#pragma unroll
+      for (int j = 0; j < kBucketIPT; ++j) {
+        const uint32_t x = wbase + j * 32 + lane;
+        kv[j] = v[j] = 0u;
+        if (x < cm) {
+          const uint32_t at = back ? c0 + x : src.seek(c0 + x, t);
+          kv[j] = back ? out_k[at] : src_k[at];
+          v[j] = back ? out_v[at] : src_v[at];
+        }
+      }
+      rank_block<kBucketThreads, kBucketIPT>(kv, cm, wbase, digit, rank, sh.whist, sh.excl, sh.scan, tot);
+#pragma unroll
+      for (int j = 0; j < kBucketIPT; ++j) {
+        if (wbase + j * 32 + lane < cm) {
+          const uint32_t d = digit(kv[j]), at = sh.excl[d] + sh.whist[warp][d] + rank[j];
+          sk[at] = kv[j];
+          sv[at] = v[j];
+        }
+      }
+      __syncthreads();
+      for (uint32_t i = tid; i < cm; i += kBucketThreads) {
+        const uint32_t k = sk[i], d = digit(k), at = to[p * kRadix + d] + (i - sh.excl[d]);
+        if (back) {
+          const uint32_t x = src.find(at);
+          src_k[x] = k;
+          src_v[x] = sv[i];
+        } else {
+          const uint32_t x = p + 1 == passes ? at + room(k) : at;
+          out_k[x] = k;
+          out_v[x] = sv[i];
+        }
+      }
+      __syncthreads();
+      if (tid < kRadix) to[p * kRadix + tid] += tot[tid];
+    }
+  }
+  if (passes & 1) return;
+  uint32_t t = 0;  // an even number of passes ends in the scratch
+  for (uint32_t i0 = 0; i0 < m; i0 += kItems * kBucketThreads) {
+    uint32_t k[kItems], v[kItems];
+#pragma unroll
+    for (uint32_t j = 0; j < kItems; ++j) {
+      const uint32_t i = i0 + j * kBucketThreads + tid;
+      const uint32_t at = i < m ? src.seek(i, t) : 0u;
+      k[j] = i < m ? src_k[at] : 0u;
+      v[j] = i < m ? src_v[at] : 0u;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kItems; ++j) {
+      const uint32_t i = i0 + j * kBucketThreads + tid;
+      if (i < m) {
+        out_k[i + room(k[j])] = k[j];
+        out_v[i + room(k[j])] = v[j];
+      }
+    }
+  }
+}
+
 // A bucket above kBucketCap elements: taken in key order, a part at a time.
 // Each round looks at the elements of [a, b], the keys still to do:
 //   at most kBucketCap of them        gathered in order, sorted, written;
@@ -1007,11 +1110,18 @@ __device__ __forceinline__ SortedView sort_resident(const Load& load, uint32_t m
 //   otherwise                         b is lowered to the end of the longest
 //                                     prefix of sub-bins that fits.
 // A round reads the bucket two or three times (from L2), 8 independent loads
-// a thread at a time.  Bound by the one CTA's chain of rounds.  (Stable 8-bit
-// passes in chunks through global memory before: a sort of 2^20 pairs of which
-// 8 % have one key 448 -> 164 us, of 2^18 Zipf(1.1) pairs 130 -> 64 us.)
+// a thread at a time.  Bound by the one CTA's chain of rounds.  (sort_digits
+// alone: a sort of 2^20 pairs of which 8 % have one key 448 us, with the rounds
+// 164.)  Their time grows with the square of the bucket, so more than kMaxParts *
+// kBucketCap elements beside the hot key are left to sort_digits: 2^18 keys, as
+// many in every octave, 15.1 -> 1.26 ms, 2^20 178 -> 4.6; 2^20 of which 2 % lie
+// anywhere and the rest below 2^24 109 -> 3.0; in ten clusters 5.9 -> 0.66.  At
+// three parts 2^14 such keys take 120 us, at two 102; below two the rounds are
+// the faster ones (four rounds of 128 batches of 8192 keys whose larger bucket
+// holds 5500: 443 us, with the passes 565).
+constexpr uint32_t kMaxParts = 2;
 template <class Src>
-__device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src_v, const Src src, uint32_t* out_k,
+__device__ __noinline__ void sort_big(uint32_t* src_k, uint32_t* src_v, const Src src, uint32_t* out_k,
                                       uint32_t* out_v, uint32_t start, uint32_t m, const BucketRange range,
                                       const PadRun pad, uint32_t* bsm, BucketShared& sh) {
   constexpr uint32_t kItems = 8, kChunk = kItems * kBucketThreads;
@@ -1059,6 +1169,7 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
       for (uint32_t j = 0; j < kItems; ++j) f(k[j], i0 + j * kBucketThreads + tid < m);
     }
   };
+  uint32_t pad_at = start;  // the padding run, after the elements below it
   if (pad.n) {
     if (tid == 0) sh.cnt[0] = 0u;
     __syncthreads();
@@ -1067,11 +1178,7 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
     L = __reduce_add_sync(0xffffffffu, L);
     if (lane == 0) atomicAdd(&sh.cnt[0], L);
     __syncthreads();
-    L = sh.cnt[0];
-    for (uint32_t j = tid; j < pad.n; j += kBucketThreads) {
-      out_k[start + L + j] = pad.kv;
-      out_v[start + L + j] = pad.v;
-    }
+    pad_at += sh.cnt[0];
   }
   uint32_t a = range.lo, b = range.hi, done = 0;
   while (done < m) {
@@ -1144,6 +1251,11 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
       below = 0;
       copies = c;
       tombs = mn & 1u ? 0u : c;
+    }
+    if (c == m && c - copies > kMaxParts * kBucketCap) {
+      __syncthreads();
+      sort_digits(src_k, src_v, src, out_k + start, out_v + start, m, mn, mx, pad, bsm, sh);
+      break;
     }
     if (c - copies > kBucketCap) {
       // Sub-bins over [mn, mx]; the lanes that share the sub-bin of the
@@ -1264,6 +1376,11 @@ __device__ __noinline__ void sort_big(const uint32_t* src_k, const uint32_t* src
     a = b + 1;
     b = range.hi;
   }
+  __syncthreads();  // (the passes use the padding's places)
+  for (uint32_t j = tid; j < pad.n; j += kBucketThreads) {
+    out_k[pad_at + j] = pad.kv;
+    out_v[pad_at + j] = pad.v;
+  }
   __syncthreads();  // the caller reads the output back
 }
 
@@ -1328,7 +1445,7 @@ __device__ __forceinline__ void resident_body(const Load& load, uint32_t* out_k,
 // padding run (a short batch's, which comes first among equal key variables
 // in the stable order) is written at its sorted place.
 template <class Src>
-__device__ __forceinline__ void bucket_body(const uint32_t* src_k, const uint32_t* src_v, const Src& src,
+__device__ __forceinline__ void bucket_body(uint32_t* src_k, uint32_t* src_v, const Src& src,
                                             uint32_t* out_k, uint32_t* out_v, uint32_t start, uint32_t m,
                                             const BucketRange& range, const PadRun& pad, BinRange bins, int ends,
                                             uint32_t* bsm, BucketShared& sh) {
@@ -1344,8 +1461,8 @@ __device__ __forceinline__ void bucket_body(const uint32_t* src_k, const uint32_
       const uint32_t i = threadIdx.x + j * kBucketThreads;
       if (i < m) {
         const uint32_t at = src.at(i);
-        kv[j] = src_k[at];
-        v[j] = src_v[at];
+        kv[j] = __ldg(src_k + at);  // (sort_digits of other buckets writes their own places only)
+        v[j] = __ldg(src_v + at);
       }
     }
   };
@@ -1432,8 +1549,7 @@ __global__ void __launch_bounds__(kBucketThreads) small_sort(Loader ld, uint32_t
   resident_body<true>(load, out_k, out_v, 0u, m, range, pad, bins, 3, bsm, sh);
 }
 
-__global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, const uint32_t* __restrict__ tmp_k,
-                                                              const uint32_t* __restrict__ tmp_v,
+__global__ void __launch_bounds__(kBucketThreads, 2) bucket_sort(Loader ld, uint32_t* tmp_k, uint32_t* tmp_v,
                                                               const uint2* __restrict__ runs, uint32_t* out_k,
                                                               uint32_t* out_v, const uint32_t* __restrict__ ctl,
                                                               uint32_t n, uint32_t* fence, int fshift,
@@ -1760,8 +1876,7 @@ cudaError_t bucket_sort_launch(const SortArgs& a, SortWorkspace& ws, cudaStream_
     return e;
   count_launches(1);
   if ((e = launch_pdl(bucket_sort, dim3(kRadix), dim3(kBucketThreads), kBucketSmem, st, ld,
-                      static_cast<const uint32_t*>(a.tmp_keys), static_cast<const uint32_t*>(a.tmp_vals),
-                      static_cast<const uint2*>(runs), a.out_keys, a.out_vals,
+                      a.tmp_keys, a.tmp_vals, static_cast<const uint2*>(runs), a.out_keys, a.out_vals,
                       static_cast<const uint32_t*>(ctl), a.n, a.fence, a.fshift, next, a.defer_err)) != cudaSuccess)
     return e;
   ws.flip ^= 1;

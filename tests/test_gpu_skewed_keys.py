@@ -1,0 +1,117 @@
+"""Keys that are not spread over their range (needs a GPU): results, and times that stay in proportion.
+
+The batch sort's buckets are equal parts of the range that samples of the batch span, so clusters, long tails and a few
+outliers put most of a batch in one bucket.  Comparisons of results are exact; comparisons of times have room for more
+than twice the ratio that was measured.
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOP = (1 << 31) - 1
+
+
+@pytest.fixture(scope="module")
+def g(lsm_lib):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return lsm_lib
+
+
+def draw(dist, n, rng):
+    """n keys below 2^31 - 1."""
+    if dist == "spread":
+        return rng.integers(0, TOP, n).astype(np.uint32)
+    if dist == "log":        # as many keys in every octave: three quarters of them in the lowest 256th of the range
+        return np.exp(rng.random(n) * np.log(TOP - 1)).astype(np.uint32)
+    if dist == "tail":       # ids below 2^24, one key in fifty anywhere
+        return np.where(rng.random(n) < 0.02, rng.integers(0, TOP, n), rng.integers(0, 1 << 24, n)).astype(np.uint32)
+    if dist == "clusters":   # ten clusters of 2^14 keys
+        return (rng.integers(0, TOP - (1 << 16), 10)[rng.integers(0, 10, n)] + rng.integers(0, 1 << 14, n)).astype(np.uint32)
+    if dist == "pile":       # a cluster of 2^8 keys and a long tail on both sides
+        return np.clip((1 << 30) + rng.standard_cauchy(n) * 100, 0, TOP - 1).astype(np.uint32)
+    raise ValueError(dist)
+
+
+def seconds(f, reps):
+    """Shortest of some timings of `reps` calls."""
+    f()
+    a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = 1e9
+    for _ in range(5):
+        torch.cuda.synchronize()
+        a.record()
+        for _ in range(reps):
+            f()
+        z.record()
+        z.synchronize()
+        best = min(best, a.elapsed_time(z) * 1e-3 / reps)
+    return best
+
+
+def sorter(g, dist, n, seed=5):
+    rng = np.random.default_rng(n + seed)
+    keys = (draw(dist, n, rng) << np.uint32(1)) | rng.integers(0, 2, n).astype(np.uint32)
+    lsm = g.LSM(n, n)
+    kd, vd = g.as_device_u32(keys, 0), g.as_device_u32(np.arange(n, dtype=np.uint32), 0)
+    ko, vo = torch.zeros_like(kd), torch.zeros_like(vd)
+    st = torch.cuda.current_stream().cuda_stream
+
+    def run():
+        g.lsm_sort_pairs(lsm.h, kd.data_ptr(), vd.data_ptr(), ko.data_ptr(), vo.data_ptr(), n, st)
+    return lsm, keys, ko, vo, run
+
+
+@pytest.mark.parametrize("n", [15400, 70001, 1 << 18, 1 << 20])
+@pytest.mark.parametrize("dist", ["log", "tail", "clusters", "pile"])
+def test_sort(g, dist, n):
+    lsm, keys, ko, vo, run = sorter(g, dist, n)
+    for _ in range(2):
+        run()
+        order = np.argsort(keys, kind="stable")
+        np.testing.assert_array_equal(g.to_numpy_u32(ko), keys[order])
+        np.testing.assert_array_equal(g.to_numpy_u32(vo), order.astype(np.uint32))
+    assert lsm.device_errors() == 0
+    lsm.close()
+
+
+@pytest.mark.parametrize("dist", ["log", "tail"])
+def test_sort_time_grows_with_the_batch(g, dist):
+    """Four times the keys take about four times as long, not sixteen.  (Keys whose samples span the whole range at
+    any size, so that the crowded bucket is as wide and holds the same share of the keys.)"""
+    t = []
+    for n in (1 << 18, 1 << 20):
+        lsm, _, _, _, run = sorter(g, dist, n)
+        t.append(seconds(run, 3))
+        lsm.close()
+    assert t[1] < 8.0 * t[0], t
+
+
+@pytest.mark.parametrize("short", [0, 1, 30000])
+@pytest.mark.parametrize("dist", ["log", "tail", "clusters", "pile"])
+def test_levels(g, dist, short):
+    """Batches with deletes, the last one padded, in both forms of the dictionary against the structural oracle."""
+    b, rng = 100000, np.random.default_rng(short + len(dist))
+    lsm, s, multi = g.LSM(b, 8 * b), oracle.StructuralOracle(b), g.MultiLSM([b, 33], 8)
+    for t in range(3):
+        n = b if t < 2 else b - short
+        k, v = draw(dist, n, rng), rng.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+        d = (rng.random(n) < 0.2).astype(np.uint8)
+        lsm.update(k, v, d)
+        s.call("update", k, v, d)
+        pad = [np.concatenate([x, np.zeros(b - n + 33, x.dtype)]) for x in (k, v, d)]
+        multi.update(*pad, counts=np.asarray([n, 33], np.uint32))
+    assert multi.sync()[0] == g.LSM_OK
+    for lv in (lsm.levels(), multi.levels(0)):
+        for i, (kv, vv) in lv.items():
+            ekv, ev = s.level(i)
+            np.testing.assert_array_equal(kv, ekv)
+            np.testing.assert_array_equal(vv, ev)
+    lsm.close()
+    multi.close()
