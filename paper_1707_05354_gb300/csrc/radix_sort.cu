@@ -18,6 +18,7 @@
 // puts the last of several equal key variables first (the "last insert wins"
 // reading of §III-A rule 4).
 #include "lsm_device.cuh"
+#include "sort_maps.h"
 
 namespace gpulsm {
 namespace {
@@ -445,7 +446,6 @@ constexpr int kBucketThreads = 512;
 constexpr int kBucketWarps = kBucketThreads / 32;
 constexpr int kBucketIPT = 10;
 constexpr uint32_t kBucketCap = kBucketThreads * kBucketIPT;  // 5120
-constexpr uint32_t kSubBins = 4096;      // counting pass of the bucket fast path
 constexpr uint32_t kSubBinMax = 48;      // larger sub-bins take the pass-by-pass path
 
 // The tile kernel runs 512 threads of 8 elements per 4096-element tile:
@@ -456,10 +456,7 @@ constexpr int kScatterIPT = int(kMsdTile) / kScatterThreads;  // 8
 static_assert(kScatterIPT * kScatterThreads == int(kMsdTile), "tile");
 static_assert(kMsdMaxTiles <= uint32_t(kBucketThreads), "one thread per tile run in the bucket kernel");
 
-// The buckets of one sort: `parts` equal parts of the key range, part(kv) =
-// floor((kv - lo) * mul / 2^32), and, of every hot key variable, a bucket of its
-// own, which splits the part that holds it in two: 256 in all, in key order.
-// lo, mul and the hot ones come from 512 elements taken at even distances
+// The buckets of one sort (KeyMap): 256 in all.  lo, mul and the hot ones come from 512 elements taken at even distances
 // (every CTA of the tile kernel reads the same ones): the range is the one
 // they span, widened by 1/128 at both ends (for evenly spread keys it then
 // misses elements with a probability of about e^-10 at either end, and those
@@ -474,48 +471,21 @@ constexpr uint32_t kHotSamples = 4, kMaxHot = 32, kSamples = 512;
 constexpr uint32_t kMaxSampledHot = kSamples / kHotSamples;
 constexpr int kSampleTableLog = 10, kSampleCellsLog = 12;
 constexpr uint32_t kSampleTable = 1u << kSampleTableLog, kSampleCells = 1u << kSampleCellsLog;
-struct KeyMap {
-  uint32_t lo, mul, parts, nhot;
-  const uint32_t* hot;  // ascending, in shared memory
-  __device__ __forceinline__ uint32_t part(uint32_t kv) const {
-    return min(__umulhi(max(kv, lo) - lo, mul), parts - 1);
+// Stores the smallest key variable of every bucket (threads 0 .. 255).
+__device__ __forceinline__ void store_bounds(const KeyMap& map, uint32_t* out) {
+  const uint32_t t = threadIdx.x;
+  if (t < map.parts) {
+    const uint32_t kv = t ? map.lower(t) : 0u;
+    uint32_t d = t;
+    for (uint32_t h = 0; h < map.nhot; ++h) d += map.hot[h] < kv ? 2u : 0u;
+    out[d] = kv;
   }
-  __device__ __forceinline__ uint32_t bucket(uint32_t kv) const {
-    uint32_t d = part(kv);
-    for (uint32_t h = 0; h < nhot; ++h) d += (kv >= hot[h] ? 1u : 0u) + (kv > hot[h] ? 1u : 0u);
-    return d;
+  if (t < map.nhot) {
+    const uint32_t d = map.part(map.hot[t]) + 2u * t;
+    out[d + 1] = map.hot[t];
+    out[d + 2] = map.hot[t] + 1u;
   }
-  // smallest key variable of part p in 1 .. parts - 1 (2^32 - 1 for a part the
-  // 32 bits do not reach: key variables are below it)
-  __device__ __forceinline__ uint32_t lower(uint32_t p) const {
-    return uint32_t(min(lo + ((uint64_t(p) << 32) + mul - 1) / mul, uint64_t(0xFFFFFFFFu)));
-  }
-  // `parts` parts of the range [lo, hi] that samples span, widened at both ends
-  static __device__ __forceinline__ KeyMap spanning(uint32_t lo, uint32_t hi, uint32_t parts, uint32_t nhot,
-                                                    const uint32_t* hot) {
-    const uint32_t ext = (hi - lo) / 128 + 1;
-    const uint32_t l = lo > ext ? lo - ext : 0u, h = hi < ~ext ? hi + ext : 0xFFFFFFFFu;
-    // (a float quotient: any factor near parts * 2^32 / range does, the same in
-    // every CTA; the conversion saturates)
-    const float q = __fdividef(float(parts) * 4294967296.0f, float(h - l) + 1.0f);
-    return KeyMap{l, max(1u, __float2uint_rd(q)), parts, nhot, hot};
-  }
-  // Stores the smallest key variable of every bucket (threads 0 .. 255).
-  __device__ __forceinline__ void bounds(uint32_t* out) const {
-    const uint32_t t = threadIdx.x;
-    if (t < parts) {
-      const uint32_t kv = t ? lower(t) : 0u;
-      uint32_t d = t;
-      for (uint32_t h = 0; h < nhot; ++h) d += hot[h] < kv ? 2u : 0u;
-      out[d] = kv;
-    }
-    if (t < nhot) {
-      const uint32_t d = part(hot[t]) + 2u * t;
-      out[d + 1] = hot[t];
-      out[d + 2] = hot[t] + 1u;
-    }
-  }
-};
+}
 static_assert(kRadix == 256 && 2 * kMaxHot < kRadix, "the hot keys' buckets leave parts over");
 static_assert(kSamples == uint32_t(kScatterThreads), "one sample a thread");
 static_assert(kSampleTable == 2 * kSamples && 2 * kSampleTable == 4 * uint32_t(kScatterThreads) &&
@@ -671,7 +641,7 @@ __global__ void __maxnreg__(48) msd_tile(Loader ld, uint32_t* __restrict__ tmp_k
   if (tid == 0) check.done(ctl, any_bad != 0);
   const KeyMap map = sample_map(sample, n - npad, s_keys, s_vals, s_sample);
   if (tile == gridDim.x - 1) {  // the last tile's CTA (the shortest) publishes the buckets' bounds
-    map.bounds(ctl + kSortCtlBounds);
+    store_bounds(map, ctl + kSortCtlBounds);
     if (tid == kRadix) {
       ctl[kSortCtlMap] = map.lo;
       ctl[kSortCtlMap + 1] = map.mul;
@@ -736,25 +706,6 @@ __device__ __forceinline__ uint32_t lower_bound_sorted(const uint32_t* a, uint32
 
 // A bucket: its elements' key variables lie in [lo, hi]; `map` spreads them
 // over the sub-bins of the counting pass.
-// Sub-bin of kv: floor((kv - off) * mul / 2^32), for kv below base as for
-// base, kept below kSubBins; monotone.
-struct SubMap {
-  uint32_t base, off, mul;
-  // `width` key variables from base: for up to kSubBins of them each has a
-  // sub-bin of its own (off = base - 1: (x + 1) (2^32 - 1) / 2^32 is x)
-  static __device__ __forceinline__ SubMap of(uint32_t base, float width) {
-    if (width <= float(kSubBins)) return SubMap{base, base - 1u, 0xFFFFFFFFu};
-    return SubMap{base, base, __float2uint_rd(__fdividef(float(1ull << 44), width))};
-  }
-  __device__ __forceinline__ uint32_t sub(uint32_t kv) const {
-    return min(__umulhi(max(kv, base) - off, mul), kSubBins - 1);
-  }
-  // the largest key variable of sub-bin s
-  __device__ __forceinline__ uint32_t last(uint32_t s) const {
-    return off + uint32_t(((uint64_t(s + 1) << 32) + mul - 1) / mul) - 1;
-  }
-};
-static_assert(kSubBins == 4096, "2^44 = kSubBins * 2^32");
 struct BucketRange {
   uint32_t lo, hi;
   SubMap map;
@@ -1102,7 +1053,7 @@ __device__ __noinline__ void sort_digits(uint32_t* src_k, uint32_t* src_v, const
 }
 
 // A bucket above kBucketCap elements: taken in key order, a part at a time.
-// Each round looks at the elements of [a, b], the keys still to do:
+// Each round looks at the elements of [a, b], the keys still to do (KeyTurn):
 //   at most kBucketCap of them        gathered in order, sorted, written;
 //   all but at most kBucketCap have   the hot key's tombstones and regular
 //   one key (a hot key)               elements go straight to their places in
@@ -1180,8 +1131,10 @@ __device__ __noinline__ void sort_big(uint32_t* src_k, uint32_t* src_v, const Sr
     __syncthreads();
     pad_at += sh.cnt[0];
   }
-  uint32_t a = range.lo, b = range.hi, done = 0;
+  KeyTurn turn;
+  uint32_t done = 0;
   while (done < m) {
+    const uint32_t a = turn.a, b = turn.b;
     // A key that may be hot: the most frequent one within a warp among 512
     // elements taken at even distances.
     __syncthreads();
@@ -1242,8 +1195,7 @@ __device__ __noinline__ void sort_big(uint32_t* src_k, uint32_t* src_v, const Sr
     tombs = 0;
     for (int w = 0; w < kBucketWarps; ++w) tombs += sh.excl[w];
     if (c == 0) {  // (only below an upper part that is still to do)
-      a = b + 1;
-      b = range.hi;
+      turn.next();
       continue;
     }
     if (mn == mx) {  // one key variable (the candidate may be another key)
@@ -1288,8 +1240,7 @@ __device__ __noinline__ void sort_big(uint32_t* src_k, uint32_t* src_v, const Sr
       if (fit) atomicMax(&sh.max, fit);
       __syncthreads();
       fit = sh.max;
-      a = mn;
-      b = map.last(fit ? fit - 1 : 0u);
+      turn.narrow(mn, map, fit);
       continue;
     }
     if (c <= kBucketCap) copies = tombs = 0;  // all of them fit: no key is singled out
@@ -1373,8 +1324,7 @@ __device__ __noinline__ void sort_big(uint32_t* src_k, uint32_t* src_v, const Sr
       });
     }
     done += c;
-    a = b + 1;
-    b = range.hi;
+    turn.next();
   }
   __syncthreads();  // (the passes use the padding's places)
   for (uint32_t j = tid; j < pad.n; j += kBucketThreads) {

@@ -1,0 +1,96 @@
+// Key arithmetic of the batch sort: which bucket and sub-bin a key variable
+// falls in, and which keys a round over a crowded bucket takes.  Plain integer
+// functions without CUDA constructs, so that they can be checked on the host.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define GPULSM_HD __host__ __device__ __forceinline__
+#else
+#define GPULSM_HD inline
+#endif
+
+namespace gpulsm {
+
+GPULSM_HD uint32_t mul_hi(uint32_t a, uint32_t b) { return uint32_t((uint64_t(a) * b) >> 32); }
+GPULSM_HD uint32_t lesser(uint32_t a, uint32_t b) { return a < b ? a : b; }
+GPULSM_HD uint32_t greater(uint32_t a, uint32_t b) { return a < b ? b : a; }
+// a / b rounded down to a whole number below 2^32 (larger quotients become
+// 2^32 - 1); the device's quotient may be off by a few units in the last place.
+GPULSM_HD uint32_t floor_quotient(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __float2uint_rd(__fdividef(a, b));
+#else
+  const float q = a / b;
+  return q >= 4294967296.0f ? 0xFFFFFFFFu : uint32_t(q);
+#endif
+}
+
+// The buckets of one sort: `parts` equal parts of the key range, part(kv) =
+// floor((kv - lo) * mul / 2^32), and, of every hot key variable, a bucket of its
+// own, which splits the part that holds it in two: in key order.
+struct KeyMap {
+  uint32_t lo, mul, parts, nhot;
+  const uint32_t* hot;  // ascending
+  GPULSM_HD uint32_t part(uint32_t kv) const { return lesser(mul_hi(greater(kv, lo) - lo, mul), parts - 1); }
+  GPULSM_HD uint32_t bucket(uint32_t kv) const {
+    uint32_t d = part(kv);
+    for (uint32_t h = 0; h < nhot; ++h) d += (kv >= hot[h] ? 1u : 0u) + (kv > hot[h] ? 1u : 0u);
+    return d;
+  }
+  // smallest key variable of part p in 1 .. parts - 1 (2^32 - 1 for a part the
+  // 32 bits do not reach: key variables are below it)
+  GPULSM_HD uint32_t lower(uint32_t p) const {
+    const uint64_t kv = lo + ((uint64_t(p) << 32) + mul - 1) / mul;
+    return kv < 0xFFFFFFFFull ? uint32_t(kv) : 0xFFFFFFFFu;
+  }
+  // `parts` parts of the range [lo, hi] that samples span, widened at both ends
+  static GPULSM_HD KeyMap spanning(uint32_t lo, uint32_t hi, uint32_t parts, uint32_t nhot, const uint32_t* hot) {
+    const uint32_t ext = (hi - lo) / 128 + 1;
+    const uint32_t l = lo > ext ? lo - ext : 0u, h = hi < ~ext ? hi + ext : 0xFFFFFFFFu;
+    // (a float quotient: any factor near parts * 2^32 / range does, the same in
+    // every CTA)
+    const uint32_t q = floor_quotient(float(parts) * 4294967296.0f, float(h - l) + 1.0f);
+    return KeyMap{l, greater(1u, q), parts, nhot, hot};
+  }
+};
+
+// Sub-bin of kv: floor((kv - off) * mul / 2^32), for kv below base as for
+// base, kept below kSubBins; monotone.
+constexpr uint32_t kSubBins = 4096;  // counting pass over a bucket's elements
+struct SubMap {
+  uint32_t base, off, mul;
+  // `width` key variables from base: for up to kSubBins of them each has a
+  // sub-bin of its own (off = base - 1: (x + 1) (2^32 - 1) / 2^32 is x)
+  static GPULSM_HD SubMap of(uint32_t base, float width) {
+    if (width <= float(kSubBins)) return SubMap{base, base - 1u, 0xFFFFFFFFu};
+    return SubMap{base, base, floor_quotient(float(1ull << 44), width)};
+  }
+  GPULSM_HD uint32_t sub(uint32_t kv) const { return lesser(mul_hi(greater(kv, base) - off, mul), kSubBins - 1); }
+  // the largest key variable of sub-bin s
+  GPULSM_HD uint32_t last(uint32_t s) const {
+    return off + uint32_t(((uint64_t(s + 1) << 32) + mul - 1) / mul) - 1;
+  }
+};
+static_assert(kSubBins == 4096, "2^44 = kSubBins * 2^32");
+
+// The keys [a, b] that the rounds over a crowded bucket have still to do: at
+// first all keys there are, whatever range the bucket is said to have, so that
+// every element has its turn and the rounds end.
+struct KeyTurn {
+  uint32_t a = 0u, b = 0xFFFFFFFFu;
+  // The next round takes the elements' range [mn, mx] in sub-bins and looks at
+  // the first `fit` of them (at least one; fewer than reach mx).
+  GPULSM_HD void narrow(uint32_t mn, const SubMap& map, uint32_t fit) {
+    a = mn;
+    b = map.last(fit ? fit - 1 : 0u);
+  }
+  // [a, b] is done.
+  GPULSM_HD void next() {
+    a = b + 1;
+    b = 0xFFFFFFFFu;
+  }
+};
+
+}  // namespace gpulsm
