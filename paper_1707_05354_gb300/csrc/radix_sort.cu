@@ -456,13 +456,12 @@ constexpr int kScatterIPT = int(kMsdTile) / kScatterThreads;  // 8
 static_assert(kScatterIPT * kScatterThreads == int(kMsdTile), "tile");
 static_assert(kMsdMaxTiles <= uint32_t(kBucketThreads), "one thread per tile run in the bucket kernel");
 
-// The buckets of one sort (KeyMap): 256 in all.  lo, mul and the hot ones come from 512 elements taken at even distances
-// (every CTA of the tile kernel reads the same ones): the range is the one
-// they span, widened by 1/128 at both ends (for evenly spread keys it then
-// misses elements with a probability of about e^-10 at either end, and those
-// fall in the first or last bucket); hot is what comes up kHotSamples times or
-// more, about 0.8 % of the batch, and would overflow a bucket of 2^20 / 256
-// elements.
+// The buckets of one sort (KeyMap): 256 in all.  lo, mul and the hot ones come
+// from 512 elements taken at even distances (every CTA of the tile kernel reads
+// the same ones): the range is the one they span, widened at both ends (elements
+// beyond it fall in the first or last bucket); hot is what comes up kHotSamples
+// times or more, about 0.8 % of the batch, and would overflow a bucket of
+// 2^20 / 256 elements.
 // With the top byte as the bucket, batches of 2^18 ids below 2^25 took 553 us
 // in bucket_sort and 2^20 keys below 2^30 154 us; now 21.7 and 21.3 us.  Without
 // buckets for the hot keys a sort of 2^18 Zipf(1.1) pairs took 63 us, of 2^20

@@ -45,9 +45,14 @@ struct KeyMap {
     const uint64_t kv = lo + ((uint64_t(p) << 32) + mul - 1) / mul;
     return kv < 0xFFFFFFFFull ? uint32_t(kv) : 0xFFFFFFFFu;
   }
-  // `parts` parts of the range [lo, hi] that samples span, widened at both ends
+  // `parts` parts of the range [lo, hi] that 512 samples span, widened by 1/50
+  // at both ends: evenly spread keys reach beyond it with a probability of
+  // about e^-10 at either end, 512 / 50.  (What does falls in the first or last
+  // sub-bin; more than a few there and the bucket takes 8-bit passes.  With
+  // 1/128, e^-4, that was one batch in fifty at either end: four rounds of 34
+  // batches of 30000 took 256 us, now 244; one sort of 2^20 24.9 and 25.0.)
   static GPULSM_HD KeyMap spanning(uint32_t lo, uint32_t hi, uint32_t parts, uint32_t nhot, const uint32_t* hot) {
-    const uint32_t ext = (hi - lo) / 128 + 1;
+    const uint32_t ext = (hi - lo) / 50 + 1;
     const uint32_t l = lo > ext ? lo - ext : 0u, h = hi < ~ext ? hi + ext : 0xFFFFFFFFu;
     // (a float quotient: any factor near parts * 2^32 / range does, the same in
     // every CTA)

@@ -76,3 +76,49 @@ def test_rounds_end_for_any_keys(tmp_path):
     out = run(tmp_path, ROUNDS, *cases)
     for c, o in zip(cases, out):
         assert o.isdigit() and int(o) <= 8 * (c[0] // c[1] + 2) + min(c[0], 4 * (c[3] - c[2] + 1)), (c, o)
+
+
+# Of 1000 batches of n keys spread evenly from lo to hi, those with more than `few` keys beyond the range that the map of
+# 512 samples covers.
+COVER = r"""
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+#include "sort_maps.h"
+using namespace gpulsm;
+int main(int argc, char** argv) {
+  const uint32_t n = strtoul(argv[1], 0, 0), lo = strtoul(argv[2], 0, 0), hi = strtoul(argv[3], 0, 0),
+                 few = strtoul(argv[4], 0, 0);
+  uint64_t s = 88172645463325252ull;
+  std::vector<uint32_t> x(n);
+  int bad = 0;
+  for (int t = 0; t < 1000; ++t) {
+    for (auto& k : x) {
+      s ^= s << 13; s ^= s >> 7; s ^= s << 17;
+      k = lo + uint32_t((s >> 20) % (uint64_t(hi) - lo + 1));
+    }
+    uint32_t mn = ~0u, mx = 0;
+    for (uint64_t e = 0; e < 512; ++e) {
+      mn = std::min(mn, x[e * n / 512]);
+      mx = std::max(mx, x[e * n / 512]);
+    }
+    const KeyMap m = KeyMap::spanning(mn, mx, 256, 0, nullptr);
+    uint32_t below = 0, above = 0;
+    for (uint32_t k : x) {
+      below += k < m.lo;
+      above += k > m.lo && mul_hi(k - m.lo, m.mul) >= m.parts;
+    }
+    bad += below > few || above > few;
+  }
+  printf("%d\n", bad);
+}
+"""
+
+
+def test_sampled_range_covers_even_keys(tmp_path):
+    """More than the 48 keys that a sub-bin may hold are beyond the range in about two of e^10 = 22000 batches; three of
+    1000 would be there with a probability of 10^-4."""
+    cases = [(30000, 1 << 29, 5 << 29, 48), (1 << 17, 0, 1 << 31, 48), (30000, 1 << 20, 1 << 25, 48)]
+    for c, o in zip(cases, run(tmp_path, COVER, *cases)):
+        assert int(o) <= 2, (c, o)
