@@ -1578,7 +1578,7 @@ __global__ void __launch_bounds__(256) check_keys(const uint32_t* __restrict__ k
 // The batch sort of the batched form: the same bucket scheme on every
 // instance's batch at once.  Instance i splits the key range of its batch, by
 // 512 samples of it that every CTA of mseg_count reads, in 2^d_i parts of about
-// 4096 elements (KeyMap; without hot keys); its batch is cut into
+// 4096 elements (PartMap; without hot keys); its batch is cut into
 // kMultiSortTile-element tiles; one launch per phase covers every tile or
 // bucket of every instance.  Instances without a batch this round (count 0,
 // or refused by the prep kernel) leave at once.
@@ -1661,11 +1661,11 @@ __global__ void __launch_bounds__(kThreads) mseg_count(MultiArena ar, MultiBatch
   }
   __syncthreads();
   const uint32_t w = lane_id() & uint32_t(kWarps - 1);
-  const KeyMap map = KeyMap::spanning(__reduce_min_sync(0xffffffffu, s_mn[w]), __reduce_max_sync(0xffffffffu, s_mx[w]),
-                                      1u << d.msd_bits, 0u, nullptr);
+  const PartMap map = PartMap::spanning(__reduce_min_sync(0xffffffffu, s_mn[w]),
+                                        __reduce_max_sync(0xffffffffu, s_mx[w]), d.msd_bits);
   if (t0 == 0 && tid == 0) {
-    ar.map[2 * i] = map.lo;
-    ar.map[2 * i + 1] = map.mul;
+    ar.map[2 * i] = map.fine.lo;
+    ar.map[2 * i + 1] = map.fine.mul;
   }
 #pragma unroll
   for (int j = 0; j < kMultiIPT; ++j)
@@ -1699,7 +1699,7 @@ __global__ void __launch_bounds__(kThreads) mseg_offsets(MultiArena ar) {
     }
     ar.bstart[d.bucket0 + tid] = start;
     ar.bcnt[d.bucket0 + tid] = total;
-    const KeyMap map{ar.map[2 * i], ar.map[2 * i + 1], nbk, 0u, nullptr};
+    const PartMap map = PartMap::of(ar.map[2 * i], ar.map[2 * i + 1], d.msd_bits);
     ar.blo[d.bucket0 + tid] = tid ? map.lower(tid) : 0u;
   }
 }
@@ -1716,7 +1716,7 @@ __global__ void __launch_bounds__(kScatterThreads) mseg_scatter(MultiArena ar, M
   const uint32_t nops = multi_ops(in, d, i);
   const uint32_t t0 = (gt - d.stile0) * kMultiSortTile;
   const uint32_t m = (d.b - t0) < kMultiSortTile ? (d.b - t0) : kMultiSortTile;
-  const KeyMap map{ar.map[2 * i], ar.map[2 * i + 1], 1u << d.msd_bits, 0u, nullptr};
+  const PartMap map = PartMap::of(ar.map[2 * i], ar.map[2 * i + 1], d.msd_bits);
   const uint32_t base = warp * (32 * kScatterIPT);
   uint32_t kv[kScatterIPT], v[kScatterIPT], rank[kScatterIPT];
   bool bad_any = false;  // (mseg_count has seen them)
@@ -1781,8 +1781,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) mseg_bucket(MultiArena ar) 
   const bool top = bucket == (1u << d.msd_bits) - 1;
   const uint32_t lo = ar.blo[gb], next = top ? 0xFFFFFFFFu : ar.blo[gb + 1];
   const uint32_t hi = next == 0xFFFFFFFFu ? next : next - 1;
-  const BucketRange range{lo, hi, SubMap::of(bucket ? lo : ar.map[2 * i],
-                                             __fdividef(4294967296.0f, float(ar.map[2 * i + 1])) + 1.0f)};
+  const BucketRange range{lo, hi, SubMap::of(bucket ? lo : ar.map[2 * i], PartMap::width(ar.map[2 * i + 1], d.msd_bits))};
   const BinRange bins{of, fs, bucket ? ((lo - 1) >> fs) + 1 : 0u, (hi >> fs) + 1};
   bucket_body(tk, tv, ContigSrc{start}, ok, ov, start, m, range, PadRun{0u, 0u, 0u}, bins, 0, bsm, sh);
   if (top && threadIdx.x == 0) {

@@ -16,13 +16,20 @@ namespace gpulsm {
 GPULSM_HD uint32_t mul_hi(uint32_t a, uint32_t b) { return uint32_t((uint64_t(a) * b) >> 32); }
 GPULSM_HD uint32_t lesser(uint32_t a, uint32_t b) { return a < b ? a : b; }
 GPULSM_HD uint32_t greater(uint32_t a, uint32_t b) { return a < b ? b : a; }
-// a / b rounded down to a whole number below 2^32 (larger quotients become
-// 2^32 - 1); the device's quotient may be off by a few units in the last place.
+// a / b; the device's quotient may be off by a few units in the last place.
+GPULSM_HD float quotient(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(a, b);
+#else
+  return a / b;
+#endif
+}
+// The same rounded down to a whole number (from 2^32 on: 2^32 - 1).
 GPULSM_HD uint32_t floor_quotient(float a, float b) {
 #ifdef __CUDA_ARCH__
-  return __float2uint_rd(__fdividef(a, b));
+  return __float2uint_rd(quotient(a, b));
 #else
-  const float q = a / b;
+  const float q = quotient(a, b);
   return q >= 4294967296.0f ? 0xFFFFFFFFu : uint32_t(q);
 #endif
 }
@@ -58,6 +65,27 @@ struct KeyMap {
     // every CTA)
     const uint32_t q = floor_quotient(float(parts) * 4294967296.0f, float(h - l) + 1.0f);
     return KeyMap{l, greater(1u, q), parts, nhot, hot};
+  }
+};
+
+// Few equal parts, 2^bits <= 256 of them: runs of the parts of a map of 256.
+// (The factor of a map of two parts over nearly 2^32 keys is 2 or 3, whole, so
+// that one of them could get two thirds of the range and overflow: four rounds
+// of 128 batches of 8192 keys below 2^30 took 435 us, now 252.)
+struct PartMap {
+  KeyMap fine;
+  uint32_t drop;
+  static GPULSM_HD PartMap of(uint32_t lo, uint32_t mul, uint32_t bits) {
+    return PartMap{KeyMap{lo, mul, 256u, 0u, nullptr}, 8u - bits};
+  }
+  static GPULSM_HD PartMap spanning(uint32_t lo, uint32_t hi, uint32_t bits) {
+    return PartMap{KeyMap::spanning(lo, hi, 256u, 0u, nullptr), 8u - bits};
+  }
+  GPULSM_HD uint32_t part(uint32_t kv) const { return fine.part(kv) >> drop; }
+  GPULSM_HD uint32_t lower(uint32_t p) const { return fine.lower(p << drop); }
+  // about the key variables of a part
+  static GPULSM_HD float width(uint32_t mul, uint32_t bits) {
+    return quotient(1099511627776.0f, float(mul) * float(1u << bits)) + 1.0f;
   }
 };
 

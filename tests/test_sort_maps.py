@@ -122,3 +122,37 @@ def test_sampled_range_covers_even_keys(tmp_path):
     cases = [(30000, 1 << 29, 5 << 29, 48), (1 << 17, 0, 1 << 31, 48), (30000, 1 << 20, 1 << 25, 48)]
     for c, o in zip(cases, run(tmp_path, COVER, *cases)):
         assert int(o) <= 2, (c, o)
+
+
+# The largest part of the batched form's map over keys spread evenly from lo to hi, in percent of an even share, or what
+# is wrong with the parts' bounds.
+PARTS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "sort_maps.h"
+using namespace gpulsm;
+int main(int argc, char** argv) {
+  const uint32_t lo = strtoul(argv[1], 0, 0), hi = strtoul(argv[2], 0, 0), bits = strtoul(argv[3], 0, 0), n = 1u << bits;
+  const PartMap m = PartMap::spanning(lo, hi, bits);
+  uint64_t most = 0;
+  for (uint32_t p = 0; p < n; ++p) {
+    const uint64_t a = p ? m.lower(p) : 0, z = p + 1 < n ? m.lower(p + 1) : 1ull << 32;
+    if (a < 0xFFFFFFFFull && z > a && (m.part(uint32_t(a)) != p || m.part(uint32_t(z - 1)) != p)) {
+      if (z != 0xFFFFFFFFull) return puts("bounds"), 0;
+    }
+    const uint64_t x = a < lo ? lo : a, y = z > uint64_t(hi) + 1 ? uint64_t(hi) + 1 : z;
+    if (y > x && y - x > most) most = y - x;
+  }
+  printf("%.1f\n", 100.0 * double(most) * n / (double(hi) - lo + 1));
+}
+"""
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3, 8])
+def test_parts_are_even(tmp_path, bits):
+    """A part is at most 5 % above its share: the range is widened by 1/50 at both ends (4 %), the factor rounded down by
+    1/256 at most (0.4 %), and a bound to a whole key (of 780 at least)."""
+    cases = [(lo, hi, bits) for lo, hi in ((0, 0xFFFFFFFE), (0, 1 << 31), (0, 3200000000), (1 << 30, 3 << 30),
+                                           (0, 0xC0000000), (12345, 0x70000000), (0, 1 << 25), (77, 200000))]
+    for c, o in zip(cases, run(tmp_path, PARTS, *cases)):
+        assert float(o) <= 105.0, (c, o)
