@@ -206,7 +206,6 @@ lsm_status lsm_multi_create(lsm_multi_t** out, uint32_t n_inst, const uint32_t* 
       foff += rup(fence_words(d.lvl_fshift[l]), 64);
     }
     d.fshift0 = d.lvl_fshift[0];
-    if (32 - int(d.msd_bits) < d.fshift0) return LSM_ERR_ARG;  // a bucket spans whole bins
     d.batch_fence = foff;
     foff += rup(fence_words(d.fshift0), 64);
     part_words += ((uint64_t(b) << (L - 1)) + tile - 1) / tile + 1;
