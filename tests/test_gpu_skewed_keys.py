@@ -115,3 +115,31 @@ def test_levels(g, dist, short):
             np.testing.assert_array_equal(vv, ev)
     lsm.close()
     multi.close()
+
+
+@pytest.mark.parametrize("sizes", [[1, 7, 8, 9], [63, 64, 65], [66, 200, 5000], [3, 64, 65, 1000]])
+@pytest.mark.parametrize("shape", ["low", "high", "spread", "both"])
+def test_searches_in_crowded_bins(g, sizes, shape):
+    """Bins of the prefix index (2^15 keys wide here) of chosen sizes, with the keys at either end of the bin or spread
+    over it: lookups and counts at every key, beside it and between the bins."""
+    rng = np.random.default_rng(sum(sizes) + len(shape))
+    keys = []
+    for i, m in enumerate(sizes * 6):
+        x = {"low": np.arange(m), "high": (1 << 15) - 1 - np.arange(m), "spread": rng.choice(1 << 15, m, replace=False),
+             "both": np.concatenate([np.arange(m // 2), (1 << 15) - 1 - np.arange(m - m // 2)])}[shape]
+        keys.append(((3 * i + 1) << 15) + x)
+    keys = np.sort(np.concatenate(keys + [[TOP - 1]])).astype(np.uint32)
+    vals = rng.integers(0, 1 << 31, len(keys)).astype(np.uint32)
+    lsm = g.LSM(len(keys), len(keys))
+    lsm.bulk_build(keys, vals)
+    q = np.unique(np.concatenate([keys, keys - 1, keys + 1, np.arange(0, TOP, 1 << 22), [0, TOP - 1, TOP]])).astype(np.uint32)
+    at = np.minimum(np.searchsorted(keys, q), len(keys) - 1)
+    hit = keys[at] == q
+    val, found = lsm.lookup(q)
+    np.testing.assert_array_equal(found.cpu().numpy(), hit.astype(np.uint8))
+    np.testing.assert_array_equal(g.to_numpy_u32(val), np.where(hit, vals[at], 0))
+    k1 = q[q < TOP]
+    k2 = np.minimum(k1.astype(np.int64) + rng.integers(0, 70000, len(k1)), TOP - 1).astype(np.uint32)
+    want = np.searchsorted(keys, k2, side="right") - np.searchsorted(keys, k1)
+    np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), want)
+    lsm.close()
