@@ -626,6 +626,106 @@ __device__ __forceinline__ uint32_t lower_bound_smem(const uint32_t* a, uint32_t
   return lo;
 }
 
+// Windows in which most keys repeat (many stale versions in each level): the
+// versions are skipped instead of read.  A group of lanes, one per level, takes
+// the keys of its part of the windows one after another: the smallest head
+// among the lanes is the next key, the newest level's element decides, and
+// every lane whose head it is goes to the end of its run, whose length is
+// guessed from the run before.  The parts are cut at even places of the largest
+// window.  Key `past` has been decided already.  Result as wide_merge in x, the
+// number of runs in y; kEmit: the parts' counts come from a first pass.  Bound
+// by the chain of loads, a few per key and level.
+template <bool kEmit>
+__device__ __forceinline__ uint2 repeat_merge(const LevelSet& ls, uint32_t pos, uint32_t end, uint32_t past,
+                                              uint32_t* out_k, uint32_t* out_v, uint64_t room) {
+  const uint32_t lane = lane_id();
+  uint32_t width = 1;  // lanes of a group
+  while (width < uint32_t(ls.count)) width *= 2;
+  const uint32_t l = lane & (width - 1), part = lane / width, parts = 32 / width;
+  const bool act = l < uint32_t(ls.count);
+  const uint32_t *keys = act ? ls.keys[l] : nullptr, *vals = act ? ls.vals[l] : nullptr;
+  // the part's start in every level, and the next part's
+  const uint32_t most = __reduce_max_sync(0xffffffffu, end - pos);
+  const int big = __ffs(int(__ballot_sync(0xffffffffu, end - pos == most))) - 1;
+  const uint32_t cut = __shfl_sync(0xffffffffu, pos, big) + uint32_t(uint64_t(most) * part / parts);
+  const uint32_t from = part ? key_of(__ldg(ls.keys[big] + cut)) : 0u;
+  const uint32_t p = __shfl_sync(0xffffffffu, pos, int(l)), e = __shfl_sync(0xffffffffu, end, int(l));
+  const uint32_t start = act ? (part ? lower_bound_kv(keys, p, e, from << 1) : p) : 0u;
+  const uint32_t next = __shfl_down_sync(0xffffffffu, start, width);
+  const uint32_t stop = act ? (part + 1 < parts ? next : e) : 0u;
+  uint32_t before = 0, live = 0, runs = 0;
+#pragma unroll 1
+  for (int pass = kEmit ? 0 : 1; pass < 2; ++pass) {
+    uint32_t cur = start, run = 1;
+    uint32_t kv = cur < stop ? __ldg(keys + cur) : 0xFFFFFFFFu;
+    uint32_t value = 0, *to_value = nullptr;  // of the last key emitted: stored with the next one
+    live = runs = 0;
+    for (;;) {
+      const uint32_t head = cur < stop ? key_of(kv) : 0xFFFFFFFFu;
+      uint32_t k = head;
+      for (uint32_t o = 1; o < width; o <<= 1) k = min(k, __shfl_xor_sync(0xffffffffu, k, int(o)));
+      if (!__any_sync(0xffffffffu, k != 0xFFFFFFFFu)) break;
+      const bool mine = head == k && k != 0xFFFFFFFFu;
+      const uint32_t who = __ballot_sync(0xffffffffu, mine), live_who = __ballot_sync(0xffffffffu, mine && (kv & 1u));
+      const uint32_t group = who & (0xffffffffu >> (32 - width)) << (part * width);
+      const uint32_t newest = group & (0u - group);  // its lane's bit
+      if ((live_who & newest) && k != past) {
+        if (kEmit && pass && newest == 1u << lane && before + live < room) {
+          out_k[before + live] = k;
+          if (to_value) *to_value = value;
+          to_value = out_v + before + live;
+          value = __ldg(vals + cur);
+        }
+        ++live;
+      }
+      if (mine) {  // past the run: [cur, at] are of it, kv becomes the element at `to`, which is not
+        uint32_t at = cur, to = cur + run;
+        for (; to < stop; run *= 2) {
+          kv = __ldg(keys + to);
+          if (key_of(kv) != k) break;
+          at = to;
+          to += run;
+        }
+        to = min(to, stop);
+        while (to - at > 1) {
+          const uint32_t mid = at + (to - at) / 2, x = __ldg(keys + mid);
+          if (key_of(x) == k) {
+            at = mid;
+          } else {
+            to = mid;
+            kv = x;
+          }
+        }
+        run = to - cur;
+        cur = to;
+        ++runs;
+      }
+    }
+    if (to_value) *to_value = value;
+    const uint32_t share = l == 0 ? live : 0u;
+    const uint32_t sum = warp_incl_scan(share);
+    before = __shfl_sync(0xffffffffu, sum - share, int(part * width));
+    live = __shfl_sync(0xffffffffu, sum, 31);
+  }
+  return make_uint2(live, warp_sum(runs));
+}
+
+// When kSame of 32 elements of a piece have the key of the one before, or after
+// kAlone keys that fill a piece alone, the next kReach elements are taken by
+// repeat_merge, then four times as many, while they have kRepeats per run; when
+// they do not, it takes more to come back to it.  One level, which is read
+// straight through, when 32 elements in a row have one key, and kRepeatsOne per
+// run.
+// (31 batches of 2^18 keys below 2^16, about 24 copies of a key per level:
+// 65536 counts of 64 keys 4690 us read piece by piece, now about 560, ranges
+// 16.1 and 2.5 ms; 256 counts of 50000 keys 225 and 19 ms.  One level of 2^24
+// with 256 copies: 65536 counts of 64 keys 1315 and 355 us.  Zipf keys, of which
+// most runs are short, lose by skipping: 8192 ranges of 1000 keys 430 us read,
+// 650 with what is tried and given up.  The tests themselves cost spread keys
+// 1 %: range_wide needs 64 registers instead of 48, without which the value of
+// a key found is waited for.)
+constexpr uint32_t kSame = 24, kRepeats = 3, kRepeatsOne = 32, kAlone = 6, kReach = 1024, kMaxReach = 1u << 24;
+
 // Live keys of the windows [pos, end) (lane l holds level l's), emitted to
 // out_k/out_v in key order when kEmit (at most `room`); returns their number.
 template <class Shared>
@@ -636,44 +736,50 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
   const int nl = ls.count;
   const bool act = lane < uint32_t(nl);
   const uint32_t* keys = act ? ls.keys[lane] : nullptr;
-  uint32_t done = 0;
-  if (nl == 1) {  // nothing to look for in other levels: the window is read through, in order
-    const uint32_t last = __shfl_sync(0xffffffffu, end, 0), lt = lanemask_lt();
-    uint32_t before = 0xFFFFFFFFu;  // key before the chunk
-    for (uint32_t i0 = __shfl_sync(0xffffffffu, pos, 0); i0 < last;) {
-      uint32_t kv[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t i = i0 + 32 * j + lane;
-        kv[j] = i < last ? __ldg(ls.keys[0] + i) : 0xFFFFFFFEu;  // (no regular element)
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t k = key_of(kv[j]), up = __shfl_up_sync(0xffffffffu, k, 1);
-        const bool ok = (kv[j] & 1u) && k != (lane ? up : before);
-        before = __shfl_sync(0xffffffffu, k, 31);
-        const uint32_t m = __ballot_sync(0xffffffffu, ok), at = done + __popc(m & lt);
-        if (kEmit && ok && at < room) {
-          out_k[at] = k;
-          out_v[at] = __ldg(ls.vals[0] + (i0 + 32 * j + lane));
-        }
-        done += __popc(m);
-      }
-      i0 += 128;
-      // a long run of one key (a short batch's padding): past its end
-      if (i0 < last && __shfl_sync(0xffffffffu, key_of(kv[0]), 0) == before)
-        i0 = upper_bound_key(ls.keys[0], i0, last, before);
-    }
-    return done;
-  }
+  const uint32_t per_run = nl == 1 ? kRepeatsOne : kRepeats;
+  uint32_t done = 0, alone = 0, enter = nl == 1 ? 31u : kSame, past = 0xFFFFFFFFu;
+  uint32_t reach = 0;  // elements that repeat_merge takes next, 0 when it does not
   for (;;) {
+    if (nl == 1 && reach == 0) {  // nothing to look for in other levels: the window is read through, in order
+      const uint32_t last = __shfl_sync(0xffffffffu, end, 0), lt = lanemask_lt();
+      uint32_t before = past;  // key before the chunk
+      uint32_t i0 = __shfl_sync(0xffffffffu, pos, 0);
+      while (i0 < last && reach == 0) {
+        uint32_t kv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t i = i0 + 32 * j + lane;
+          kv[j] = i < last ? __ldg(ls.keys[0] + i) : 0xFFFFFFFEu;  // (no regular element)
+        }
+        uint32_t same = 0;  // of the first 32, those with the key of the one before
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t k = key_of(kv[j]), up = __shfl_up_sync(0xffffffffu, k, 1);
+          const bool first = k != (lane ? up : before), ok = (kv[j] & 1u) && first;
+          if (j == 0) same = 32u - __popc(__ballot_sync(0xffffffffu, first));
+          before = __shfl_sync(0xffffffffu, k, 31);
+          const uint32_t m = __ballot_sync(0xffffffffu, ok), at = done + __popc(m & lt);
+          if (kEmit && ok && at < room) {
+            out_k[at] = k;
+            out_v[at] = __ldg(ls.vals[0] + (i0 + 32 * j + lane));
+          }
+          done += __popc(m);
+        }
+        i0 += 128;
+        if (same >= enter && i0 + 128 < last) reach = kReach;
+      }
+      if (i0 >= last) return done;
+      pos = lane ? 0u : i0;
+      past = before;
+    }
     const uint32_t left = act ? end - pos : 0u;
     const uint32_t total = warp_sum(left);
     if (total == 0) return done;
     // this piece: [pos, pos + n) of every level
     uint32_t n = left;
-    if (total > kWideCap) {
-      const uint32_t share = kWideCap / uint32_t(nl);
+    const uint32_t cap = max(reach, kWideCap);
+    if (total > cap) {
+      const uint32_t share = cap / uint32_t(nl);
       const uint32_t lim = __reduce_min_sync(0xffffffffu, left > share ? key_of(__ldg(keys + pos + share)) : 0xFFFFFFFFu);
       n = left ? lower_bound_kv(keys, pos, pos + min(left, share), lim << 1) - pos : 0u;
       if (!__any_sync(0xffffffffu, n != 0u)) {
@@ -683,7 +789,7 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
         const uint32_t has = __ballot_sync(0xffffffffu, left && key_of(first) == lim);
         const int newest = __ffs(int(has)) - 1;
         const bool live = (__shfl_sync(0xffffffffu, first, newest) & 1u) != 0u;
-        if (live) {
+        if (live && lim != past) {
           if (kEmit && int(lane) == newest && done < room) {
             out_k[done] = lim;
             out_v[done] = __ldg(ls.vals[lane] + pos);
@@ -691,8 +797,21 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
           ++done;
         }
         if (left && key_of(first) == lim) pos = upper_bound_key(keys, pos, end, lim);
+        if (reach || ++alone >= kAlone) reach = min(4 * cap, kMaxReach);
         continue;
       }
+    }
+    if (reach) {
+      const uint2 got = repeat_merge<kEmit>(ls, pos, pos + n, past, out_k + done, out_v + done,
+                                            room > done ? room - done : 0u);
+      done += got.x;
+      pos += n;
+      past = 0xFFFFFFFFu;
+      alone = 0;
+      const bool paid = warp_sum(n) >= per_run * got.y;
+      if (!paid) enter = (enter + 34) / 2;  // (33: never)
+      reach = paid ? min(4 * reach, kMaxReach) : 0u;
+      continue;
     }
     const uint32_t off = warp_incl_scan(n) - n;
     __syncwarp();
@@ -775,14 +894,19 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
     }
     done += live;
     pos += n;
+    if (total > all) {
+      const uint32_t t = 1 + (lane * all) / 33;  // (all > 1: a piece with nothing in it takes a key alone)
+      const bool same = t < all && key_of(sh.kv[t - 1]) == key_of(sh.kv[t]);
+      if (uint32_t(__popc(__ballot_sync(0xffffffffu, same))) >= enter) reach = kReach;
+    }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) count_wide(LevelSet ls, const uint32_t* __restrict__ k1,
-                                                       const uint32_t* __restrict__ k2, uint64_t nq,
-                                                       uint32_t* __restrict__ out_count,
-                                                       const uint32_t* __restrict__ perm,
-                                                       const uint32_t* __restrict__ wide) {
+__global__ void __launch_bounds__(kThreads, 8) count_wide(LevelSet ls, const uint32_t* __restrict__ k1,
+                                                          const uint32_t* __restrict__ k2, uint64_t nq,
+                                                          uint32_t* __restrict__ out_count,
+                                                          const uint32_t* __restrict__ perm,
+                                                          const uint32_t* __restrict__ wide) {
   __shared__ WideCount s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
   const uint32_t lane = lane_id();
@@ -800,10 +924,10 @@ __global__ void __launch_bounds__(kThreads) count_wide(LevelSet ls, const uint32
 
 // The windows are those that the count pass stored.
 __global__ void __launch_bounds__(kThreads) range_wide(LevelSet ls, uint64_t nq, const uint32_t* __restrict__ bounds,
-                                                       const uint64_t* __restrict__ offsets,
-                                                       uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                       const uint32_t* __restrict__ perm,
-                                                       const uint32_t* __restrict__ wide) {
+                                                          const uint64_t* __restrict__ offsets,
+                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                          const uint32_t* __restrict__ perm,
+                                                          const uint32_t* __restrict__ wide) {
   __shared__ WideEmit s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
   const uint32_t lane = lane_id();

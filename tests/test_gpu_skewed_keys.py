@@ -143,3 +143,56 @@ def test_searches_in_crowded_bins(g, sizes, shape):
     want = np.searchsorted(keys, k2, side="right") - np.searchsorted(keys, k1)
     np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), want)
     lsm.close()
+
+
+def repeated(dist, n, space, rng):
+    """Keys below `space` of which most are stored many times: evenly, as Zipf's, or a few runs among single keys."""
+    if dist == "even":
+        return rng.integers(0, space, n)
+    if dist == "zipf":
+        return (rng.zipf(1.3, n) * 7919) % space
+    return np.where(rng.random(n) < 0.9, rng.integers(0, 9, n) * (space // 9), rng.integers(0, space, n))
+
+
+@pytest.mark.parametrize("batches", [1, 3, 8, 16, 31])
+@pytest.mark.parametrize("dist,space", [("even", 100), ("even", 3000), ("even", 1 << 16), ("zipf", 1 << 20), ("runs", 1 << 16)])
+def test_windows_of_repeated_keys(g, batches, dist, space):
+    """Counts and ranges over windows of one to all keys, each stored many times in a level and over the levels, with
+    deletes and short batches, against the ordered map."""
+    b, rng = 20000, np.random.default_rng(batches + space)
+    lsm, o1 = g.LSM(b, 32 * b), oracle.MapOracle(b)
+    for t in range(batches):
+        n = b if t % 5 != 4 else b // 3
+        k = repeated(dist, n, space, rng).astype(np.uint32)
+        v = rng.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+        d = (rng.random(n) < (0.0 if t % 3 else 0.3)).astype(np.uint8)
+        lsm.update(k, v, d)
+        o1.call("update", k, v, d)
+    k1 = np.concatenate([rng.integers(0, space, 200), rng.choice(k, 50), [0, 0, space]])
+    w = rng.choice([0, 1, 2, 7, 40, 300, 2500, 1 << 14, 1 << 16, 1 << 20], len(k1))
+    k2 = np.minimum(k1 + w, TOP - 1)
+    k1, k2 = k1.astype(np.uint32), k2.astype(np.uint32)
+    np.testing.assert_array_equal(g.to_numpy_u32(lsm.count(k1, k2)), o1.count(k1, k2))
+    off, rk, rv = lsm.range(k1, k2)
+    eo, ek, ev = o1.range(k1, k2)
+    np.testing.assert_array_equal(off.cpu().numpy().astype(np.uint64), eo)
+    np.testing.assert_array_equal(g.to_numpy_u32(rk), ek)
+    np.testing.assert_array_equal(g.to_numpy_u32(rv), ev)
+    assert lsm.device_errors() == 0
+    lsm.close()
+
+
+def test_repeated_keys_are_skipped(g):
+    """Counts over all of 31 batches: windows of as many elements are counted in less than half of the time when each
+    key is stored a hundred times (a seventh was measured), since old versions are not read."""
+    b, t = 1 << 17, []
+    for space in (1 << 15, TOP):
+        rng = np.random.default_rng(space % 101)
+        lsm = g.LSM(b, 32 * b)
+        for _ in range(31):
+            lsm.insert(rng.integers(0, space, b).astype(np.uint32), np.zeros(b, np.uint32))
+        k1 = g.as_device_u32(np.arange(256), 0)
+        k2 = g.as_device_u32(np.full(256, TOP - 1), 0)
+        t.append(seconds(lambda: lsm.count(k1, k2), 2))
+        lsm.close()
+    assert t[0] < 0.5 * t[1], t
