@@ -509,7 +509,9 @@ __device__ __forceinline__ uint32_t merge_windows(const LevelSet& ls, const uint
 // Queries whose windows hold more than kWideMin elements in all are wide:
 // with a wide list, the count kernel appends them to it (their count and
 // output are then written by the warp kernels below) instead of merging
-// hundreds of elements in one thread.
+// hundreds of elements in one thread.  (The line comes from the warp kernels'
+// first form.  2^18 counts in six levels, windows of 30 / 60 / 90 elements: 305 /
+// 341 / 378 us with a line at 16, 142 / 361 / 378 at 40, 138 / 225 / 314 at 120.)
 constexpr uint32_t kWideMin = 40;
 
 template <int L>

@@ -246,12 +246,13 @@ __global__ void __launch_bounds__(kPassThreads) sort_histogram(Loader ld, uint32
 // One 8-bit pass over a tile of 8192 elements, bound by the chain of phases
 // of a tile (loads, ranks, look-back, scatter) with two tiles an SM in flight:
 // 290 us a pass at n = 5 10^7 (2.8 TB/s of reads and writes).  Tiles of 4096
-// in CTAs of 143 registers, one an SM, took 1161 us: the look-back advances by
-// at most its window (8 tiles) per round trip to L2, and one CTA an SM hides
-// nothing.  Keys are ranked and put in shared memory before the values are
-// loaded, so that 16 items a thread fit 64 registers.  Measured beside it (four
-// passes and the histogram, 5 10^7 pairs: 1170 us): tiles of 6144 at three CTAs
-// an SM 1413 us, of 10240 1258 us, windows of 4 and 12 tiles 1207 and 1242 us.
+// in CTAs of 143 registers, one an SM, took 1161 us a pass: the look-back
+// advances by at most its window (8 tiles) per round trip to L2, and one CTA an
+// SM hides nothing.  Keys are ranked and put in shared memory before the values
+// are loaded, so that 16 items a thread fit 64 registers.  Measured beside it
+// (the whole sort of 5 10^7 pairs, four passes and the histogram: 1170 us):
+// tiles of 6144 at three CTAs an SM 1413 us, of 10240 1258 us, windows of 4 and
+// 12 tiles 1207 and 1242 us.
 struct PassShared {
   union {
     struct {
@@ -302,8 +303,9 @@ __global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const ui
   // Rank within the warp, items in (j, lane) order = input order.  The lanes
   // with an item's digit are found by ballots for every other item and
   // through shared memory for the rest: ballots alone kept the ALUs 66 % busy
-  // and the shared-memory pipe 44 %, atomics alone 24 % and 55 %; halves of
-  // each took 1311 us against 1368 and 1466 for 5 10^7 pairs.
+  // and the shared-memory pipe 44 %, atomics alone 24 % and 55 %.  (All three on
+  // the build before the look-back had a thread per digit, whole sorts of 5 10^7
+  // pairs: ballots 1368 us, atomics 1466, halves of each 1311; since then 1170.)
   const uint32_t lt = lanemask_lt();
 #pragma unroll
   for (int j = 0; j < kIPT; ++j) {
@@ -1444,7 +1446,9 @@ __device__ __forceinline__ void write_placebos(uint32_t* out_k, uint32_t* out_v,
 // elements; with a prefix index, which has 2^16 entries or more however small
 // the batch, every CTA of the grid sorts the batch and writes its share of the
 // entries.  (Update calls of 1051 / 5000 uniform keys: 28.8 / 39.8 us with all
-// entries written by one CTA, now 10.4 / 10.7; the two kernels 19.6 / 21.1.)
+// entries written by one CTA, now 10.4 / 10.7; the two kernels 19.6 / 21.1.
+// Between 512 and 16384 entries a CTA the calls differ by their spread only:
+// 15.2 .. 16.4 and 16.4 .. 17.1 us with a reset in the loop.)
 constexpr uint32_t kSmallBins = 2048;  // entries per CTA
 __global__ void __launch_bounds__(kBucketThreads) small_sort(Loader ld, uint32_t* out_k, uint32_t* out_v,
                                                              uint32_t* fence, int fshift, uint32_t* host,
