@@ -634,21 +634,22 @@ __device__ __forceinline__ uint32_t lower_bound_smem(const uint32_t* a, uint32_t
 // among the lanes is the next key, the newest level's element decides, and
 // every lane whose head it is goes to the end of its run, whose length is
 // guessed from the run before.  The parts are cut at even places of the largest
-// window.  Key `past` has been decided already.  Result as wide_merge in x, the
-// number of runs in y; kEmit: the parts' counts come from a first pass.  Bound
-// by the chain of loads, a few per key and level.
-template <bool kEmit>
-__device__ __forceinline__ uint2 repeat_merge(const LevelSet& ls, uint32_t pos, uint32_t end, uint32_t past,
-                                              uint32_t* out_k, uint32_t* out_v, uint64_t room) {
+// window.  The live keys as wide_merge in x, the number of runs in y; kEmit: the
+// parts' counts come from a first pass.  Bound by the chain of loads, a few per
+// key and level.
+template <bool kEmit, bool kOne>
+__device__ __forceinline__ uint2 repeat_merge(const LevelSet& ls, uint32_t pos, uint32_t end, uint32_t* out_k,
+                                              uint32_t* out_v, uint64_t room) {
   const uint32_t lane = lane_id();
   uint32_t width = 1;  // lanes of a group
-  while (width < uint32_t(ls.count)) width *= 2;
+  if (!kOne)
+    while (width < uint32_t(ls.count)) width *= 2;
   const uint32_t l = lane & (width - 1), part = lane / width, parts = 32 / width;
   const bool act = l < uint32_t(ls.count);
   const uint32_t *keys = act ? ls.keys[l] : nullptr, *vals = act ? ls.vals[l] : nullptr;
   // the part's start in every level, and the next part's
   const uint32_t most = __reduce_max_sync(0xffffffffu, end - pos);
-  const int big = __ffs(int(__ballot_sync(0xffffffffu, end - pos == most))) - 1;
+  const int big = kOne ? 0 : __ffs(int(__ballot_sync(0xffffffffu, end - pos == most))) - 1;
   const uint32_t cut = __shfl_sync(0xffffffffu, pos, big) + uint32_t(uint64_t(most) * part / parts);
   const uint32_t from = part ? key_of(__ldg(ls.keys[big] + cut)) : 0u;
   const uint32_t p = __shfl_sync(0xffffffffu, pos, int(l)), e = __shfl_sync(0xffffffffu, end, int(l));
@@ -671,7 +672,7 @@ __device__ __forceinline__ uint2 repeat_merge(const LevelSet& ls, uint32_t pos, 
       const uint32_t who = __ballot_sync(0xffffffffu, mine), live_who = __ballot_sync(0xffffffffu, mine && (kv & 1u));
       const uint32_t group = who & (0xffffffffu >> (32 - width)) << (part * width);
       const uint32_t newest = group & (0u - group);  // its lane's bit
-      if ((live_who & newest) && k != past) {
+      if (live_who & newest) {
         if (kEmit && pass && newest == 1u << lane && before + live < room) {
           out_k[before + live] = k;
           if (to_value) *to_value = value;
@@ -712,24 +713,80 @@ __device__ __forceinline__ uint2 repeat_merge(const LevelSet& ls, uint32_t pos, 
   return make_uint2(live, warp_sum(runs));
 }
 
-// When kSame of 32 elements of a piece have the key of the one before, or after
-// kAlone keys that fill a piece alone, the next kReach elements are taken by
-// repeat_merge, then four times as many, while they have kRepeats per run; when
-// they do not, it takes more to come back to it.  One level, which is read
-// straight through, when 32 elements in a row have one key, and kRepeatsOne per
-// run.
+// Versions are skipped from kAgain pieces in a row on that repeat: kSame of 32
+// elements have the key of the one before, or a key fills a piece alone.  The
+// next kReach elements are then taken by repeat_merge, then four times as many,
+// while they have kRepeats per run; when they do not, it takes twice as many
+// pieces to come back to it.  One level, which is read straight through, from
+// kAgainOne chunks of 128 in a row on that end in 32 of one key (one that is all
+// one key counts twice), while there are kRepeatsOne per run.
 // (31 batches of 2^18 keys below 2^16, about 24 copies of a key per level:
-// 65536 counts of 64 keys 4690 us read piece by piece, now about 560, ranges
-// 16.1 and 2.5 ms; 256 counts of 50000 keys 225 and 19 ms.  One level of 2^24
-// with 256 copies: 65536 counts of 64 keys 1315 and 355 us.  Zipf keys, of which
-// most runs are short, lose by skipping: 8192 ranges of 1000 keys 430 us read,
-// 650 with what is tried and given up.  The tests themselves cost spread keys
-// 1 %: range_wide needs 64 registers instead of 48, without which the value of
-// a key found is waited for.)
-constexpr uint32_t kSame = 24, kRepeats = 3, kRepeatsOne = 32, kAlone = 6, kReach = 1024, kMaxReach = 1u << 24;
+// 65536 counts of 64 keys 4690 us read piece by piece, so 579, ranges 16.1 and 2.6
+// ms; 256 counts of 50000 keys 225 and 19 ms.  One level of 2^24 with 256 copies:
+// 65536 counts of 64 keys 1315 and 329 us.  Zipf keys have such pieces, but seldom
+// two in a row: 8192 ranges of 1000 keys 430 us read, 434 so, 690 when one piece
+// was enough.  range_wide takes 64 registers instead of 48 for it, without which
+// the value of a key found is waited for; no fewer CTAs fit beside its shared
+// memory.)
+constexpr uint32_t kSame = 24, kAgain = 2, kRepeats = 3, kReach = 2048, kMaxReach = 1u << 24;
+constexpr uint32_t kAgainOne = 4, kRepeatsOne = 32;
 
-// Live keys of the windows [pos, end) (lane l holds level l's), emitted to
-// out_k/out_v in key order when kEmit (at most `room`); returns their number.
+// Live keys of the window [i0, last) of the only level: nothing to look for in
+// other levels, so the window is read through, in order.
+template <bool kEmit>
+__device__ __forceinline__ uint32_t wide_one(const LevelSet& ls, uint32_t i0, const uint32_t last, uint32_t* out_k,
+                                             uint32_t* out_v, uint64_t room) {
+  const uint32_t lane = lane_id(), lt = lanemask_lt();
+  const uint32_t* keys = ls.keys[0];
+  uint32_t done = 0, again = 0, before = 0xFFFFFFFFu;  // before: key before the chunk
+  while (i0 < last) {
+    uint32_t kv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t i = i0 + 32 * j + lane;
+      kv[j] = i < last ? __ldg(keys + i) : 0xFFFFFFFEu;  // (no regular element)
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t k = key_of(kv[j]), up = __shfl_up_sync(0xffffffffu, k, 1);
+      const bool ok = (kv[j] & 1u) && k != (lane ? up : before);
+      before = __shfl_sync(0xffffffffu, k, 31);
+      const uint32_t m = __ballot_sync(0xffffffffu, ok), at = done + __popc(m & lt);
+      if (kEmit && ok && at < room) {
+        out_k[at] = k;
+        out_v[at] = __ldg(ls.vals[0] + (i0 + 32 * j + lane));
+      }
+      done += __popc(m);
+    }
+    i0 += 128;
+    const bool one = __shfl_sync(0xffffffffu, key_of(kv[0]), 0) == before;
+    again = __shfl_sync(0xffffffffu, key_of(kv[3]), 0) == before ? again + (one ? 2u : 1u) : 0u;
+    if (i0 >= last || (!one && again < kAgainOne)) continue;
+    i0 = upper_bound_key(keys, i0, last, before);  // past a long run (a short batch's padding is one)
+    if (again < kAgainOne) continue;
+    bool paid = true;
+    for (uint32_t reach = kReach; paid && i0 < last; reach = min(4 * reach, kMaxReach)) {
+      uint32_t to = last;
+      if (last - i0 > reach) {  // up to the start of a run, or the end of one that is longer
+        const uint32_t k = key_of(__ldg(keys + i0 + reach));
+        to = lower_bound_kv(keys, i0, i0 + reach, k << 1);
+        if (to == i0) to = upper_bound_key(keys, i0 + reach, last, k);
+      }
+      const uint2 got = repeat_merge<kEmit, true>(ls, lane ? 0u : i0, lane ? 0u : to, out_k + done, out_v + done,
+                                                  room > done ? room - done : 0u);
+      done += got.x;
+      paid = to - i0 >= kRepeatsOne * got.y;
+      i0 = to;
+    }
+    again = 0;
+    before = 0xFFFFFFFFu;
+  }
+  return done;
+}
+
+// Live keys of the windows [pos, end) (lane l holds level l's) of several
+// levels, emitted to out_k/out_v in key order when kEmit (at most `room`);
+// returns their number.
 template <class Shared>
 __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos, uint32_t end, Shared& sh,
                                                uint32_t* out_k, uint32_t* out_v, uint64_t room) {
@@ -738,42 +795,9 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
   const int nl = ls.count;
   const bool act = lane < uint32_t(nl);
   const uint32_t* keys = act ? ls.keys[lane] : nullptr;
-  const uint32_t per_run = nl == 1 ? kRepeatsOne : kRepeats;
-  uint32_t done = 0, alone = 0, enter = nl == 1 ? 31u : kSame, past = 0xFFFFFFFFu;
+  uint32_t done = 0, again = 0, enough = kAgain;
   uint32_t reach = 0;  // elements that repeat_merge takes next, 0 when it does not
   for (;;) {
-    if (nl == 1 && reach == 0) {  // nothing to look for in other levels: the window is read through, in order
-      const uint32_t last = __shfl_sync(0xffffffffu, end, 0), lt = lanemask_lt();
-      uint32_t before = past;  // key before the chunk
-      uint32_t i0 = __shfl_sync(0xffffffffu, pos, 0);
-      while (i0 < last && reach == 0) {
-        uint32_t kv[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t i = i0 + 32 * j + lane;
-          kv[j] = i < last ? __ldg(ls.keys[0] + i) : 0xFFFFFFFEu;  // (no regular element)
-        }
-        uint32_t same = 0;  // of the first 32, those with the key of the one before
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t k = key_of(kv[j]), up = __shfl_up_sync(0xffffffffu, k, 1);
-          const bool first = k != (lane ? up : before), ok = (kv[j] & 1u) && first;
-          if (j == 0) same = 32u - __popc(__ballot_sync(0xffffffffu, first));
-          before = __shfl_sync(0xffffffffu, k, 31);
-          const uint32_t m = __ballot_sync(0xffffffffu, ok), at = done + __popc(m & lt);
-          if (kEmit && ok && at < room) {
-            out_k[at] = k;
-            out_v[at] = __ldg(ls.vals[0] + (i0 + 32 * j + lane));
-          }
-          done += __popc(m);
-        }
-        i0 += 128;
-        if (same >= enter && i0 + 128 < last) reach = kReach;
-      }
-      if (i0 >= last) return done;
-      pos = lane ? 0u : i0;
-      past = before;
-    }
     const uint32_t left = act ? end - pos : 0u;
     const uint32_t total = warp_sum(left);
     if (total == 0) return done;
@@ -791,7 +815,7 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
         const uint32_t has = __ballot_sync(0xffffffffu, left && key_of(first) == lim);
         const int newest = __ffs(int(has)) - 1;
         const bool live = (__shfl_sync(0xffffffffu, first, newest) & 1u) != 0u;
-        if (live && lim != past) {
+        if (live) {
           if (kEmit && int(lane) == newest && done < room) {
             out_k[done] = lim;
             out_v[done] = __ldg(ls.vals[lane] + pos);
@@ -799,19 +823,19 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
           ++done;
         }
         if (left && key_of(first) == lim) pos = upper_bound_key(keys, pos, end, lim);
-        if (reach || ++alone >= kAlone) reach = min(4 * cap, kMaxReach);
+        if (reach) reach = min(4 * reach, kMaxReach);
+        else if (++again >= enough) reach = kReach;
         continue;
       }
     }
     if (reach) {
-      const uint2 got = repeat_merge<kEmit>(ls, pos, pos + n, past, out_k + done, out_v + done,
-                                            room > done ? room - done : 0u);
+      const uint2 got = repeat_merge<kEmit, false>(ls, pos, pos + n, out_k + done, out_v + done,
+                                                   room > done ? room - done : 0u);
       done += got.x;
       pos += n;
-      past = 0xFFFFFFFFu;
-      alone = 0;
-      const bool paid = warp_sum(n) >= per_run * got.y;
-      if (!paid) enter = (enter + 34) / 2;  // (33: never)
+      again = 0;
+      const bool paid = warp_sum(n) >= kRepeats * got.y;
+      if (!paid) enough *= 2;
       reach = paid ? min(4 * reach, kMaxReach) : 0u;
       continue;
     }
@@ -899,17 +923,18 @@ __device__ __forceinline__ uint32_t wide_merge(const LevelSet& ls, uint32_t pos,
     if (total > all) {
       const uint32_t t = 1 + (lane * all) / 33;  // (all > 1: a piece with nothing in it takes a key alone)
       const bool same = t < all && key_of(sh.kv[t - 1]) == key_of(sh.kv[t]);
-      if (uint32_t(__popc(__ballot_sync(0xffffffffu, same))) >= enter) reach = kReach;
+      again = uint32_t(__popc(__ballot_sync(0xffffffffu, same))) >= kSame ? again + 1 : 0u;
+      if (again >= enough) reach = kReach;
     }
   }
 }
 
+template <bool kOne>
 __global__ void __launch_bounds__(kThreads, 8) count_wide(LevelSet ls, const uint32_t* __restrict__ k1,
                                                           const uint32_t* __restrict__ k2, uint64_t nq,
                                                           uint32_t* __restrict__ out_count,
                                                           const uint32_t* __restrict__ perm,
                                                           const uint32_t* __restrict__ wide) {
-  __shared__ WideCount s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
   const uint32_t lane = lane_id();
   for (uint32_t w = (blockIdx.x * kThreads + threadIdx.x) >> 5; w < nw; w += (gridDim.x * kThreads) >> 5) {
@@ -919,18 +944,24 @@ __global__ void __launch_bounds__(kThreads, 8) count_wide(LevelSet ls, const uin
     const uint32_t a = __ldg(k1 + i0), z = min(__ldg(k2 + i), kMaxUserKey);
     uint32_t lo = 0, hi = 0;
     if (lane < uint32_t(ls.count) && a <= z) level_window(ls, int(lane), a << 1, (z + 1u) << 1, lo, hi);
-    const uint32_t c = wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], nullptr, nullptr, 0);
+    uint32_t c;
+    if constexpr (kOne) {
+      c = wide_one<false>(ls, __shfl_sync(0xffffffffu, lo, 0), __shfl_sync(0xffffffffu, hi, 0), nullptr, nullptr, 0);
+    } else {
+      __shared__ WideCount s_warp[kThreads / 32];
+      c = wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], nullptr, nullptr, 0);
+    }
     if (lane == 0) out_count[i] = c;
   }
 }
 
 // The windows are those that the count pass stored.
+template <bool kOne>
 __global__ void __launch_bounds__(kThreads) range_wide(LevelSet ls, uint64_t nq, const uint32_t* __restrict__ bounds,
                                                           const uint64_t* __restrict__ offsets,
                                                           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                           const uint32_t* __restrict__ perm,
                                                           const uint32_t* __restrict__ wide) {
-  __shared__ WideEmit s_warp[kThreads / 32];
   const uint32_t nw = *reinterpret_cast<const volatile uint32_t*>(wide);
   const uint32_t lane = lane_id();
   for (uint32_t w = (blockIdx.x * kThreads + threadIdx.x) >> 5; w < nw; w += (gridDim.x * kThreads) >> 5) {
@@ -942,8 +973,13 @@ __global__ void __launch_bounds__(kThreads) range_wide(LevelSet ls, uint64_t nq,
       lo = __ldg(bounds + (i * ls.count + lane) * 2);
       hi = __ldg(bounds + (i * ls.count + lane) * 2 + 1);
     }
-    const uint64_t o = offsets[i];
-    wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], keys + o, vals + o, offsets[i + 1] - o);
+    const uint64_t o = offsets[i], room = offsets[i + 1] - o;
+    if constexpr (kOne) {
+      wide_one<true>(ls, __shfl_sync(0xffffffffu, lo, 0), __shfl_sync(0xffffffffu, hi, 0), keys + o, vals + o, room);
+    } else {
+      __shared__ WideEmit s_warp[kThreads / 32];
+      wide_merge(ls, lo, hi, s_warp[threadIdx.x >> 5], keys + o, vals + o, room);
+    }
   }
 }
 
@@ -1209,7 +1245,8 @@ cudaError_t count_launch(const LevelSet& ls, const uint32_t* k1, const uint32_t*
   // all are wide; an empty list ends at once)
   const unsigned wgrid = persistent_grid(nq * 32, kThreads, 152 * 8);
   count_launches(1);
-  count_wide<<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
+  if (ls.count <= 1) count_wide<true><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
+  else count_wide<false><<<wgrid, kThreads, 0, st>>>(ls, k1, k2, nq, count, perm, wide);
   return cudaGetLastError();
 }
 
@@ -1242,7 +1279,8 @@ cudaError_t range_emit_launch(const LevelSet& ls, uint64_t nq, const uint32_t* b
   if ((e = cudaGetLastError()) != cudaSuccess || !w) return e;
   const unsigned wgrid = persistent_grid(nq * 32, kThreads, 152 * 8);
   count_launches(1);
-  range_wide<<<wgrid, kThreads, 0, st>>>(ls, nq, bounds, offsets, keys, vals, perm, wide);
+  if (ls.count <= 1) range_wide<true><<<wgrid, kThreads, 0, st>>>(ls, nq, bounds, offsets, keys, vals, perm, wide);
+  else range_wide<false><<<wgrid, kThreads, 0, st>>>(ls, nq, bounds, offsets, keys, vals, perm, wide);
   return cudaGetLastError();
 }
 
