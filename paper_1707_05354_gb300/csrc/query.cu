@@ -172,7 +172,8 @@ __global__ void __launch_bounds__(kThreads) lookup_direct(LevelSet ls, const uin
 // each part of a level and of its prefix index comes from HBM once.  (2^24
 // lookups, half of them hits: seven levels of 133 million elements 835 us, one
 // level of 2^27 469 us; in input order 2197 and 866.  bulk_search takes 723 and 328
-// us of that, bound by its searches' L2 accesses and the grouping.)
+// us of that, bound by its instructions and the latency of the loads between
+// them: it issues in two cycles of three, DRAM and L2 are a fifth busy.)
 constexpr uint32_t kBulkTile = 8192, kBulkParts = 256, kBulkChunk = 2048, kBulkThreads = 512, kBulkSub = 2048;
 constexpr uint32_t kBulkItems = kBulkTile / kBulkThreads;          // per thread of the tile kernels
 constexpr uint32_t kBulkChunkItems = kBulkChunk / kBulkThreads;    // per thread of the search

@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) sort_pass(Loader ld, const ui
 //                out with the prefix index entries of the bins that start in
 //                its range.  A bucket above kBucketCap elements (many copies
 //                of a few keys, or keys in clusters) is taken by the same
-//                CTA in parts that fit.
+//                CTA in parts that fit or in 8-bit passes (sort_big).
 // The buckets split the range of the keys that the batch holds (KeyMap), not
 // the 32 bits of the key variable: ids below 2^25 would otherwise fall in
 // four buckets and be sorted by four CTAs; hot keys have buckets of their own.
